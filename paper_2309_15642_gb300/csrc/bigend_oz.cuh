@@ -1,0 +1,491 @@
+// Gram and update products of the larger end of a bond in complex128 on the
+// tensor cores: error-free splitting into fixed-point digits (the scheme of
+// Ozaki, Ogita, Oishi and Rump), tcgen05.mma of kind::f16 with FP32 accumulators.
+//
+// GB300 runs FP64 at 1.2 TFLOP/s (an FP64 instruction of a warp holds its SMSP's
+// unit for 64 cycles) and f16 products at 2 PFLOP/s, so the two streaming
+// products, which are plain contractions, are formed from integers:
+//
+//   x = 2^(E-6) sum_i d_i 2^(-8 i),  i = 0..6,  |d_i| <= 128 integers (|d_0| <= 65),
+//
+// with one exponent E per operand row (|x| < 2^E over the contraction), that is
+// x rounded to a multiple of 2^-54 of its row's power of two.  The digits are
+// exact in f16, their products and the FP32 sums of up to 7 x 128 of them are
+// below 2^24, so every accumulator is an exact integer whatever the order:
+//
+//   sum_k x_k y_k = 2^(Ex+Ey-12) sum_{l=0..6} 2^(-8 l) v_l,  v_l = sum_{i+j=l} sum_k d_i(x_k) d_j(y_k).
+//
+// The levels l > 6 are below 2^-54 of the row maxima's product.  The seven v_l of
+// an output are combined in a 64-bit integer of unit 2^(Ex+Ey-52) and rounded
+// once to FP64.  An FP64 sum of K products rounds K times at 2^-53, so the result
+// is at least as accurate against the row maxima.
+//
+// The digits of a double cost about 30 integer instructions and no FP64 one.
+// Slices are stored as K-major operands without swizzle, slice after slice, so
+// that one instruction multiplies slice i of A with several slices j of B at once
+// (N = slices x columns) and lands on the adjacent accumulators of the levels
+// i + j.
+//
+//   oz_gram_kernel    one CTA per row tile (and spin, beyond D = 32): kicks the
+//       rows (writing them, unweighted, to `at` for the update, with the largest
+//       exponent of each row), weights them, and writes the tile's Gram blocks in
+//       FP64 (the partials of gram_kernel).
+//   oz_update_kernel  one CTA per 128 rows, spin and 32 new bond indices:
+//       Gamma_a'[s] = mask (Ã_s Y_s) from `at`.
+//
+// Included by su_kernels.cu after its row/element helpers.
+#pragma once
+#include <cuda_fp16.h>
+
+#include "tcgen05.cuh"
+
+namespace gpeps {
+
+constexpr int kOzThreads = 512;
+constexpr int kOzSlices = 7;
+constexpr int kOzOperand = kOzSlices * 128 * 64 * 2;  // bytes of 7 slices of 8192 digits
+constexpr int kOzDumpLd = 129;                        // row stride (doubles) of the Gram readout
+constexpr size_t kOzGramSmem = (size_t)128 * kOzDumpLd * 8;
+constexpr size_t kOzUpdateSmem = (size_t)kOzOperand + kOzOperand / 2;
+
+__device__ __forceinline__ int oz_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// Biased fixed point: round(x 2^(54 - E)) + 0x80 in each of the 7 digit bytes, E =
+// em - 1022 for the row's largest biased exponent em: byte 6 - i minus 128 is d_i.
+__device__ __forceinline__ unsigned long long oz_fixed(double x, int em, bool negate = false) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(b >> 52) & 0x7ff, d = em - ex;
+  unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 1;
+  m = (m + ((1ull << (d & 63)) >> 1)) >> (d & 63);
+  if (d > 55 || ex == 0) m = 0;
+  const bool neg = ((long long)b < 0) != negate;
+  return (neg ? 0ull - m : m) + 0x0080808080808080ull;
+}
+
+// The digits of 8 consecutive K values of one operand row: one 16-byte store per slice.
+__device__ __forceinline__ void oz_store(unsigned char* p, uint32_t slice_bytes, const unsigned long long* v) {
+#pragma unroll
+  for (int i = 0; i < kOzSlices; ++i) {
+    const int byte = 6 - i;
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t a = (uint32_t)(v[2 * q] >> (byte >= 4 ? 32 : 0));
+      const uint32_t b = (uint32_t)(v[2 * q + 1] >> (byte >= 4 ? 32 : 0));
+      const uint32_t s = byte & 3;
+      // two bytes -> f16 1024 + byte -> byte - 128
+      const uint32_t t = (__byte_perm(a, b, s | (s << 4) | ((4 + s) << 8) | ((4 + s) << 12)) & 0x00ff00ffu) | 0x64006400u;
+      const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&t), __half2half2(__ushort_as_half(0x6480)));
+      w[q] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    *reinterpret_cast<uint4*>(p + (size_t)i * slice_bytes) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// t 2^(ea + eb - 2044 - 52) rounded to FP64 (ea, eb: biased exponents of the two rows);
+// NaN when a row held a value that is not finite.
+__device__ __forceinline__ double oz_value(long long t, int ea, int eb) {
+  if (ea == 0x7ff || eb == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);
+  const unsigned long long u = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
+  if (u == 0) return 0.0;
+  const int n = __clzll((long long)u);
+  const unsigned long long m = u << n;  // top bit at 63: value m 2^(-n) 2^(...)
+  const int e = 1023 + 63 - n + ea + eb - 2044 - 52;
+  if (e <= 0) return 0.0;
+  if (e >= 0x7ff) return __longlong_as_double(t < 0 ? 0xfff0000000000000ll : 0x7ff0000000000000ll);
+  const unsigned long long r = ((unsigned long long)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+  return __longlong_as_double((long long)(r | (t < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, int n, uint32_t accumulate) {
+  // FP32 accumulator, f16 operands, both K-major, M = 128
+  const uint32_t idesc = (1u << 4) | ((uint32_t)(n >> 3) << 17) | (8u << 24);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// 32 lanes x 8 consecutive FP32 columns (the caller waits: tcgen05.wait::ld)
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// Commit the issued products and wait (bounded) for them; the outcome is uniform over the CTA.
+__device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t& phase) {
+  const bool ok = tc_wait(bar, phase, kTcWaitCycles);
+  tc::fence_after_sync();
+  return ok;
+}
+
+// cos and sin of half the pending kick of end a, once per bond (an FP64 sincos per
+// thread of every tile would cost more than the tile's products).
+__global__ void oz_kick_kernel(const BondDesc* __restrict__ bonds, int n, const double* __restrict__ pending,
+                               double2* __restrict__ cs) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double h = 0.5 * pending[bonds[i].a.site];
+  cs[i] = make_double2(cos(h), sin(h));
+}
+
+// Slot of one row tile in `at`: Ã [s][row][re/im][k] (doubles), and of its largest exponents [s][row].
+__device__ __forceinline__ int64_t oz_at(int part, int s, int row, int ri, int tr, int D) {
+  return (int64_t)part * 4 * tr * D + ((int64_t)(s * tr + row) * 2 + ri) * D;
+}
+
+// kMode 0: D <= 32, one CTA per 64-row tile, operand rows (s, re/im, k), k padded to 32;
+// kMode 1: D <= 64, one per tile and spin, rows (re/im, k), k padded to 64;
+// kMode 2: D <= 128, one per 32-row tile and spin, rows (re/im, k), k padded to 128: two
+//          products, Re = re re^T + im im^T and T = re im^T (Im = T - T^T).
+// In each, 16 warps take 8 rows x 32 bond indices of one spin: 8192 digits per slice.
+template <int kMode>
+__global__ void __launch_bounds__(kOzThreads, 1)
+    oz_gram_kernel(const TileDesc* __restrict__ tiles, const BondDesc* __restrict__ bonds,
+                   const double2* __restrict__ gamma, const double* __restrict__ lam, const double2* __restrict__ cs,
+                   double2* __restrict__ partials, double* __restrict__ at, int* __restrict__ rexp, int* flags,
+                   int D) {
+  constexpr int Kt = kMode == 2 ? 32 : 64, kRows = kMode == 2 ? 256 : 128;
+  constexpr uint32_t kSlice = kRows * Kt * 2, kSbo = Kt * 16;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int cmax[kMode == 2 ? 128 : 64], rmax[128];
+  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ uint32_t tslot;
+  const TileDesc t = tiles[blockIdx.x];
+  const SideDesc sa = bonds[t.bond].a;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < 128) {
+    if (threadIdx.x < (int)(sizeof(cmax) / 4)) cmax[threadIdx.x] = 0;
+    rmax[threadIdx.x] = 0;
+  }
+  const uint32_t tmem = tc_setup(&tslot, bars, 512);
+  // rows of this warp: 8 rows from rg * 8, bond index k, spin s
+  const int rg = kMode == 2 ? (warp & 3) : (warp & 7);
+  const int kb = kMode == 0 ? 0 : kMode == 1 ? (warp >> 3) : (warp >> 2);
+  const int s = kMode == 0 ? (warp >> 3) : (int)blockIdx.y;
+  const int k = kb * 32 + lane;
+  const int tr = kMode == 2 ? 32 : 64;
+  double2 x[8];
+  {
+    const double2 c = cs[t.bond];
+    double2 g0[8], g1[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = rg * 8 + i;
+      g0[i] = g1[i] = make_double2(0.0, 0.0);
+      if (r < t.nrows && k < D) {
+        const int64_t e = elem(sa, 0, row_pos(sa, t.row0 + r), k);
+        g0[i] = gamma[e];
+        g1[i] = gamma[e + sa.str_s];
+      }
+    }
+    int cm = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = rg * 8 + i;
+      double2 a = make_double2(0.0, 0.0);
+      double w = 0.0;
+      if (r < t.nrows) {
+        // component s of exp(-i theta X / 2) (as kick2)
+        const double2 p = s ? g1[i] : g0[i], q = s ? g0[i] : g1[i];
+        a = make_double2(c.x * p.x + c.y * q.y, c.x * p.y - c.y * q.x);
+        w = row_weight(sa, lam, row_pos(sa, t.row0 + r));
+        if (k < D) {
+          at[oz_at(t.part, s, r, 0, tr, D) + k] = a.x;
+          at[oz_at(t.part, s, r, 1, tr, D) + k] = a.y;
+        }
+      }
+      const int re = __reduce_max_sync(0xffffffffu, max(oz_exp(a.x), oz_exp(a.y)));
+      if (lane == 0 && re) atomicMax(rmax + (kMode == 0 ? s * 64 : 0) + r, re);
+      x[i] = make_double2(a.x * w, a.y * w);
+      cm = max(cm, max(oz_exp(x[i].x), oz_exp(x[i].y)));
+    }
+    if (cm) atomicMax(cmax + (kMode == 0 ? s * 32 : 0) + k, cm);
+  }
+  __syncthreads();
+  if (threadIdx.x < (kMode == 0 ? 128 : tr))
+    rexp[(int64_t)t.part * 2 * tr + (kMode == 0 ? 0 : s * tr) + threadIdx.x] = rmax[threadIdx.x];
+  {
+    const int em = cmax[(kMode == 0 ? s * 32 : 0) + k];
+#pragma unroll
+    for (int ri = 0; ri < 2; ++ri) {
+      const int c = kMode == 0 ? (s * 2 + ri) * 32 + k : ri * (kRows / 2) + k;
+      unsigned long long v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = oz_fixed(ri ? x[i].y : x[i].x, em);
+      oz_store(smem_raw + (uint32_t)(c >> 3) * kSbo + rg * 128 + (c & 7) * 16, kSlice, v);
+    }
+  }
+  tc::fence_async_smem();
+  __syncthreads();
+  const uint32_t base = tc::smem_u32(smem_raw);
+  // levels [l0, l1) of product `prod` into the accumulators at column (l - l0) * 128
+  auto issue = [&](int prod, int l0, int l1) {
+    if (threadIdx.x != 0) return;
+    tc::fence_after_sync();
+    for (int ks = 0; ks < Kt / 16; ++ks) {
+      auto desc = [&](int slice, int row) {
+        return tc::smem_desc(base + slice * kSlice + (uint32_t)(row >> 3) * kSbo + ks * 256, 128, kSbo);
+      };
+      for (int i = 0; i < l1; ++i) {
+        const int j0 = l0 > i ? l0 - i : 0, j1 = l1 - i;  // j0 <= j < j1
+        if (kMode == 2) {
+          for (int j = j0; j < j1; ++j) {
+            const uint32_t d = tmem + (uint32_t)(i + j - l0) * 128u;
+            mma_f16(d, desc(i, 0), desc(j, prod ? 128 : 0), 128, ks || i ? 1u : 0u);
+            if (!prod) mma_f16(d, desc(i, 128), desc(j, 128), 128, 1u);
+          }
+        } else {
+          for (int j = j0; j < j1; j += 2)
+            mma_f16(tmem + (uint32_t)(i + j - l0) * 128u, desc(i, 0), desc(j, 0), j + 1 < j1 ? 256 : 128,
+                    ks || i ? 1u : 0u);
+        }
+      }
+    }
+    tc::mma_commit(bars);
+  };
+  uint32_t phase = 0;
+  bool ok = true;
+  const int m = 32 * (warp & 3) + lane, n0 = 32 * (warp >> 2);
+  const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)n0;
+  double* dump = reinterpret_cast<double*>(smem_raw);
+  const int D2 = D * D;
+  double2* out = partials + (int64_t)t.part * 2 * D2;
+  for (int prod = 0; prod < (kMode == 2 ? 2 : 1) && ok; ++prod) {
+    long long acc[32];
+    issue(prod, 0, 4);
+    ok = oz_wait(bars, phase);
+    if (!ok) break;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      uint32_t v[4][8];
+#pragma unroll
+      for (int l = 0; l < 4; ++l) tmem_ld8(tq + l * 128 + b * 8, v[l]);
+      tmem_ld_wait();
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        long long h = 0;
+#pragma unroll
+        for (int l = 0; l < 4; ++l)
+          h += (long long)__float2int_rn(__uint_as_float(v[l][q])) * (1ll << (8 * (3 - l)));
+        acc[8 * b + q] = h * 65536;
+      }
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    issue(prod, 4, 7);
+    ok = oz_wait(bars, phase);
+    if (!ok) break;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      uint32_t v[3][8];
+#pragma unroll
+      for (int l = 0; l < 3; ++l) tmem_ld8(tq + l * 128 + b * 8, v[l]);
+      tmem_ld_wait();
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        long long h = 0;
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+          h += (long long)__float2int_rn(__uint_as_float(v[l][q])) * (1ll << (8 * (2 - l)));
+        acc[8 * b + q] += h >> 8;
+      }
+    }
+    tc::fence_before_sync();
+    // both passes are complete: the digits are free unless a second product follows
+    if (kMode == 2 && prod == 0) {
+      const int ea = cmax[m];
+#pragma unroll
+      for (int q = 0; q < 32; ++q) {
+        const int l = n0 + q;
+        if (m < D && l < D) out[s * D2 + m * D + l].x = oz_value(acc[q], ea, cmax[l]);
+      }
+    } else {
+      auto ce = [&](int c) { return cmax[kMode == 0 ? (c >> 6) * 32 + (c & 31) : kMode == 1 ? (c & 63) : c]; };
+      const int ea = ce(m);
+#pragma unroll
+      for (int q = 0; q < 32; ++q) dump[m * kOzDumpLd + n0 + q] = oz_value(acc[q], ea, ce(n0 + q));
+    }
+    __syncthreads();
+  }
+  if (ok) {
+    if (kMode == 2) {
+      for (int o = threadIdx.x; o < D2; o += kOzThreads) {
+        const int a = o / D, b = o - a * D;
+        out[s * D2 + o].y = dump[a * kOzDumpLd + b] - dump[b * kOzDumpLd + a];
+      }
+    } else {
+      constexpr int kp = kMode == 0 ? 32 : 64;
+      for (int o = threadIdx.x; o < (kMode == 0 ? 2 : 1) * D2; o += kOzThreads) {
+        const int sp = kMode == 0 ? o / D2 : s, ab = kMode == 0 ? o - sp * D2 : o, a = ab / D, b = ab - a * D;
+        const int ra = (kMode == 0 ? sp * 64 : 0) + a, rb = (kMode == 0 ? sp * 64 : 0) + b;
+        out[sp * D2 + ab] = make_double2(dump[ra * kOzDumpLd + rb] + dump[(ra + kp) * kOzDumpLd + rb + kp],
+                                         dump[ra * kOzDumpLd + rb + kp] - dump[(ra + kp) * kOzDumpLd + rb]);
+      }
+    }
+  } else if (threadIdx.x == 0) {
+    atomicOr(flags, 4);
+  }
+  tc_teardown(tmem, 512);
+}
+
+// Rows [row0, row0 + 128) of end a, spin blockIdx.y, new bond indices [32 blockIdx.z, +32):
+// Gamma_a'[s][r][k'] = mask_r sum_k Ã_s[r][k] Y_s[k][k'] as a real product over K = (re/im, k),
+// 32 k at a time: M = 128 rows, N = (re/im, k') = 64.  Launched over the row tiles; the tiles
+// that do not start a 128-row block return at once.
+__global__ void __launch_bounds__(kOzThreads, 1)
+    oz_update_kernel(const TileDesc* __restrict__ tiles, const BondDesc* __restrict__ bonds, double2* gamma,
+                     const double* __restrict__ lam, const double2* __restrict__ Yall, const double* __restrict__ at,
+                     const int* __restrict__ rexp, int* flags, int D) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int ymax[32];
+  __shared__ __align__(8) uint64_t bars[2];
+  __shared__ uint32_t tslot;
+  __shared__ float mask[128];
+  __shared__ double cut[2];
+  const TileDesc t = tiles[blockIdx.x];
+  if (t.row0 & 127) return;
+  const SideDesc sa = bonds[t.bond].a;
+  const int s = blockIdx.y, kp0 = 32 * blockIdx.z, D2 = D * D;
+  const double2* Y = Yall + ((int64_t)t.bond * 2 + s) * D2;
+  const int nrows = sa.rows - t.row0 < 128 ? sa.rows - t.row0 : 128;
+  const int tr = tile_rows(D, 16);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < 32) ymax[threadIdx.x] = 0;
+  const uint32_t tmem = tc_setup(&tslot, bars, 512);
+  tc_row_mask<false>(sa, lam, t.row0, nrows, D, mask, cut);
+  {
+    int e = 0;
+    if (kp0 + lane < D)
+      for (int k = warp; k < D; k += 16) {
+        const double2 y = Y[k * D + kp0 + lane];
+        e = max(e, max(oz_exp(y.x), oz_exp(y.y)));
+      }
+    if (e) atomicMax(ymax + lane, e);
+  }
+  __syncthreads();
+  unsigned char* sb = smem_raw + kOzOperand;
+  constexpr uint32_t kSa = 128 * 64 * 2, kSb = 64 * 64 * 2, kSbo = 64 * 16;
+  const uint32_t abase = tc::smem_u32(smem_raw), bbase = tc::smem_u32(sb);
+  const int nchunk = (D + 31) / 32;
+  const int m = 32 * (warp & 3) + lane, q0 = 8 * (warp >> 2);
+  const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)q0;
+  long long ar[8], ai[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) ar[q] = ai[q] = 0;
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int ch = 0; ch < nchunk && ok; ++ch) {
+    const int k0 = 32 * ch;
+    // left operand: 8 rows x 4 groups of 8 k per warp and part (re, im)
+#pragma unroll
+    for (int ri = 0; ri < 2; ++ri) {
+      const int r = warp * 8 + (lane & 7), kg = lane >> 3, kk = k0 + kg * 8;
+      unsigned long long v[8];
+      double a[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) a[e] = 0.0;
+      int em = 0;
+      if (r < nrows) {
+        const int part = t.part + r / tr, rr = r % tr;
+        em = rexp[(int64_t)part * 2 * tr + s * tr + rr];
+        const double* src = at + oz_at(part, s, rr, ri, tr, D) + kk;
+        if ((D & 7) == 0 && kk < D) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const double2 d = *reinterpret_cast<const double2*>(src + 2 * e);
+            a[2 * e] = d.x;
+            a[2 * e + 1] = d.y;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            if (kk + e < D) a[e] = src[e];
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = oz_fixed(a[e], em);
+      oz_store(smem_raw + warp * kSbo + (ri * 4 + kg) * 128 + (lane & 7) * 16, kSa, v);
+    }
+    // right operand: row n = (ro, k'), K = (ri, k): ro = ri -> yr; (0, 1) -> -yi; (1, 0) -> yi
+    {
+      const int ro = warp >> 3, ri = (warp >> 2) & 1, kp = (warp & 3) * 8 + (lane & 7), kg = lane >> 3;
+      const int em = ymax[kp];
+      unsigned long long v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int k = k0 + kg * 8 + e;
+        double2 y = make_double2(0.0, 0.0);
+        if (k < D && kp0 + kp < D) y = Y[k * D + kp0 + kp];
+        v[e] = oz_fixed(ro == ri ? y.x : y.y, em, ro < ri);
+      }
+      oz_store(sb + (uint32_t)(ro * 4 + (warp & 3)) * kSbo + (ri * 4 + kg) * 128 + (lane & 7) * 16, kSb, v);
+    }
+    tc::fence_async_smem();
+    __syncthreads();
+    const bool fresh = (ch & 1) == 0;
+    if (threadIdx.x == 0) {
+      tc::fence_after_sync();
+      for (int ks = 0; ks < 4; ++ks)
+        for (int i = 0; i < kOzSlices; ++i)
+          for (int j = 0; j < kOzSlices - i; j += 4) {
+            const int cnt = kOzSlices - i - j < 4 ? kOzSlices - i - j : 4;
+            mma_f16(tmem + (uint32_t)(i + j) * 64u, tc::smem_desc(abase + i * kSa + ks * 256, 128, kSbo),
+                    tc::smem_desc(bbase + j * kSb + ks * 256, 128, kSbo), 64 * cnt, fresh && !ks && !i ? 0u : 1u);
+          }
+      tc::mma_commit(bars);
+    }
+    ok = oz_wait(bars, phase);
+    // exact to 128 K values: read the accumulators after every second chunk
+    if (ok && (!fresh || ch + 1 == nchunk)) {
+      long long hr[8], hi[8], lr[8], li[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) hr[q] = hi[q] = lr[q] = li[q] = 0;
+#pragma unroll
+      for (int l = 0; l < kOzSlices; ++l) {
+        uint32_t vr[8], vi[8];
+        tmem_ld8(tq + l * 64, vr);
+        tmem_ld8(tq + l * 64 + 32, vi);
+        tmem_ld_wait();
+        const long long f = 1ll << (l < 4 ? 8 * (3 - l) : 8 * (6 - l));
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          (l < 4 ? hr : lr)[q] += (long long)__float2int_rn(__uint_as_float(vr[q])) * f;
+          (l < 4 ? hi : li)[q] += (long long)__float2int_rn(__uint_as_float(vi[q])) * f;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        ar[q] += hr[q] * 65536 + (lr[q] >> 8);
+        ai[q] += hi[q] * 65536 + (li[q] >> 8);
+      }
+      tc::fence_before_sync();
+    }
+    __syncthreads();
+  }
+  if (ok && m < nrows) {
+    const int part = t.part + m / tr, rr = m % tr;
+    const int em = rexp[(int64_t)part * 2 * tr + s * tr + rr];
+    const bool cut_row = mask[m] == 0.f;
+    const RowPos p = row_pos(sa, t.row0 + m);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int kp = kp0 + q0 + q;
+      if (kp < D) {
+        const int ey = ymax[q0 + q];
+        double2 v = make_double2(oz_value(ar[q], em, ey), oz_value(ai[q], em, ey));
+        if (cut_row) v = cscale(v, 0.0);
+        gamma[elem(sa, s, p, kp)] = v;
+      }
+    }
+  }
+  if (!ok && threadIdx.x == 0) atomicOr(flags, 4);
+  tc_teardown(tmem, 512);
+}
+
+}  // namespace gpeps

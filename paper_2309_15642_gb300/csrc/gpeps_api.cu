@@ -74,6 +74,7 @@ struct gpeps_handle {
   size_t s_lam = 0, s_gamma = 0;
   size_t w_pending = 0, w_flags = 0, w_sweeps = 0, w_cycles = 0, w_queue = 0, w_z = 0, w_mean = 0, w_sites = 0, w_inst_site0 = 0,
          w_site_inst = 0, w_site_off = 0, w_partials = 0, w_Y = 0, w_theta_a = 0, w_bond_scratch = 0;
+  size_t w_at = 0, w_rexp = 0, w_cs = 0;  // complex128 tensor-core passes
   size_t bond_slot = 0;  // bytes per bond-kernel CTA of global scratch for its n x n matrices
   int bond_slots = 0;    // slots in the work buffer
   char* d_state = nullptr;
@@ -106,6 +107,13 @@ struct gpeps_handle {
   unsigned long long* cycles() const { return reinterpret_cast<unsigned long long*>(d_work + w_cycles); }
   double* z() const { return reinterpret_cast<double*>(d_work + w_z); }
   double* mean() const { return reinterpret_cast<double*>(d_work + w_mean); }
+  // complex128 from D = kOzMinD: the larger ends' passes run on the tensor cores, as launches of
+  // their own (they take a whole SM's shared memory and TMEM), so a step is layered on every schedule
+  bool oz() const { return elt == 16 && OzPass::supported(D); }
+  bool fused() const { return schedule >= 4 && !oz(); }
+  OzPass::Scratch oz_scratch() const {
+    return OzPass::Scratch{at<double>(w_at), at<int>(w_rexp), d_work + w_cs};
+  }
   template <typename P>
   P* at(size_t off) const {
     return reinterpret_cast<P*>(d_work + off);
@@ -227,8 +235,13 @@ struct PhaseEvents {
 };
 
 // CTAs per SM of the layered bond launch (schedule 4 runs its layers, outside
-// gpeps_step, on the work queue with two CTAs per SM where they fit)
-int layered_per_sm(const gpeps_handle* h) {
+// gpeps_step, on the work queue with two CTAs per SM where they fit).  A
+// complex128 class that leaves SMs without a bond takes one 512-thread CTA per
+// SM whatever the schedule: sharing an SM would only halve the threads of each
+// (48 bonds at D = 64: 116 M SM cycles per bond at two 256-thread CTAs per SM,
+// 100 M at one of 512).
+int layered_per_sm(const gpeps_handle* h, int n_bonds) {
+  if (h->elt == 16 && n_bonds <= h->n_sms) return 1;
   switch (h->schedule) {
     case 2: return 2;
     case 3: return 4;
@@ -268,7 +281,10 @@ int layer_impl(gpeps_handle* h, int c, PhaseEvents* pe = nullptr, void* vsave = 
   void* Y = h->d_work + h->w_Y;
   double* theta_a = h->at<double>(h->w_theta_a);
   if (pe) GP_CUDA(cudaEventRecord(pe->ev[0], h->stream));
-  if (h->tensor)
+  if (h->oz())
+    GP_CUDA(OzPass::gram(tiles, nt, bonds, nbd, h->gamma(), h->lam(), h->pending(), partials, h->oz_scratch(),
+                         h->flags(), h->D, h->stream));
+  else if (h->tensor)
     GP_CUDA(Launch<T>::gram_tc(bonds, nbd, h->gamma(), h->lam(), h->pending(), partials, h->flags(), h->D,
                                h->stream));
   else
@@ -277,9 +293,11 @@ int layer_impl(gpeps_handle* h, int c, PhaseEvents* pe = nullptr, void* vsave = 
   GP_CUDA(Launch<T>::bond(bonds, nbd, partials, h->gamma(), h->lam(), h->pending(), Y, theta_a, h->flags(),
                           h->sweeps(), h->cycles(), vsave, h->D, h->jp, h->stream,
                           h->schedule ? h->at<unsigned int>(h->w_queue) : nullptr, h->n_sms,
-                          h->d_work + h->w_bond_scratch, layered_per_sm(h)));
+                          h->d_work + h->w_bond_scratch, layered_per_sm(h, nbd)));
   if (pe) GP_CUDA(cudaEventRecord(pe->ev[2], h->stream));
-  if (h->tensor)
+  if (h->oz())
+    GP_CUDA(OzPass::update(tiles, nt, bonds, h->gamma(), h->lam(), Y, h->oz_scratch(), h->flags(), h->D, h->stream));
+  else if (h->tensor)
     GP_CUDA(Launch<T>::update_tc(bonds, nbd, h->gamma(), h->lam(), Y, theta_a, h->flags(), h->D, h->stream));
   else
     GP_CUDA(Launch<T>::update(tiles, nt, bonds, h->gamma(), h->lam(), Y, theta_a, h->D, h->stream));
@@ -320,7 +338,7 @@ int readout_impl(gpeps_handle* h) {
 int one_step(gpeps_handle* h, const double* theta, int per_qubit) {
   int st = kick_impl(h, theta, per_qubit);
   if (st) return st;
-  if (h->schedule >= 4) {
+  if (h->fused()) {
     st = h->dtype == GPEPS_C128 ? fused_step_impl<double>(h) : fused_step_impl<float>(h);
     if (st) return st;
   } else {
@@ -521,6 +539,11 @@ int gpeps_create(const gpeps_graph* graphs, int32_t n_instances, int32_t D, int3
   h->w_partials = carve((size_t)h->max_parts * 2 * D * D * h->elt);
   h->w_Y = carve((size_t)h->max_bonds * 2 * D * D * h->elt);
   h->w_theta_a = carve((size_t)h->max_bonds * sizeof(double));
+  if (h->oz()) {
+    h->w_at = carve((size_t)h->max_parts * OzPass::at_doubles(D) * sizeof(double));
+    h->w_rexp = carve((size_t)h->max_parts * OzPass::rexp_ints(D) * sizeof(int));
+    h->w_cs = carve((size_t)h->max_bonds * sizeof(double2));
+  }
   // n x n bond matrices outside shared memory (a CTA indexes its slot by
   // blockIdx.x): beyond the shared-memory limit one slot per bond of the largest
   // class; otherwise slots for the two-CTAs-per-SM schedule only
@@ -554,6 +577,7 @@ int gpeps_bind(gpeps_handle* h, void* d_state, void* d_work) {
   h->d_state = static_cast<char*>(d_state);
   h->d_work = static_cast<char*>(d_work);
   GP_CUDA(h->dtype == GPEPS_C128 ? Launch<double>::init() : Launch<float>::init());
+  if (h->oz()) GP_CUDA(OzPass::init());
   {
     int dev = 0;
     GP_CUDA(cudaGetDevice(&dev));
@@ -633,7 +657,7 @@ int gpeps_step_profiled(gpeps_handle* h, const double* theta, int32_t per_qubit,
     int st = kick_impl(h, theta, per_qubit ? 1 : 0);
     if (st) return st;
     GP_CUDA(cudaEventRecord(ev[1], h->stream));
-    if (h->schedule >= 4) {
+    if (h->fused()) {
       st = h->dtype == GPEPS_C128 ? fused_step_impl<double>(h) : fused_step_impl<float>(h);
     } else {
       for (int c = 0; c < (int)h->colours.size() && !st; ++c) st = layer(h, c);

@@ -22,6 +22,7 @@ constexpr int kTileRows = 64;      // rows of a big-side tile (Gram and update l
 __host__ __device__ constexpr int tile_rows(int D, size_t elt) { return (D > kMaxD && elt == 16) ? 32 : kTileRows; }
 // Columns of Y_s that the update passes hold in shared memory at once
 __host__ __device__ constexpr int y_cols(int D) { return D > kMaxD ? 32 : D; }
+constexpr int kOzMinD = 17;        // smallest D of the complex128 tensor-core passes
 constexpr int kThreads = 256;      // threads of the streaming and readout CTAs
 constexpr int kBondThreads = 512;  // threads of the bond-eigenproblem CTA (one CTA per SM: more warps hide FP64 latency)
 constexpr double kLambdaCut = 1e-13;  // pseudo-inverse threshold relative to max(lambda)
@@ -161,6 +162,24 @@ struct Launch {
                           void* scratch, size_t slot, int per_sm, bool tc = false);
 };
 
+
+// Gram and update passes of the larger ends in complex128 on the tensor cores (bigend_oz.cuh).
+struct OzPass {
+  struct Scratch {
+    double* at;   // kicked rows of end a, one slot of at_doubles per row tile
+    int* rexp;    // largest exponent of each of them, one slot of rexp_ints per row tile
+    void* cs;     // cos and sin of half the kick of end a, two doubles per bond
+  };
+  static constexpr bool supported(int D) { return D >= kOzMinD && D <= kMaxDc128; }
+  static size_t at_doubles(int D) { return (size_t)4 * tile_rows(D, 16) * D; }
+  static size_t rexp_ints(int D) { return (size_t)2 * tile_rows(D, 16); }
+  static cudaError_t init();
+  static cudaError_t gram(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, int n_bonds, const void* gamma,
+                          const double* lam, const double* pending, void* partials, const Scratch& ws, int* flags,
+                          int D, cudaStream_t st);
+  static cudaError_t update(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, void* gamma, const double* lam,
+                            const void* Y, const Scratch& ws, int* flags, int D, cudaStream_t st);
+};
 
 constexpr int kMaxGradD = 16;  // bond dimension limit of the reverse mode (shared memory of its bond kernel)
 

@@ -1800,6 +1800,11 @@ __device__ bool tc_update_pass(const SideDesc& sa, float2* gamma, const double* 
   return ok;
 }
 
+}  // namespace gpeps
+// complex128 passes on the tensor cores (they use the setup and mask helpers above)
+#include "bigend_oz.cuh"
+namespace gpeps {
+
 // Gram partials of one bond on the tensor cores, one partial per 64-row tile
 // (layered form of the mixed path; the partial layout of gram_kernel).
 __global__ void __launch_bounds__(128)
@@ -2357,6 +2362,45 @@ cudaError_t Launch<T>::update(const TileDesc* tiles, int n_tiles, const BondDesc
   const size_t sm = update_smem(D, sizeof(V2<T>));
   update_kernel<T><<<n_tiles, kThreads, sm, st>>>(tiles, bonds, static_cast<V2<T>*>(gamma), lam,
                                                    static_cast<const V2<T>*>(Y), theta_a, D);
+  return cudaGetLastError();
+}
+
+cudaError_t OzPass::init() {
+  cudaError_t e = cudaFuncSetAttribute(oz_gram_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzGramSmem);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(oz_gram_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzGramSmem);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(oz_gram_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzGramSmem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(oz_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzUpdateSmem);
+}
+
+cudaError_t OzPass::gram(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, int n_bonds, const void* gamma,
+                         const double* lam, const double* pending, void* partials, const Scratch& ws, int* flags,
+                         int D, cudaStream_t st) {
+  if (n_tiles == 0) return cudaSuccess;
+  if (!supported(D)) return cudaErrorInvalidValue;
+  double2* cs = static_cast<double2*>(ws.cs);
+  oz_kick_kernel<<<(n_bonds + 127) / 128, 128, 0, st>>>(bonds, n_bonds, pending, cs);
+  const double2* g = static_cast<const double2*>(gamma);
+  double2* out = static_cast<double2*>(partials);
+  if (D <= 32)
+    oz_gram_kernel<0><<<n_tiles, kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, ws.rexp, flags, D);
+  else if (D <= 64)
+    oz_gram_kernel<1><<<dim3(n_tiles, 2), kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, ws.rexp,
+                                                                          flags, D);
+  else
+    oz_gram_kernel<2><<<dim3(n_tiles, 2), kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, ws.rexp,
+                                                                          flags, D);
+  return cudaGetLastError();
+}
+
+cudaError_t OzPass::update(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, void* gamma, const double* lam,
+                           const void* Y, const Scratch& ws, int* flags, int D, cudaStream_t st) {
+  if (n_tiles == 0) return cudaSuccess;
+  if (!supported(D)) return cudaErrorInvalidValue;
+  oz_update_kernel<<<dim3(n_tiles, 2, (D + 31) / 32), kOzThreads, kOzUpdateSmem, st>>>(
+      tiles, bonds, static_cast<double2*>(gamma), lam, static_cast<const double2*>(Y), ws.at, ws.rexp, flags, D);
   return cudaGetLastError();
 }
 
