@@ -958,6 +958,8 @@ int grad_check(const gpeps_handle* h, int n_steps, int k) {
 
 JacobiParams grad_jacobi(const gpeps_handle* h) {
   JacobiParams jp = h->jp;
+  // forward and recomputed segments alike, so that both take the same gauge
+  jp.full_basis = 1;
   jp.ev_cut = 1e-14;  // Schmidt values <= 1e-7 of the largest are zero in both directions
   return jp;
 }

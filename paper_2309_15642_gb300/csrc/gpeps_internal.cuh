@@ -99,6 +99,7 @@ struct JacobiParams {
   double level_ratio;  // an extra FP32 level takes the diagonals below this fraction of their block's scale
   int levels;          // extra FP32 levels at most (0..kMaxExtraLevels)
   long long wait_cycles;  // fused step: a wait for an earlier task gives up after this many SM cycles
+  int full_basis;         // complex128: keep a complete unitary V per bond (the reverse mode; see bond_front_svd)
   int gate_sign;          // +1: the paper's exp(+i pi/4 Z Z); -1: its inverse exp(-i pi/4 Z Z)
 };
 
@@ -211,8 +212,9 @@ struct BondFootprint {
 // complex128, whose unsquared form always keeps its matrices in a global slot).
 BondFootprint bond_footprint(int D, size_t smem_optin, size_t elt);
 // The same with the n x n matrices always in a global slot (the FP32 level in
-// shared memory): the layout of the two-CTAs-per-SM schedule.
-BondFootprint bond_footprint_global(int D, size_t elt);
+// shared memory): the layout of the two-CTAs-per-SM schedule.  complex128 also
+// keeps the matrix it works on in shared memory where that stays within smem_limit.
+BondFootprint bond_footprint_global(int D, size_t elt, size_t smem_limit = 0);
 // CTAs of the bond kernel sharing an SM in the global-matrix schedules: 2 of
 // 256 threads or 4 of 128 threads, each with at most 1/k of the SM's 228 KB of
 // shared memory (less 1 KB for the CTA's own reservation)

@@ -122,48 +122,44 @@ __device__ __forceinline__ bool rotation(double app, double aqq, double2 apq, do
   return true;
 }
 
-// Rotation of the column pair with squared norms a, b and inner product
-// g = b_p^H b_q (g != 0), the one that diagonalises [[a, g], [conj(g), b]]:
-// the phase e = conj(g) / |g| first, then t = tan of the angle from
-// t^2 + 2 zeta t - 1 = 0, zeta = (b - a) / (2 |g|) (Golub & Van Loan Alg. 8.4.1),
-// for the one-sided Jacobi of the unsquared bond SVD.  The three entries are
-// first rescaled by the same power of two so that |g| ~ 1 (exact; the angle is
-// scale-free), so that the FP32 seeds below cannot underflow; then the
-// Newton-Raphson refinements of `rotation` (two reciprocal-square-root steps
-// for 1/|g| and for c = 1/sqrt(1 + t^2), one step on the angle equation) make
-// the rotation unitary to FP64 rounding without FP64 divides or square roots.
-// When |zeta| is beyond FP32 range t = 1 / (2 zeta).
-// Also returns |g|.
-__device__ __forceinline__ void os_rotation(double a, double b, double2 g, double& c, double& s, double2& e,
-                                            double& ag) {
-  int ex;
-  frexp(fma(g.x, g.x, g.y * g.y), &ex);
-  const int k = ex >> 1;  // |g| ~ 2^k
-  a = ldexp(a, -k);
-  b = ldexp(b, -k);
-  g = make_double2(ldexp(g.x, -k), ldexp(g.y, -k));
-  const double g2 = fma(g.x, g.x, g.y * g.y);  // in [1/4, 2)
-  double ig = (double)rsqrtf((float)g2);
-  ig = ig * (1.5 - 0.5 * g2 * ig * ig);
-  ig = ig * (1.5 - 0.5 * g2 * ig * ig);
-  const double zeta = (b - a) * (0.5 * ig);
-  double t;
-  if (fabs(zeta) < 1e18) {
-    const float zf = (float)zeta;
-    t = (double)(copysignf(1.f, zf) / (fabsf(zf) + sqrtf(fmaf(zf, zf, 1.f))));
-    const double f = fma(t, t, fma(2.0 * zeta, t, -1.0));
-    t -= f * (double)__frcp_rn((float)(2.0 * (t + zeta)));
-  } else {
-    t = 0.5 / zeta;
-  }
-  const double u = fma(t, t, 1.0);
-  double cc = (double)rsqrtf((float)u);
-  cc = cc * (1.5 - 0.5 * u * cc * cc);
-  cc = cc * (1.5 - 0.5 * u * cc * cc);
-  c = cc;
-  s = t * cc;
-  e = make_double2(g.x * ig, -g.y * ig);
-  ag = ldexp(g2 * ig, k);
+// v 2^(1023 - E) as a float (E: a biased exponent; zero below the float range) and back:
+// integer arithmetic, since the FP64 <-> FP32 conversions run on the FP64 unit
+__device__ __forceinline__ float os_down(double v, int E) {
+  const int hi = __double2hiint(v), lo = __double2loint(v), e = ((hi >> 20) & 0x7ff) - E + 127;
+  const int m = ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29);
+  return e > 0 && e < 255 ? __int_as_float((hi & 0x80000000) | (e << 23) | m) : 0.f;
+}
+__device__ __forceinline__ double os_up(float f, int E) {  // f 2^(1023 - E), f a normal number
+  const int b = __float_as_int(f), e = ((b >> 23) & 0xff) - 127 + 2046 - E;
+  return __hiloint2double((b & 0x80000000) | (e << 20) | ((b & 0x7fffff) >> 3), b << 29);
+}
+
+// Rotation of the column pair with squared norms a, b, inner product g = b_p^H b_q
+// and g2 = |g|^2 (not zero), the one that diagonalises [[a, g], [conj(g), b]], for
+// the one-sided Jacobi of the unsquared bond SVD: b_p <- c (b_p - z b_q), b_q <-
+// c (b_q + conj(z) b_p), z = t e, e = conj(g) / |g| (Golub & Van Loan Alg. 8.4.1
+// without the phase on b_q, which changes no angle).  tau = t / |g| is the small
+// root of g2 tau^2 + (b - a) tau - 1 = 0, so neither |g| nor its inverse is formed:
+// an FP32 value, from operands scaled by the power of two of the largest, and one
+// Newton step with the FP32 derivative (relative error about 1e-7 x 1e-7).  c =
+// 1 / sqrt(1 + t^2) from FP32 and one third-order step, to rounding, so that the
+// rotation is unitary whatever the angle's error.  Returns tau, c, u = 1 + t^2 and
+// w = t |g| (the squared norms become a - w and b + w).
+__device__ __forceinline__ void os_rotation(double a, double b, double2 g, double g2, double& tau, double& c,
+                                            double& u, double& w) {
+  const double del = b - a;
+  const int eg = max((__double2hiint(g.x) >> 20) & 0x7ff, (__double2hiint(g.y) >> 20) & 0x7ff);
+  const int E = max(eg, (__double2hiint(del) >> 20) & 0x7ff);
+  const float df = os_down(del, E), gx = os_down(g.x, E), gy = os_down(g.y, E);
+  const float sq = copysignf(sqrtf(fmaf(df, df, 4.f * fmaf(gx, gx, gy * gy))), df);
+  tau = os_up(2.f / (df + sq), E);
+  const double w0 = __dmul_rn(g2, tau);
+  tau = fma(-fma(w0, tau, fma(del, tau, -1.0)), os_up(1.f / sq, E), tau);
+  w = __dmul_rn(g2, tau);  // (rounded products: the same bits in every kernel that inlines this)
+  u = fma(w, tau, 1.0);
+  const double y = os_up(rsqrtf(os_down(u, 1023)), 1023);
+  const double rho = fma(-u, y * y, 1.0);
+  c = fma(y, rho * fma(rho, 0.375, 0.5), y);
 }
 
 // Storage of the Hermitian matrix of a Jacobi solve.  HermFull: n x n with row

@@ -21,11 +21,16 @@ __global__ void rotation_selftest_kernel(int which, int n, const double* __restr
   if (k >= n) return;
   const double a = in[4 * k], b = in[4 * k + 1];
   const double2 g = make_double2(in[4 * k + 2], in[4 * k + 3]);
-  double c = 1.0, s = 0.0, ag = 0.0;
+  double c = 1.0, s = 0.0;
   double2 e = make_double2(1.0, 0.0);
   if (which == 0) rotation(a, b, g, 0.0, 0.0, c, s, e);  // thresholds 0: every g != 0 rotates
-  else os_rotation(a, b, g, c, s, e, ag);
   const double gr = hypot(g.x, g.y);
+  if (which == 1) {  // tau = t / |g| and c; s and e from them
+    double tau, u, w;
+    os_rotation(a, b, g, fma(g.x, g.x, g.y * g.y), tau, c, u, w);
+    s = tau * gr * c;
+    e = make_double2(g.x / gr, -g.y / gr);
+  }
   const double zeta = (b - a) / (2.0 * gr);
   const double t = fabs(zeta) > 1e150 ? 0.5 / zeta : copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
   const double cr = rsqrt(fma(t, t, 1.0));

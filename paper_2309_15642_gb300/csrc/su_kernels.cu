@@ -193,19 +193,24 @@ struct BondSmem {
 // the unsquared SVD form (SvdLayout, declared below) for complex128.
 __host__ __device__ size_t bond_big(int D, size_t elt);
 // Shared scratch after the small arrays: the FP32 level of the squared form, or
-// the FP32 warm start and levels of the unsquared form (svd_f32_bytes, below).
-__host__ __device__ size_t svd_f32_bytes(int D);
-static size_t bond_f32(int D, size_t elt) { return elt == 16 ? svd_f32_bytes(D) : BondSmem(D, 2 * D).f32; }
+// that of the unsquared form (below), with or without the matrix it works on.
+__host__ __device__ size_t svd_shared_bytes(int D, bool with_work);
+__host__ __device__ size_t svd_shared_work(int D);
+static size_t bond_f32(int D, size_t elt, bool with_work) {
+  return elt == 16 ? svd_shared_bytes(D, with_work) : BondSmem(D, 2 * D).f32;
+}
+
+BondFootprint bond_footprint_global(int D, size_t elt, size_t smem_limit) {
+  const BondSmem L(D, 2 * D);
+  const size_t with = L.small + bond_f32(D, elt, true);
+  return BondFootprint{with <= smem_limit ? with : L.small + bond_f32(D, elt, false),
+                       (bond_big(D, elt) + 255) & ~(size_t)255};
+}
 
 BondFootprint bond_footprint(int D, size_t smem_optin, size_t elt) {
   const BondSmem L(D, 2 * D);
   if (elt == 8 && L.big + L.small <= smem_optin) return BondFootprint{L.big + L.small, 0};
-  return BondFootprint{L.small + bond_f32(D, elt), (bond_big(D, elt) + 255) & ~(size_t)255};
-}
-
-BondFootprint bond_footprint_global(int D, size_t elt) {
-  const BondSmem L(D, 2 * D);
-  return BondFootprint{L.small + bond_f32(D, elt), (bond_big(D, elt) + 255) & ~(size_t)255};
+  return bond_footprint_global(D, elt, smem_optin);
 }
 
 
@@ -693,22 +698,21 @@ __device__ void load_F(const SideDesc& sb, const V2<T>* gamma, const double* lam
 // and Q_s isometric on the range of A~_s: Psi and M have the same singular
 // values and right singular vectors.  R_s is the pivoted Cholesky factor of G_s
 // (the bond's own lam enters only through M, so a pivot cut on G_s never drops a
-// bond index of small lam); the SVD of M is one-sided (Hestenes) Jacobi on B = M V0, preconditioned
-// by V0, the FP32 eigenvectors of M^H M re-orthonormalised in FP64, and by FP32
-// levels on rescaled blocks of B^H B whose columns are small (the Gram of B is
-// accurate relative to each column, unlike rho).  The Schmidt values are the
-// column norms of B, accurate to eps of the largest.
+// bond index of small lam); the SVD of M is one-sided (Hestenes) Jacobi on Z = M^H U0,
+// U0 the left singular vectors of M from FP32 (svd_basis) re-orthonormalised in FP64,
+// with FP32 levels on rescaled blocks of Z whose columns are small.  The Schmidt
+// values are the column norms of Z, accurate to eps of the largest.
 
 constexpr double kCholCut = 1e-15;     // pivoted Cholesky stops below this fraction of the largest diagonal
 constexpr double kNoiseRelSvd = 1e-30; // columns of B with |b|^2 below this fraction of ||M||_F^2 are rounding
 
 // Global-slot layout (complex doubles) of the unsquared bond update, fixed for
 // n = 2D so that every bond of a launch shares it:
-//   Mt  [2D][2D]     M^T (Mt[x][s D + j]); F [n][D] again for the epilogue
-//   RB  [2D][2D+1]   rho = M^H M (row stride n + 1); then B^T (Bt[j][r] = B[r][j], row stride 2D)
-//   Vx  [2D][2D]     F [n][D] first; then V0 and finally V (row x, column j)
-//   Xs  [2D][2D+1]   G_s [2][D][D+1] and R_s [2][D][D] first; then the FP32
-//                    level's scratch; then V^T (Vt[j][x], row stride n)
+//   Mt  [2D][2D]     M^T (Mt[x][s D + j]); scratch of the levels; F [n][D] again for the epilogue
+//   RB  [2D][2D+1]   FP32 warm start, then the columns worked on, where shared memory has no room for them
+//   Vx  [2D][2D]     F [n][D] first; then U0 (or V0) and finally V (row x, column j)
+//   Xs  [2D][2D+1]   G_s [2][D][D+1] and R_s [2][D][D] first; then the scratch of
+//                    `orthonormalise`; then V^T (Vt[j][x], row stride n) where it is accumulated
 struct SvdLayout {
   size_t off_Mt, off_RB, off_V, off_X, big;
   __host__ __device__ explicit SvdLayout(int D) {
@@ -798,8 +802,8 @@ __device__ void pivoted_cholesky2(double2* Cw, double2* Rr, int D, int* mask, in
       const double2* r = Rr + (size_t)sidx * D * D + (size_t)k * D;
       const double2 ri = r[i], rj = r[j];
       double2& c = Cw[(size_t)sidx * D * ldc + i * ldc + j];
-      c.x -= ri.x * rj.x + ri.y * rj.y;
-      c.y -= ri.x * rj.y - ri.y * rj.x;
+      c.x = fma(-ri.x, rj.x, fma(-ri.y, rj.y, c.x));
+      c.y = fma(-ri.x, rj.y, fma(ri.y, rj.x, c.y));
     }
     __syncthreads();
   }
@@ -837,13 +841,13 @@ __device__ __forceinline__ void round_pair(int r, int k, int n, int& p, int& q) 
   }
 }
 
-// Rotation of a column pair in FP32 (the warm start and the levels): the same
-// angle as `os_rotation`, in plain FP32 arithmetic (the FP32 stages work on
-// matrices scaled to unit Frobenius norm and skip pairs with |g| below 1e-13,
-// so nothing underflows).  1/|g| and c = 1/sqrt(1+t^2) get one Newton step each
-// so that |e| = 1 and c^2 + s^2 = 1 to FP32 rounding: a column of a 128-wide
-// solve takes ~1500 rotations, and the ~2e-7 of rsqrtf alone would leave the
-// accumulated rotation ~3e-4 away from unitary.
+// Rotation of a column pair in FP32 (the warm start and the levels), from its
+// squared norms a, b and g = b_p^H b_q (g != 0): the phase e = conj(g) / |g|, then
+// t = tan of the angle from t^2 + 2 zeta t - 1 = 0, zeta = (b - a) / (2 |g|) (Golub
+// & Van Loan Alg. 8.4.1).  1/|g| and c = 1/sqrt(1+t^2) get one Newton step each so
+// that |e| = 1 and c^2 + s^2 = 1 to FP32 rounding: a column of a 128-wide solve
+// takes ~1000 rotations, and the ~2e-7 of rsqrtf alone would leave the accumulated
+// rotation ~3e-4 away from unitary.
 __device__ __forceinline__ void os_rot(float a, float b, float2 g, float& c, float& s, float2& e) {
   const float g2 = fmaf(g.x, g.x, g.y * g.y);
   float ig = rsqrtf(g2);
@@ -857,38 +861,29 @@ __device__ __forceinline__ void os_rot(float a, float b, float2 g, float& c, flo
   s = t * cc;
   e = make_float2(g.x * ig, -g.y * ig);
 }
-__device__ __forceinline__ void os_rot(double a, double b, double2 g, double& c, double& s, double2& e) {
-  double ag;
-  os_rotation(a, b, g, c, s, e, ag);
-}
 
-// One-sided (Hestenes) Jacobi on the n columns of B (Bt [n][rows]), with V^T
-// (Vt [n][n]) rotated alongside, in the arithmetic of R (FP32 for the warm start
-// and the levels, FP64 for the final sweeps).  A sweep runs the n - 1 rounds of
-// the round-robin pairing; a round (1) forms |b_p|^2, |b_q|^2 and g = b_p^H b_q
-// of its n/2 disjoint pairs from the columns themselves (8 lanes per pair), (2)
-// decides and builds every rotation with one thread per pair (`os_rot`): pair
+// One-sided (Hestenes) Jacobi in FP32 on the n columns of B (Bt [n], stride ld, of
+// `rows` entries), with W^T (Wt [n][n], or null) rotated alongside.  A sweep runs
+// the n - 1 rounds of the round-robin pairing; a round (1) forms |b_p|^2, |b_q|^2
+// and g = b_p^H b_q of its n/2 disjoint pairs from the columns themselves (8 lanes
+// per pair), (2) decides and builds every rotation with one thread per pair: pair
 // (p, q) rotates when |g| > max(tol |b_p| |b_q|, floor_abs), by
-// b_p <- c b_p - s e b_q, b_q <- s b_p + c e b_q, (3) applies the rotations of
-// the active pairs only, over the rows of B and V.  Norms are never carried
-// over from earlier rotations (a closed-form update loses digits when a pair is
-// nearly parallel, and every later angle of that column would inherit the
-// error).  A sweep without rotations ends the solve.  Returns the sweeps
+// b_p <- c b_p - s e b_q, b_q <- s b_p + c e b_q, (3) applies the rotations of the
+// active pairs only.  A sweep without rotations ends the solve.  Returns the sweeps
 // (max_sweeps + 1 = cap hit); work[0] += pair checks, work[1] += rotations,
 // rot_count[sweep] += rotations of the first kRotSweeps sweeps (either may be
 // null).  rc, rs: n/2 reals; re: n/2 complex; iflag: the integer scratch of
 // jacobi_hermitian.  n <= 256, blockDim.x >= n/2 rounded up to 32.
-template <typename R>
-__device__ int one_sided_jacobi(V2<R>* Bt, int rows, V2<R>* Vt, int n, R tol, R floor_abs, int max_sweeps, R* rc,
-                                R* rs, V2<R>* re, int* iflag, unsigned long long* work,
-                                unsigned long long* rot_count) {
+__device__ int one_sided_jacobi32(float2* Bt, int ld, int rows, float2* Wt, int n, float tol, float floor_abs,
+                                  int max_sweeps, float* rc, float* rs, float2* re, int* iflag,
+                                  unsigned long long* work, unsigned long long* rot_count) {
   const int m = n / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int sub = lane & 7, grp = lane >> 3;
   int* act = iflag + 8;     // [4 warps][32] active pairs of the round
   int* wcnt = iflag + 136;  // active pairs per warp
   const int npw = (m + 31) >> 5;  // warps that build the rotations (n <= 256: at most 4)
-  const R tol2 = tol * tol, floor2 = floor_abs * floor_abs;
-  const int len = rows + n;
+  const float tol2 = tol * tol, floor2 = floor_abs * floor_abs;
+  const int len = rows + (Wt ? n : 0);
   unsigned long long n_chk = 0, n_rot = 0;
   int result = max_sweeps + 1;
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
@@ -897,18 +892,18 @@ __device__ int one_sided_jacobi(V2<R>* Bt, int rows, V2<R>* Vt, int n, R tol, R 
       // (1) norms and inner product of every pair: rc[k] = |b_p|^2, rs[k] = |b_q|^2, re[k] = g
       for (int k0 = warp * 4; k0 < m; k0 += nw * 4) {
         const int k = k0 + grp;
-        R a = 0, b = 0;
-        V2<R> g = mk<R>(0, 0);
+        float a = 0, b = 0;
+        float2 g = make_float2(0.f, 0.f);
         if (k < m) {
           int p, q;
           round_pair(r, k, n, p, q);
-          const V2<R>* bp = Bt + (size_t)p * rows;
-          const V2<R>* bq = Bt + (size_t)q * rows;
+          const float2* bp = Bt + (size_t)p * ld;
+          const float2* bq = Bt + (size_t)q * ld;
           for (int i = sub; i < rows; i += 8) {
-            const V2<R> u = bp[i], v = bq[i];
-            a = fma(u.x, u.x, fma(u.y, u.y, a));
-            b = fma(v.x, v.x, fma(v.y, v.y, b));
-            fma_conj<R>(g, u, v);
+            const float2 u = bp[i], v = bq[i];
+            a = fmaf(u.x, u.x, fmaf(u.y, u.y, a));
+            b = fmaf(v.x, v.x, fmaf(v.y, v.y, b));
+            fma_conj<float>(g, u, v);
           }
         }
         for (int off = 4; off > 0; off >>= 1) {
@@ -929,13 +924,13 @@ __device__ int one_sided_jacobi(V2<R>* Bt, int rows, V2<R>* Vt, int n, R tol, R 
         const int k = threadIdx.x;
         bool on = false;
         if (k < m) {
-          const V2<R> g = re[k];
-          const R a = rc[k], b = rs[k];
-          const R g2 = fma(g.x, g.x, g.y * g.y);
+          const float2 g = re[k];
+          const float a = rc[k], b = rs[k];
+          const float g2 = fmaf(g.x, g.x, g.y * g.y);
           on = g2 > tol2 * a * b && g2 > floor2;
           if (on) {
-            R c, sn;
-            V2<R> e;
+            float c, sn;
+            float2 e;
             os_rot(a, b, g, c, sn, e);
             rc[k] = c;
             rs[k] = sn;
@@ -956,18 +951,20 @@ __device__ int one_sided_jacobi(V2<R>* Bt, int rows, V2<R>* Vt, int n, R tol, R 
         n_rot += (unsigned long long)na;
       }
       if (na == 0) continue;  // nothing below reads this round's scratch
-      // (3) the active rotations over the rows of B, then of V
+      // (3) the active rotations over the rows of B, then of W
       for (int t = threadIdx.x; t < na * len; t += blockDim.x) {
         const int ia = t / len, i = t - ia * len;
         const int k = ia < p1 ? act[ia] : ia < p2 ? act[32 + ia - p1] : ia < p3 ? act[64 + ia - p2] : act[96 + ia - p3];
         int p, q;
         round_pair(r, k, n, p, q);
-        V2<R>* xp = i < rows ? Bt + (size_t)p * rows + i : Vt + (size_t)p * n + (i - rows);
-        V2<R>* xq = i < rows ? Bt + (size_t)q * rows + i : Vt + (size_t)q * n + (i - rows);
-        const R c = rc[k], sn = rs[k];
-        const V2<R> u = *xp, v = c_mul<R>(*xq, re[k]);
-        *xp = mk<R>(c * u.x - sn * v.x, c * u.y - sn * v.y);
-        *xq = mk<R>(sn * u.x + c * v.x, sn * u.y + c * v.y);
+        float2* xp = i < rows ? Bt + (size_t)p * ld + i : Wt + (size_t)p * n + (i - rows);
+        float2* xq = i < rows ? Bt + (size_t)q * ld + i : Wt + (size_t)q * n + (i - rows);
+        const float c = rc[k], sn = rs[k];
+        // explicit roundings: the same bits in every kernel that inlines this
+        const float2 u = *xp, y = *xq, e = re[k];
+        const float2 v = make_float2(fmaf(y.x, e.x, -__fmul_rn(y.y, e.y)), fmaf(y.x, e.y, __fmul_rn(y.y, e.x)));
+        *xp = make_float2(fmaf(c, u.x, -__fmul_rn(sn, v.x)), fmaf(c, u.y, -__fmul_rn(sn, v.y)));
+        *xq = make_float2(fmaf(sn, u.x, __fmul_rn(c, v.x)), fmaf(sn, u.y, __fmul_rn(c, v.y)));
       }
       __syncthreads();
     }
@@ -986,47 +983,347 @@ __device__ int one_sided_jacobi(V2<R>* Bt, int rows, V2<R>* Vt, int n, R tol, R 
   return result;
 }
 
+// FP64 sweeps of the one-sided Jacobi on the n columns of Z (Zt [n][rows]), with
+// V^T (Vt [n][n], or null) rotated alongside; same rounds as one_sided_jacobi32.
+//
+// Bound by the FP64 unit (64 cycles per warp instruction), so the work per pair is
+// cut to what the rotation needs:
+//   * a round forms only g = z_p^H z_q (4 multiply-adds per element).  The squared
+//     norms are summed at the start of each sweep and follow the rotations in closed
+//     form, a' = a - t |g|, b' = b + t |g|; a column whose norm loses more than ~5
+//     bits in one rotation is marked (negative) and summed again when next used.
+//   * scaled rotations: the columns carry factors d (column = d y), so that a rotation is
+//     y_p -= al y_q, y_q += be y_p, al = z d_q / d_p, be = conj(z) d_p / d_q, d' = c d
+//     (8 multiply-adds per element pair instead of 12); the factors are multiplied
+//     out after each sweep.
+//   * os_rotation finds the angle without |g|, FP64 divides, square roots or conversions.
+//
+// A pair is left alone when |g| <= tol |z_p| |z_q|, when either column is rounding
+// (|z|^2 <= kNoiseRelSvd trace), or when |g| <= floor_abs; without V (the columns
+// become the singular vectors) only if also their overlap |g| / (|z_p| |z_q|) times
+// the larger norm, the error it makes in the state, is below 1e-16 of the matrix.
+// nrm: the squared norms on return.  dsc, dinv: n doubles; al, be: n/2 complex.
+__device__ int os_sweeps(double2* Zt, int rows, double2* Vt, int n, double tol, double floor_abs, double trace,
+                         int max_sweeps, double* nrm, double* dsc, double* dinv, double2* al, double2* be,
+                         int* iflag, unsigned long long* work, unsigned long long* rot_count) {
+  const int m = n / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int* act = iflag + 8;     // [4 warps][32] active pairs of the round
+  int* wcnt = iflag + 136;  // active pairs per warp
+  const int npw = (m + 31) >> 5;
+  // lanes per pair: the pairs of a round over four warps, one per SMSP, where n allows
+  int lpp = 32;
+  while (lpp > 4 && lpp * m > 128) lpp >>= 1;
+  const int sub = lane & (lpp - 1), ppw = 32 / lpp, grp = lane / lpp;
+  const double tol2 = tol * tol, noise = kNoiseRelSvd * trace, floor2 = floor_abs * floor_abs;
+  const double over = 1e-32 * trace;
+  unsigned long long n_chk = 0, n_rot = 0;
+  int result = max_sweeps + 1;
+  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
+    column_norms(Zt, rows, n, nrm);
+    for (int j = threadIdx.x; j < n; j += blockDim.x) dsc[j] = dinv[j] = 1.0;
+    if (threadIdx.x == 0) iflag[3] = 0;
+    __syncthreads();
+    for (int r = 0; r < n - 1; ++r) {
+      for (int k0 = warp * ppw; k0 < m; k0 += nw * ppw) {
+        const int k = k0 + grp;
+        int p = 0, q = 0;
+        double2 g = make_double2(0.0, 0.0);
+        bool dirty = false;
+        if (k < m) {
+          round_pair(r, k, n, p, q);
+          const double2* zp = Zt + (size_t)p * rows;
+          const double2* zq = Zt + (size_t)q * rows;
+#pragma unroll 4
+          for (int i = sub; i < rows; i += lpp) fma_conj<double>(g, zp[i], zq[i]);
+          dirty = __double2hiint(nrm[p]) < 0 || __double2hiint(nrm[q]) < 0;
+        }
+        for (int off = lpp >> 1; off > 0; off >>= 1) {
+          g.x += __shfl_xor_sync(0xffffffffu, g.x, off);
+          g.y += __shfl_xor_sync(0xffffffffu, g.y, off);
+        }
+        if (__any_sync(0xffffffffu, dirty)) {
+          double a = 0.0, b = 0.0;
+          if (dirty) {
+            const double2* zp = Zt + (size_t)p * rows;
+            const double2* zq = Zt + (size_t)q * rows;
+            for (int i = sub; i < rows; i += lpp) {
+              a = fma(zp[i].x, zp[i].x, fma(zp[i].y, zp[i].y, a));
+              b = fma(zq[i].x, zq[i].x, fma(zq[i].y, zq[i].y, b));
+            }
+          }
+          for (int off = lpp >> 1; off > 0; off >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, off);
+            b += __shfl_xor_sync(0xffffffffu, b, off);
+          }
+          if (dirty && sub == 0) {
+            nrm[p] = a * dsc[p] * dsc[p];
+            nrm[q] = b * dsc[q] * dsc[q];
+          }
+        }
+        if (k < m && sub == 0) al[k] = g;
+      }
+      __syncthreads();
+      if (warp < npw) {
+        const int k = threadIdx.x;
+        bool on = false;
+        int p = 0, q = 0;
+        double a = 0.0, b = 0.0, g2 = 0.0, dp = 1.0, dq = 1.0;
+        double2 g = make_double2(0.0, 0.0);
+        if (k < m) {
+          round_pair(r, k, n, p, q);
+          a = nrm[p];
+          b = nrm[q];
+          dp = dsc[p];
+          dq = dsc[q];
+          g = cscale(al[k], dp * dq);
+          g2 = fma(g.x, g.x, g.y * g.y);
+          const double lo = fmin(a, b);
+          on = g2 > tol2 * (a * b) && lo > noise && (g2 > floor2 || (!Vt && g2 > over * lo));
+        }
+        if (on) {
+          double tau, c, u, w;
+          os_rotation(a, b, g, g2, tau, c, u, w);
+          const double ic = c * u;
+          const double2 z = make_double2(tau * g.x, -tau * g.y);
+          const double ip = dinv[p], iq = dinv[q];
+          const double fa = dq * ip, fb = dp * iq;
+          al[k] = make_double2(z.x * fa, z.y * fa);
+          be[k] = make_double2(z.x * fb, -z.y * fb);
+          dsc[p] = dp * c;
+          dsc[q] = dq * c;
+          dinv[p] = ip * ic;
+          dinv[q] = iq * ic;
+          const double a1 = __dadd_rn(a, -w), b1 = __dadd_rn(b, w);
+          nrm[p] = a1 < 0.03 * a ? -1.0 : a1;
+          nrm[q] = b1 < 0.03 * b ? -1.0 : b1;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, on);
+        if (on) act[warp * 32 + __popc(bal & ((1u << lane) - 1u))] = k;
+        if (lane == 0) wcnt[warp] = __popc(bal);
+      }
+      __syncthreads();
+      const int p1 = wcnt[0], p2 = p1 + (npw > 1 ? wcnt[1] : 0), p3 = p2 + (npw > 2 ? wcnt[2] : 0);
+      const int na = p3 + (npw > 3 ? wcnt[3] : 0);
+      if (threadIdx.x == 0) {
+        iflag[3] += na;
+        n_chk += (unsigned long long)m;
+        n_rot += (unsigned long long)na;
+      }
+      if (na == 0) continue;  // nothing below reads this round's scratch
+      for (int ia = warp; ia < na; ia += nw) {
+        const int k = ia < p1 ? act[ia] : ia < p2 ? act[32 + ia - p1] : ia < p3 ? act[64 + ia - p2] : act[96 + ia - p3];
+        int p, q;
+        round_pair(r, k, n, p, q);
+        const double2 a = al[k], b = be[k];
+        auto rotate = [&](double2* xp, double2* xq, int len) {
+#pragma unroll 2
+          for (int i = lane; i < len; i += 32) {
+            const double2 u = xp[i], v = xq[i];
+            double2 up = u, vq = v;
+            fma_c<double>(up, make_double2(-a.x, -a.y), v);
+            fma_c<double>(vq, b, u);
+            xp[i] = up;
+            xq[i] = vq;
+          }
+        };
+        rotate(Zt + (size_t)p * rows, Zt + (size_t)q * rows, rows);
+        if (Vt) rotate(Vt + (size_t)p * n, Vt + (size_t)q * n, n);
+      }
+      __syncthreads();
+    }
+    const int total = iflag[3];
+    if (threadIdx.x == 0 && rot_count && sweep < kRotSweeps) atomicAdd(rot_count + sweep, (unsigned long long)total);
+    if (total) {  // multiply the factors out
+      for (int idx = threadIdx.x; idx < n * rows; idx += blockDim.x) Zt[idx] = cscale(Zt[idx], dsc[idx / rows]);
+      if (Vt)
+        for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) Vt[idx] = cscale(Vt[idx], dsc[idx / n]);
+    }
+    __syncthreads();
+    if (total == 0) {
+      result = sweep + 1;
+      break;
+    }
+  }
+  if (work && threadIdx.x == 0) {
+    atomicAdd(work, n_chk);
+    atomicAdd(work + 1, n_rot);
+  }
+  return result;
+}
+
 // FP32 one-sided stages: relative threshold jp.tol32 (at the rounding of an FP32 dot product) and
-// this absolute one, in units of the largest squared column norm
-constexpr float kOsFloor32 = 1e-13f;
+// this absolute one, in units of the largest squared column norm (its square stays an FP32 normal)
+constexpr float kOsFloor32 = 1e-18f;
+// The warm start replaces remaining columns below this fraction of the first pivot by unit vectors of that size
+constexpr float kBasisCut = 1e-6f;
 
-// Shared scratch (bytes) after the small arrays of the unsquared bond update:
-// the FP32 warm start's B32 [n][2D] and V^T32 [n][n] (complex float) when D <= 32
-// (beyond, they use the global slot), and the FP32 levels' block of at most
-// lv = min(D, kMaxLevel) columns: B32 [lv][2D], W^T32 [lv][lv] (complex float),
-// W64 [lv][lv] and Gw [lv][lv+1] (complex double).
-__host__ __device__ size_t svd_level_w64_off(int cap, int rows) {
-  return ((size_t)cap * rows * 8 + (size_t)cap * cap * 8 + 15) & ~(size_t)15;
-}
-__host__ __device__ size_t svd_f32_bytes(int D) {
-  const size_t n = (size_t)2 * D, lv = D < kMaxLevel ? (size_t)D : (size_t)kMaxLevel;
-  const size_t lvl = svd_level_w64_off((int)lv, (int)n) + lv * lv * 16 + lv * (lv + 1) * 16;
-  const size_t warm = D <= 32 ? 2 * n * n * 8 : 0;
-  return lvl > warm ? lvl : warm;
+// FP32 warm start: a unitary basis of the space of the nv indices of the vectors a_v
+// (A [nv], stride ld, `len` entries each) in which the columns of A = [a_v] are
+// nearly orthogonal: A's right singular vectors to FP32 accuracy, X [nv][nv] (row
+// v, column i), widened to FP64 (not yet unitary to FP64 rounding).
+//
+// A P = Q R by modified Gram-Schmidt with column pivoting, one warp per vector, each
+// row i of R replacing (conjugated) the vector of its pivot; then the one-sided
+// Jacobi on the columns of R^H, which after pivoting converge in about half the
+// sweeps that A itself needs (Drmac and Veselic) and whose directions are the
+// vectors sought, so that no rotation product is accumulated.  When every remaining
+// vector is below kBasisCut of the first pivot the rest of R is replaced by that
+// multiple of the identity: below FP32's resolution any completion serves, and the
+// Jacobi makes it orthogonal to the others.  nv even; len, nv <= ld <= 256.
+__device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* nrm, const JacobiParams& jp, float* rc,
+                         float* rs, float2* re, int* iflag, unsigned long long* work,
+                         unsigned long long* rot_count) {
+  constexpr int kT = kMaxDc128 * 2 / 32;  // elements of a vector per lane
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  auto wsum = [](float v) {
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+  };
+  for (int v = warp; v < nv; v += nw) {
+    float s = 0.f;
+    for (int x = lane; x < len; x += 32) {
+      const float2 a = A[(size_t)v * ld + x];
+      s = fmaf(a.x, a.x, fmaf(a.y, a.y, s));
+    }
+    s = wsum(s);
+    if (lane == 0) nrm[v] = s;
+  }
+  __syncthreads();
+  float first = 0.f;
+  for (int i = 0; i < nv; ++i) {
+    // the pivot: every warp finds it for itself (norms of used vectors are -1)
+    float best = -1.f;
+    int p = 0;
+    for (int v = lane; v < nv; v += 32) {
+      const float s = nrm[v];
+      if (s > best) {
+        best = s;
+        p = v;
+      }
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      const float ob = __shfl_xor_sync(0xffffffffu, best, off);
+      const int op = __shfl_xor_sync(0xffffffffu, p, off);
+      if (ob > best || (ob == best && op < p)) {
+        best = ob;
+        p = op;
+      }
+    }
+    if (i == 0) first = sqrtf(best);
+    if (!(best > kBasisCut * kBasisCut * first * first)) break;  // uniform: every warp has the same norms
+    const float norm = sqrtf(best), inv = 1.f / norm;
+    float2 qv[kT];
+#pragma unroll
+    for (int t = 0; t < kT; ++t) {
+      const int x = lane + 32 * t;
+      if (x < len) {
+        const float2 a = A[(size_t)p * ld + x];
+        qv[t] = make_float2(a.x * inv, a.y * inv);
+      }
+    }
+    __syncthreads();  // the pivot's vector is read: row i of R^* takes its place
+    for (int v = warp; v < nv; v += nw) {
+      float2 l = make_float2(0.f, 0.f);
+      if (v == p) {
+        l.x = norm;
+        if (lane == 0) nrm[v] = -1.f;
+      } else if (nrm[v] >= 0.f) {
+        float2* a = A + (size_t)v * ld;
+        float2 d = make_float2(0.f, 0.f), av[kT];
+#pragma unroll
+        for (int t = 0; t < kT; ++t) {
+          const int x = lane + 32 * t;
+          if (x < len) {
+            av[t] = a[x];
+            fma_conj<float>(d, qv[t], av[t]);
+          }
+        }
+        d.x = wsum(d.x);
+        d.y = wsum(d.y);
+        float s = 0.f;
+#pragma unroll
+        for (int t = 0; t < kT; ++t) {
+          const int x = lane + 32 * t;
+          if (x < len) {
+            fma_c<float>(av[t], make_float2(-d.x, -d.y), qv[t]);
+            a[x] = av[t];
+            s = fmaf(av[t].x, av[t].x, fmaf(av[t].y, av[t].y, s));
+          }
+        }
+        s = wsum(s);
+        if (lane == 0) nrm[v] = s;
+        l = make_float2(d.x, -d.y);
+      }
+      if (lane == 0) A[(size_t)p * ld + v] = l;
+    }
+    __syncthreads();
+  }
+  const float eta = first > 0.f ? kBasisCut * first : 1.f;
+  for (int v = warp; v < nv; v += nw)
+    if (nrm[v] >= 0.f)
+      for (int x = lane; x < nv; x += 32) A[(size_t)v * ld + x] = make_float2(x == v ? eta : 0.f, 0.f);
+  __syncthreads();
+  const int sw = one_sided_jacobi32(A, ld, nv, nullptr, nv, (float)jp.tol32, kOsFloor32, jp.max_sweeps32, rc, rs, re,
+                                    iflag, work, rot_count);
+  for (int v = warp; v < nv; v += nw) {
+    float s = 0.f;
+    for (int x = lane; x < nv; x += 32) {
+      const float2 a = A[(size_t)v * ld + x];
+      s = fmaf(a.x, a.x, fmaf(a.y, a.y, s));
+    }
+    s = wsum(s);
+    if (lane == 0) nrm[v] = s > 0.f ? 1.f / sqrtf(s) : 0.f;
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < nv * nv; idx += blockDim.x) {
+    const int v = idx / nv, i = idx - (idx / nv) * nv;
+    const float2 a = A[(size_t)i * ld + v];
+    X[idx] = make_double2((double)(a.x * nrm[i]), (double)(a.y * nrm[i]));
+  }
+  __syncthreads();
+  return sw;
 }
 
-// FP32 levels on the small columns of B: the columns whose squared norms lie
+// Shared memory (bytes) after the small arrays of the unsquared bond update: the
+// factors and rotations of os_sweeps, the FP32 block of the levels (B32 [lv][2D],
+// W^T32 [lv][lv], lv = min(D, kMaxLevel)), and, where the launch has room for it
+// (svd_shared_work), the matrix worked on: Z up to D = 32 (the FP32 warm start's
+// matrix before it), the warm start's alone up to D = 64; else in the global slot.
+__host__ __device__ size_t svd_rot_bytes(int D) { return (size_t)2 * D * 16 + (size_t)D * 16; }
+__host__ __device__ size_t svd_level_bytes(int D) {
+  const size_t lv = D < kMaxLevel ? (size_t)D : (size_t)kMaxLevel;
+  return (lv * 2 * D * 8 + lv * lv * 8 + 15) & ~(size_t)15;
+}
+__host__ __device__ size_t svd_shared_work(int D) {
+  return D <= 32 ? (size_t)4 * D * D * 16 : D <= 64 ? (size_t)4 * D * D * 8 : 0;
+}
+__host__ __device__ size_t svd_shared_bytes(int D, bool with_work) {
+  return svd_rot_bytes(D) + svd_level_bytes(D) + (with_work ? svd_shared_work(D) : 0);
+}
+
+// FP32 levels on the small columns of Z: the columns whose squared norms lie
 // below jp.level_ratio x the scale of the last block that held them (the
 // largest column at first) and above rounding (kNoiseRelSvd of ||M||_F^2); the
 // largest ns <= lv of them form one block.  The block is copied to FP32, scaled
 // by the power of two that brings its largest column to norm ~1; FP32 one-sided
 // Jacobi makes those columns orthogonal to FP32 accuracy relative to each
 // column; the accumulated rotation W, re-orthonormalised in FP64, rotates those
-// columns of B and of V in FP64.  Meant to run after an FP64 sweep, which has
+// columns of Z (and of V) in FP64.  Meant to run after an FP64 sweep, which has
 // removed from the small columns their components along the large ones (else
-// the block would be their contamination).  lvl: as svd_f32_bytes.
-__device__ void svd_levels(double2* Bt, int rows, double2* Vt, int n, double tr, const JacobiParams& jp,
+// the block would be their contamination).  lvl: svd_level_bytes, W64: 2 lv^2 + lv
+// complex doubles.
+__device__ void svd_levels(double2* Zt, int rows, double2* Vt, int n, double tr, const JacobiParams& jp,
                            double* alpha, double* rscale, int* mark_c, int* cand, double* scal, float2* re32,
-                           float* rc32, float* rs32, int* iflag, unsigned char* lvl, unsigned long long* sweeps_out) {
+                           float* rc32, float* rs32, int* iflag, unsigned char* lvl, double2* W64,
+                           unsigned long long* sweeps_out) {
   const int cap = (n / 2 < kMaxLevel) ? n / 2 : kMaxLevel;
-  float2* B32 = reinterpret_cast<float2*>(lvl);                                // [cap][rows]
-  float2* W32 = B32 + (size_t)cap * rows;                                      // [cap][cap], W^T
-  double2* W64 = reinterpret_cast<double2*>(lvl + svd_level_w64_off(cap, rows));  // [cap][cap]
-  double2* Gw = W64 + (size_t)cap * cap;                                       // [cap][cap+1]
+  float2* B32 = reinterpret_cast<float2*>(lvl);  // [cap][rows]
+  float2* W32 = B32 + (size_t)cap * rows;        // [cap][cap], W^T
+  double2* Gw = W64 + (size_t)cap * cap;         // [cap][cap+1]
   const double lo = kNoiseRelSvd * tr;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int level = 0; level < jp.levels; ++level) {
-    column_norms(Bt, rows, n, alpha);
+    column_norms(Zt, rows, n, alpha);
     if (level == 0) {
       if (threadIdx.x == 0) {
         double s0 = 0.0;
@@ -1062,14 +1359,14 @@ __device__ void svd_levels(double2* Bt, int rows, double2* Vt, int n, double tr,
     const double sc = ldexp(1.0, -(ex >> 1));  // the block's largest squared norm -> [1/2, 2)
     for (int idx = threadIdx.x; idx < ns * rows; idx += blockDim.x) {
       const int a = idx / rows, r = idx - (idx / rows) * rows;
-      const double2 v = Bt[(size_t)cand[a] * rows + r];
+      const double2 v = Zt[(size_t)cand[a] * rows + r];
       B32[idx] = make_float2((float)(v.x * sc), (float)(v.y * sc));
     }
     for (int idx = threadIdx.x; idx < ns * ns; idx += blockDim.x)
       W32[idx] = make_float2((idx / ns) == (idx % ns) ? 1.f : 0.f, 0.f);
     __syncthreads();
-    one_sided_jacobi<float>(B32, rows, W32, ns, (float)jp.tol32, kOsFloor32, jp.max_sweeps32, rc32, rs32, re32,
-                            iflag, sweeps_out + 6, nullptr);
+    one_sided_jacobi32(B32, rows, rows, W32, ns, (float)jp.tol32, kOsFloor32, jp.max_sweeps32, rc32, rs32, re32,
+                       iflag, sweeps_out + 6, nullptr);
     for (int idx = threadIdx.x; idx < ns * ns; idx += blockDim.x) {
       const int a = idx / ns, b = idx - (idx / ns) * ns;
       const float2 v = W32[(size_t)b * ns + a];
@@ -1077,9 +1374,9 @@ __device__ void svd_levels(double2* Bt, int rows, double2* Vt, int n, double tr,
     }
     __syncthreads();
     orthonormalise<false>(W64, ns, Gw, ns + 1, alpha, scal);
-    // rows of B (r < rows) and of V (x < n): new column cand[b] = sum_a old column cand[a] W[a][b]
-    for (int rr = warp; rr < rows + n; rr += nw) {
-      double2* base = rr < rows ? Bt + rr : Vt + (rr - rows);
+    // rows of Z (r < rows) and of V (x < n): new column cand[b] = sum_a old column cand[a] W[a][b]
+    for (int rr = warp; rr < rows + (Vt ? n : 0); rr += nw) {
+      double2* base = rr < rows ? Zt + rr : Vt + (rr - rows);
       const int ld = rr < rows ? rows : n;
       double2 out = make_double2(0.0, 0.0);
       if (lane < ns)
@@ -1093,7 +1390,7 @@ __device__ void svd_levels(double2* Bt, int rows, double2* Vt, int n, double tr,
     if (threadIdx.x == 0) {
       atomicAdd(sweeps_out + 2, 1ull);
       const unsigned long long nsl = (unsigned long long)ns;
-      atomicAdd(sweeps_out + 3, (unsigned long long)(rows + n) * nsl * nsl + 4ull * nsl * nsl * nsl / 3ull);
+      atomicAdd(sweeps_out + 3, (unsigned long long)(rows + (Vt ? n : 0)) * nsl * nsl + 4ull * nsl * nsl * nsl / 3ull);
     }
   }
 }
@@ -1102,18 +1399,26 @@ __device__ void svd_levels(double2* Bt, int rows, double2* Vt, int n, double tr,
 // end a (FP64 sums in gsum, or this bond's partials) and end b, the right
 // singular vectors V (Vm [n][n], row x, column j) and squared singular values
 // (ev[j]) of the gated two-site matrix.  Returns false when M vanishes or is not
-// finite (the bond is then left unchanged by the caller).  lvl: the level
-// scratch in shared memory.
+// finite (the bond is then left unchanged by the caller).  lvl: shared memory of
+// svd_shared_bytes(D, shared_work).
+//
+// Two forms.  A square core (n = 2D, every bond between ends of degree >= 2): with
+// U0 the left singular vectors of M from FP32, unitary to FP64 rounding, the columns
+// of Z = M^H U0 are nearly orthogonal, and the sweeps on Z alone end with columns
+// s_j v_j: the right singular vectors without accumulating a rotation product (half
+// the rotation work).  Columns at rounding (|z|^2 <= kNoiseRelSvd ||M||^2) are
+// dropped: their direction is noise.  With `full` (the reverse mode needs a complete
+// unitary V, in the same gauge forward and recomputed) or n < 2D (an end of degree 1): B = M V0 with V0 the right singular
+// vectors from FP32, V rotated alongside.
 template <bool kCG>
 __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ partials, const double2* gsum,
                                const double2* gamma, const double* lam, double th_b, int D, const JacobiParams& jp,
-                               unsigned char* big, double* lamo, double* ev, double* rc, double* rs, double2* re,
-                               double* scal, float2* re32, float* rc32, float* rs32, int* order, int* rp, int* rq,
-                               int* iflag,
-                               unsigned char* lvl, unsigned long long* sweeps_out, unsigned long long* cycles,
-                               int* flags, long long& t_prev, double2** Vm_out) {
+                               unsigned char* big, double* lamo, double* ev, double* rc, double2* re, double* scal,
+                               float2* re32, float* rc32, float* rs32, int* order, int* rp, int* iflag,
+                               unsigned char* lvl, bool shared_work, bool full, unsigned long long* sweeps_out,
+                               unsigned long long* cycles, int* flags, long long& t_prev, double2** Vm_out) {
   const SideDesc& sb = bd.b;
-  const int n = 2 * sb.rows, rows = 2 * D, D2 = D * D, ldr = n + 1;
+  const int n = 2 * sb.rows, rows = 2 * D, D2 = D * D;
   const SvdLayout L(D);
   double2* Mt = reinterpret_cast<double2*>(big + L.off_Mt);
   double2* RB = reinterpret_cast<double2*>(big + L.off_RB);
@@ -1123,6 +1428,11 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
   double2* Rr = Xs + (size_t)2 * D * (D + 1);  // [2][D][D]
   double2* F = Vx;                         // [n][D]
   int* mask = reinterpret_cast<int*>(Mt);  // [2][D] while the factors run
+  double* dsc = reinterpret_cast<double*>(lvl);
+  double* dinv = dsc + rows;
+  double2* be = reinterpret_cast<double2*>(dinv + rows);
+  unsigned char* work = lvl + svd_rot_bytes(D) + svd_level_bytes(D);
+  lvl += svd_rot_bytes(D);
   auto mark = [&](int phase) {
     if (threadIdx.x == 0) {
       const long long t = clock64();
@@ -1151,81 +1461,81 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
   // M^T[x][s D + j] = g(s, t_x) sum_k R_s[j][k] lam_k F[x][k], g(s, t) = (1 + i sign) / sqrt 2 for
   // s = t, (1 - i sign) / sqrt 2 otherwise (sign = gate_sign: exp(+-i pi/4 z_s z_t))
   const double r2 = 0.70710678118654752440;
+  for (int idx = threadIdx.x; idx < n * D; idx += blockDim.x) F[idx] = cscale(F[idx], lamo[idx % D]);
+  __syncthreads();
   for (int idx = threadIdx.x; idx < n * rows; idx += blockDim.x) {
     const int x = idx / rows, r = idx - (idx / rows) * rows, sidx = r / D, j = r - (r / D) * D;
     const double2* Rj = Rr + (size_t)sidx * D2 + (size_t)j * D;
     const double2* Fx = F + (size_t)x * D;
     double2 acc = make_double2(0.0, 0.0);
-    for (int k = 0; k < D; ++k) fma_c<double>(acc, Rj[k], cscale(Fx[k], lamo[k]));
+    for (int k = 0; k < D; ++k) fma_c<double>(acc, Rj[k], Fx[k]);
     const double gi = ((sidx == (x & 1)) == (jp.gate_sign > 0)) ? r2 : -r2;
-    Mt[idx] = make_double2(r2 * acc.x - gi * acc.y, r2 * acc.y + gi * acc.x);
+    Mt[idx] = make_double2(fma(r2, acc.x, -__dmul_rn(gi, acc.y)), fma(r2, acc.y, __dmul_rn(gi, acc.x)));
   }
   __syncthreads();
-  // ||M||_F^2
-  {
-    const int lane = threadIdx.x & 31;
+  // ||M||_F^2, summed in an order that does not depend on the CTA's size
+  column_norms(Mt, rows, n, ev);
+  if (threadIdx.x < 32) {
     double acc = 0.0;
-    for (int idx = threadIdx.x; idx < n * rows; idx += blockDim.x)
-      acc = fma(Mt[idx].x, Mt[idx].x, fma(Mt[idx].y, Mt[idx].y, acc));
+    for (int x = threadIdx.x; x < n; x += 32) acc += ev[x];
     acc = warp_sum(acc);
-    if (threadIdx.x == 0) scal[0] = 0.0;
-    __syncthreads();
-    if (lane == 0) atomicAdd(scal, acc);
-    __syncthreads();
+    if (threadIdx.x == 0) scal[0] = acc;
   }
+  __syncthreads();
   const double trace = scal[0];
   if (!(trace > 0.0) || !isfinite(trace)) return false;
   mark(0);
-  // FP32 one-sided warm start on M scaled by the power of two that brings ||M||_F
-  // to ~1: its rotations leave a column of Schmidt value s_j at a cosine of
-  // ~1e-7 s_max / s_j against the others (the eigenvectors of the squared M^H M
-  // in FP32 would leave ~1e-7 (s_max / s_j)^3).  B32 [n][2D] and V^T32 [n][n] in
-  // shared memory up to D = 32, else over the free rho and scratch regions.
-  float2* B32 = D <= 32 ? reinterpret_cast<float2*>(lvl) : reinterpret_cast<float2*>(RB);
-  float2* Vt32 = D <= 32 ? B32 + (size_t)n * rows : reinterpret_cast<float2*>(Xs);
+  // FP32 warm start on M scaled by the power of two that brings ||M||_F to ~1
+  const bool left = !full && n == rows;
+  const int nv = left ? rows : n;
+  float2* A32 = shared_work ? reinterpret_cast<float2*>(work) : reinterpret_cast<float2*>(RB);
   {
     int ex;
     frexp(trace, &ex);
     const double sc = ldexp(1.0, -(ex >> 1));
-    for (int idx = threadIdx.x; idx < n * rows; idx += blockDim.x)
-      B32[idx] = make_float2((float)(Mt[idx].x * sc), (float)(Mt[idx].y * sc));
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x)
-      Vt32[idx] = make_float2((idx / n) == (idx % n) ? 1.f : 0.f, 0.f);
+    for (int idx = threadIdx.x; idx < n * rows; idx += blockDim.x) {
+      const float2 v = make_float2((float)(Mt[idx].x * sc), (float)(Mt[idx].y * sc));
+      const int x = idx / rows, r = idx - (idx / rows) * rows;
+      if (left) A32[(size_t)r * rows + x] = make_float2(v.x, -v.y);  // column r of M^H
+      else A32[idx] = v;                                             // column x of M
+    }
   }
   __syncthreads();
-  const int sw32 = one_sided_jacobi<float>(B32, rows, Vt32, n, (float)jp.tol32, kOsFloor32, jp.max_sweeps32, rc32,
-                                           rs32, re32, iflag, sweeps_out + 6, cycles ? cycles + kPhases : nullptr);
-  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-    const int x = idx / n, j = idx - (idx / n) * n;
-    const float2 v = Vt32[(size_t)j * n + x];
-    Vx[idx] = make_double2((double)v.x, (double)v.y);
-  }
-  __syncthreads();
+  const int sw32 = svd_basis(A32, nv, left ? n : rows, rows, Vx, reinterpret_cast<float*>(ev), jp, rc32, rs32, re32,
+                             iflag, sweeps_out + 6, cycles ? cycles + kPhases : nullptr);
   mark(1);
   {
-    // The series of `orthonormalise` is exact to O(|E|^3), below 1e-12 for the
-    // |E| ~ 2e-5 that the FP32 warm start leaves at n = 64 (~400 rotations per
-    // column; measured <Z> parity 3e-14).  A wide solve drifts further (n = 256:
-    // ~2500 rotations per column leave |E| ~ 1e-4), so from 1e-4 on a second
-    // pass, which starts from ~|E|^3, finishes the job; a basis beyond the
-    // series' range is flagged.
-    const double emax = orthonormalise<false>(Vx, n, Xs, ldr, ev, scal);
-    const double emax2 = emax > 1e-4 ? orthonormalise<false>(Vx, n, Xs, ldr, ev, scal) : 0.0;
+    // Its columns are orthogonal to |E| ~ 1e-6; the series of `orthonormalise` is exact to
+    // O(|E|^3), and its FP32 products to ~n |E|^2 1e-7.  A basis further off takes a second
+    // pass, which starts from ~|E|^3; one beyond the series' range is flagged.
+    const double emax = orthonormalise<true>(Vx, nv, Xs, nv + 1, ev, scal);
+    const double emax2 = emax > 4e-6 ? orthonormalise<true>(Vx, nv, Xs, nv + 1, ev, scal) : 0.0;
     if (threadIdx.x == 0 && (!(emax < 1e-2) || !(emax2 < 1e-8))) atomicOr(flags, 1);
   }
   mark(2);
-  // B = M V0 (Bt[j][r] = sum_x V0[x][j] M[r][x]) and V^T, over the free regions
-  double2* Bt = RB;
-  double2* Vt = Xs;
-  for (int idx = threadIdx.x; idx < n * rows; idx += blockDim.x) {
-    const int j = idx / rows, r = idx - (idx / rows) * rows;
-    double2 acc = make_double2(0.0, 0.0);
-    for (int x = 0; x < n; ++x) fma_c<double>(acc, Vx[(size_t)x * n + j], Mt[(size_t)x * rows + r]);
-    Bt[idx] = acc;
-  }
-  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-    const int j = idx / n, x = idx - (idx / n) * n;
-    Vt[idx] = Vx[(size_t)x * n + j];
+  // Z = M^H U0 (columns of length n), or B = M V0 (length 2D) and V^T, over the free regions
+  double2* Zt = left && shared_work && D <= 32 ? reinterpret_cast<double2*>(work) : RB;
+  double2* Vt = left ? nullptr : Xs;
+  const int zr = left ? n : rows;
+  if (left) {
+    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+      const int x = idx / n, j = idx - (idx / n) * n;
+      double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 4
+      for (int r = 0; r < rows; ++r) fma_conj<double>(acc, Mt[(size_t)x * rows + r], Vx[(size_t)r * n + j]);
+      Zt[(size_t)j * n + x] = acc;
+    }
+  } else {
+    for (int idx = threadIdx.x; idx < n * rows; idx += blockDim.x) {
+      const int j = idx / rows, r = idx - (idx / rows) * rows;
+      double2 acc = make_double2(0.0, 0.0);
+      for (int x = 0; x < n; ++x) fma_c<double>(acc, Vx[(size_t)x * n + j], Mt[(size_t)x * rows + r]);
+      Zt[idx] = acc;
+    }
+    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+      const int j = idx / n, x = idx - (idx / n) * n;
+      Vt[idx] = Vx[(size_t)x * n + j];
+    }
   }
   __syncthreads();
   // One FP64 sweep first: it converges the pairs of large columns and removes
@@ -1234,26 +1544,34 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
   // size).  Only then are the small columns a clean block for the FP32 levels,
   // whose rotations leave the last sweeps little to do.
   unsigned long long* rot = cycles ? cycles + kPhases + kRotSweeps : nullptr;
-  const int sw1 = one_sided_jacobi(Bt, rows, Vt, n, jp.tol, jp.floor_rel * trace, 1, rc, rs, re, iflag,
-                                   sweeps_out + 4, rot);
+  const int sw1 = os_sweeps(Zt, zr, Vt, n, jp.tol, jp.floor_rel * trace, trace, 1, ev, dsc, dinv, re, be, iflag,
+                            sweeps_out + 4, rot);
   mark(4);
-  // level marks in rp/rq (n ints, free until a level's Jacobi), candidates in order
-  svd_levels(Bt, rows, Vt, n, trace, jp, ev, rc, rp, order, scal, re32, rc32, rs32, iflag, lvl, sweeps_out);
+  // level marks in rp (n ints, free until a level's Jacobi), candidates in order; M is not needed any more
+  svd_levels(Zt, zr, Vt, n, trace, jp, ev, rc, rp, order, scal, re32, rc32, rs32, iflag, lvl, Mt, sweeps_out);
   mark(3);
   const int sweeps = sw1 == 1 ? 1
-                              : 1 + one_sided_jacobi(Bt, rows, Vt, n, jp.tol, jp.floor_rel * trace, jp.max_sweeps - 1,
-                                                     rc, rs, re, iflag, sweeps_out + 4, rot ? rot + 1 : nullptr);
+                              : 1 + os_sweeps(Zt, zr, Vt, n, jp.tol, jp.floor_rel * trace, trace, jp.max_sweeps - 1,
+                                              ev, dsc, dinv, re, be, iflag, sweeps_out + 4, rot ? rot + 1 : nullptr);
   mark(4);
   if (threadIdx.x == 0) {
     if (sweeps > jp.max_sweeps) atomicOr(flags, 1);
     atomicAdd(sweeps_out, (unsigned long long)(sweeps > jp.max_sweeps ? jp.max_sweeps : sweeps));
     atomicAdd(sweeps_out + 1, (unsigned long long)(sw32 > jp.max_sweeps32 ? jp.max_sweeps32 : sw32));
   }
-  // squared singular values (the column norms of B) and V back in row-major order
-  column_norms(Bt, rows, n, ev);
+  // squared singular values (the column norms) and V in row-major order
+  column_norms(Zt, zr, n, ev);
+  if (left) {
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+      const bool noise = !(ev[j] > kNoiseRelSvd * trace);
+      dsc[j] = noise ? 0.0 : 1.0 / sqrt(ev[j]);
+      if (noise) ev[j] = 0.0;
+    }
+    __syncthreads();
+  }
   for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
     const int x = idx / n, j = idx - (idx / n) * n;
-    Vx[idx] = Vt[(size_t)j * n + x];
+    Vx[idx] = left ? cscale(Zt[(size_t)j * n + x], dsc[j]) : Vt[(size_t)j * n + x];
   }
   __syncthreads();
   *Vm_out = Vx;
@@ -1320,9 +1638,12 @@ __device__ void bond_body(const BondDesc bd, const V2<T>* __restrict__ partials,
   if constexpr (sizeof(T) == 8) {
     // complex128: the unsquared SVD of the bond core, in the CTA's global slot
     // (every launcher passes one for this dtype)
-    if (!big || !bond_front_svd<kCG>(bd, partials, gsum, gamma, lam, th_b, D, jp, big, lamo, ev, rc, rs, re, scal,
-                                     re32, rc32, rs32, order, rp, rq, iflag, smallp + L.small, sweeps_out, cycles,
-                                     flags, t_prev, &Vm)) {
+    uint32_t dyn;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+    const bool shared_work = svd_shared_work(D) > 0 && dyn >= BondSmem(D, 2 * D).small + svd_shared_bytes(D, true);
+    if (!big || !bond_front_svd<kCG>(bd, partials, gsum, gamma, lam, th_b, D, jp, big, lamo, ev, rc, re, scal, re32,
+                                     rc32, rs32, order, rp, iflag, smallp + L.small, shared_work, jp.full_basis != 0,
+                                     sweeps_out, cycles, flags, t_prev, &Vm)) {
       bond_fail<T, kCG>(bd, Y, theta_a, pending, flags, D);
       return;
     }
@@ -1884,7 +2205,7 @@ struct StepSlot {
 
 BondFootprint step_footprint(int D, size_t elt, bool tc) {
   const BondSmem L(D, 2 * D);
-  size_t sm = L.small + bond_f32(D, elt);
+  size_t sm = L.small + bond_f32(D, elt, D < kOzMinD);  // complex128: fused below kOzMinD only
   if (tc) {
     if (tc_gram_smem(D) > sm) sm = tc_gram_smem(D);
     if (tc_update_smem(D) > sm) sm = tc_update_smem(D);
@@ -2325,7 +2646,8 @@ cudaError_t Launch<T>::bond(const BondDesc* bonds, int n_bonds, const void* part
                             unsigned int* queue, int n_ctas, void* scratch, int per_sm) {
   if (n_bonds == 0) return cudaSuccess;
   const bool shared = per_sm > 1;
-  const BondFootprint fp = shared ? bond_footprint_global(D, sizeof(V2<T>)) : bond_footprint(D, kBondSmemMax, sizeof(V2<T>));
+  const BondFootprint fp = shared ? bond_footprint_global(D, sizeof(V2<T>), bond_share_smem(per_sm))
+                                  : bond_footprint(D, kBondSmemMax, sizeof(V2<T>));
   if (fp.slot && !scratch) return cudaErrorInvalidValue;
   if (shared && (!queue || (per_sm != 2 && per_sm != 4) || fp.smem > bond_share_smem(per_sm)))
     return cudaErrorInvalidValue;
