@@ -39,6 +39,24 @@ __device__ __forceinline__ void kick2(T c, T s, V2<T> g0, V2<T> g1, V2<T>& a0, V
   a1 = mk<T>(s * g0.y + c * g1.x, -s * g0.x + c * g1.y);
 }
 
+// cos and sin of half the kick th, formed by the CTA's first warp and read by all (every
+// FP64 instruction of the two calls holds a warp's SMSP for 64 cycles; in all eight warps
+// of a tile they cost ~13 000 cycles of the SM).  Contains barriers.
+template <typename T>
+__device__ __forceinline__ V2<T> kick_factors(double th) {
+  __shared__ double cs[2];
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double c = cos(0.5 * th), s = sin(0.5 * th);
+    if (threadIdx.x == 0) {
+      cs[0] = c;
+      cs[1] = s;
+    }
+  }
+  __syncthreads();
+  return mk<T>((T)cs[0], (T)cs[1]);
+}
+
 struct RowPos {
   int r1, r2;
 };
@@ -103,7 +121,8 @@ __global__ void __launch_bounds__(kThreads)
   const SideDesc sa = bonds[t.bond].a;
   const int ld = 2 * D + 1;
   const double th = pending[sa.site];
-  const T c = (T)cos(0.5 * th), s = (T)sin(0.5 * th);
+  const V2<T> cs = kick_factors<T>(th);
+  const T c = cs.x, s = cs.y;
   const int nel = t.nrows * D;
   for (int idx = threadIdx.x; idx < nel; idx += blockDim.x) {
     int r, k;
@@ -235,13 +254,11 @@ __device__ __forceinline__ void upper_index(int idx, int n, int& i, int& j) {
 // that are exact to O(|E|^3) ~ 1e-18, with only parallel products:
 //   X1 = P(E), X = P(E - X1^dagger X1), R = I + X, R^-1 = I - X + X^2,
 // where P keeps the strict upper triangle and half the diagonal.  Q = V R^-1
-// is formed row by row in place (one warp per row).  G holds E and X in its
-// upper triangle and X1^dagger X1, X^2 in its strict lower triangle (row
-// stride ldg); dg[n] holds their diagonals.  Returns max |E_ij|.
+// is formed row by row in place (one warp per row).  G holds E and then X^2 - X in
+// its upper triangle (row stride ldg).  Returns max |E_ij|.
 //
-// kF32Products (the complex64 path, whose bond matrix carries FP32 rounding):
-// the two products of E-sized factors, X1^dagger X1 and X^2, run in FP32 on
-// FP32 copies of X1 and X.  Their entries are O(n |E|^2) ~ 1e-10, so FP32's
+// The two products of E-sized factors, X1^dagger X1 and X^2, run in FP32 on FP32
+// copies of X1 and X.  Their entries are O(n |E|^2) ~ 1e-10, so FP32's
 // relative 1e-7 leaves absolute errors at or below the FP64 rounding of E itself
 // at the |E| ~ 1e-6 of a 64-wide FP32 solve; E = V^dagger V - I and Q = V R^-1
 // stay FP64.  The FP32 copy of upper entry (i, j) sits in the otherwise unused
@@ -252,108 +269,49 @@ __device__ __forceinline__ float2* tri32(double2* G, int ldg, int n, int i, int 
   return reinterpret_cast<float2*>(i < j ? G + j * ldg + i : G + i * ldg + n);
 }
 
-template <bool kF32Products>
-__device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double* dg, double* scal) {
-  if constexpr (kF32Products) {
-    // E = V^dagger V - I (upper triangle, FP64) and the FP32 copy of X1 = P(E)
-    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-      int i, j;
-      upper_index(idx, n, i, j);
-      double2 acc = make_double2(i == j ? -1.0 : 0.0, 0.0);
-      for (int r = 0; r < n; ++r) fma_conj<double>(acc, V[r * n + i], V[r * n + j]);
-      if (i == j) acc.y = 0.0;
-      G[i * ldg + j] = acc;
-      tri32(G, ldg, n, i, j)[0] =
-          i == j ? make_float2((float)(0.5 * acc.x), 0.f) : make_float2((float)acc.x, (float)acc.y);
-    }
-    if (threadIdx.x == 0) scal[6] = 0.0;
-    __syncthreads();
-    // K = X1^dagger X1 (FP32, K_ij = sum_{k <= i} conj(X1_ki) X1_kj), X = P(E - K) in FP64
-    // over E, and its FP32 copy; record max |E|
-    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-      int i, j;
-      upper_index(idx, n, i, j);
-      float2 k32 = make_float2(0.f, 0.f);
-      for (int k = 0; k <= i; ++k) fma_conj<float>(k32, tri32(G, ldg, n, k, i)[0], tri32(G, ldg, n, k, j)[0]);
-      const double2 e = G[i * ldg + j];
-      const double ae = fabs(e.x) + fabs(e.y);
-      if (ae > scal[6]) atomicMax(reinterpret_cast<unsigned long long*>(scal + 6), __double_as_longlong(ae));
-      const double2 x = i == j ? make_double2(0.5 * (e.x - (double)k32.x), 0.0)
-                               : make_double2(e.x - (double)k32.x, e.y - (double)k32.y);
-      G[i * ldg + j] = x;
-      tri32(G, ldg, n, i, j)[1] = make_float2((float)x.x, (float)x.y);
-    }
-    __syncthreads();
-    // M = X^2 - X in the upper triangle (X^2 upper triangular, FP32: (X^2)_ij = sum_{i<=k<=j} X_ik X_kj)
-    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-      int i, j;
-      upper_index(idx, n, i, j);
-      float2 s32 = make_float2(0.f, 0.f);
-      for (int k = i; k <= j; ++k) fma_c<float>(s32, tri32(G, ldg, n, i, k)[1], tri32(G, ldg, n, k, j)[1]);
-      const double2 x = G[i * ldg + j];
-      G[i * ldg + j] = i == j ? make_double2((double)s32.x - x.x, 0.0)
-                              : make_double2((double)s32.x - x.x, (double)s32.y - x.y);
-    }
-    __syncthreads();
-  } else {
-    // E = V^dagger V - I (upper triangle)
-    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-      int i, j;
-      upper_index(idx, n, i, j);
-      double2 acc = make_double2(i == j ? -1.0 : 0.0, 0.0);
-      for (int r = 0; r < n; ++r) fma_conj<double>(acc, V[r * n + i], V[r * n + j]);
-      if (i == j) acc.y = 0.0;
-      G[i * ldg + j] = acc;
-    }
-    if (threadIdx.x == 0) scal[6] = 0.0;
-    __syncthreads();
-    // K = X1^dagger X1 with X1 = P(E): K_ij = sum_{k <= i} conj(X1_ki) X1_kj  (i <= j)
-    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-      int i, j;
-      upper_index(idx, n, i, j);
-      double2 acc = make_double2(0.0, 0.0);
-      for (int k = 0; k <= i; ++k) {
-        double2 xki = G[k * ldg + i], xkj = G[k * ldg + j];
-        if (k == i) xki = cscale(xki, 0.5);
-        if (k == j) xkj = cscale(xkj, 0.5);
-        fma_conj<double>(acc, xki, xkj);
-      }
-      if (i == j) dg[i] = acc.x;
-      else G[j * ldg + i] = acc;
-    }
-    __syncthreads();
-    // X = P(E - K) in the upper triangle; record max |E|
-    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-      int i, j;
-      upper_index(idx, n, i, j);
-      const double2 e = G[i * ldg + j];
-      const double ae = fabs(e.x) + fabs(e.y);
-      if (ae > scal[6]) atomicMax(reinterpret_cast<unsigned long long*>(scal + 6), __double_as_longlong(ae));
-      if (i == j) G[i * ldg + i] = make_double2(0.5 * (e.x - dg[i]), 0.0);
-      else G[i * ldg + j] = csub(e, G[j * ldg + i]);
-    }
-    __syncthreads();
-    // X^2 (upper triangular) into the strict lower triangle and dg
-    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-      int i, j;
-      upper_index(idx, n, i, j);
-      double2 acc = make_double2(0.0, 0.0);
-      for (int k = i; k <= j; ++k) fma_c<double>(acc, G[i * ldg + k], G[k * ldg + j]);
-      if (i == j) dg[i] = acc.x;
-      else G[j * ldg + i] = acc;
-    }
-    __syncthreads();
-    // M = X^2 - X in the upper triangle
-    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-      int i, j;
-      upper_index(idx, n, i, j);
-      if (i == j) G[i * ldg + i] = make_double2(dg[i] - G[i * ldg + i].x, 0.0);
-      else G[i * ldg + j] = csub(G[j * ldg + i], G[i * ldg + j]);
-    }
-    __syncthreads();
+__device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double* scal) {
+  // E = V^dagger V - I (upper triangle, FP64) and the FP32 copy of X1 = P(E)
+  for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
+    int i, j;
+    upper_index(idx, n, i, j);
+    double2 acc = make_double2(i == j ? -1.0 : 0.0, 0.0);
+    for (int r = 0; r < n; ++r) fma_conj<double>(acc, V[r * n + i], V[r * n + j]);
+    if (i == j) acc.y = 0.0;
+    G[i * ldg + j] = acc;
+    tri32(G, ldg, n, i, j)[0] =
+        i == j ? make_float2((float)(0.5 * acc.x), 0.f) : make_float2((float)acc.x, (float)acc.y);
   }
+  if (threadIdx.x == 0) scal[6] = 0.0;
+  __syncthreads();
+  // K = X1^dagger X1 (FP32, K_ij = sum_{k <= i} conj(X1_ki) X1_kj), X = P(E - K) in FP64
+  // over E, and its FP32 copy; record max |E|
+  for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
+    int i, j;
+    upper_index(idx, n, i, j);
+    float2 k32 = make_float2(0.f, 0.f);
+    for (int k = 0; k <= i; ++k) fma_conj<float>(k32, tri32(G, ldg, n, k, i)[0], tri32(G, ldg, n, k, j)[0]);
+    const double2 e = G[i * ldg + j];
+    const double ae = fabs(e.x) + fabs(e.y);
+    if (ae > scal[6]) atomicMax(reinterpret_cast<unsigned long long*>(scal + 6), __double_as_longlong(ae));
+    const double2 x = i == j ? make_double2(0.5 * (e.x - (double)k32.x), 0.0)
+                             : make_double2(e.x - (double)k32.x, e.y - (double)k32.y);
+    G[i * ldg + j] = x;
+    tri32(G, ldg, n, i, j)[1] = make_float2((float)x.x, (float)x.y);
+  }
+  __syncthreads();
+  // M = X^2 - X in the upper triangle (X^2 upper triangular, FP32: (X^2)_ij = sum_{i<=k<=j} X_ik X_kj)
+  for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
+    int i, j;
+    upper_index(idx, n, i, j);
+    float2 s32 = make_float2(0.f, 0.f);
+    for (int k = i; k <= j; ++k) fma_c<float>(s32, tri32(G, ldg, n, i, k)[1], tri32(G, ldg, n, k, j)[1]);
+    const double2 x = G[i * ldg + j];
+    G[i * ldg + j] = i == j ? make_double2((double)s32.x - x.x, 0.0)
+                            : make_double2((double)s32.x - x.x, (double)s32.y - x.y);
+  }
+  __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (kF32Products && n <= 128) {
+  if (n <= 128) {
     // Q[r][j] = V[r][j] + sum_{i <= j} V[r][i] M[i][j], one warp per row, in place: lane l
     // forms the column pairs (j, n-1-j) for j = l and l + 32 (below n/2) in one pass of n + 1
     // products each (i = t for column j while t <= j, then i = t - j - 1 for column n-1-j),
@@ -412,7 +370,9 @@ __device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double*
     }
   }
   __syncthreads();
-  return scal[6];
+  const double emax = scal[6];
+  __syncthreads();  // every thread has it before a next call resets it
+  return emax;
 }
 
 // FP32 warm start of a Hermitian eigenproblem: the FP64 n x n matrix RHO (row
@@ -422,8 +382,8 @@ __device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double*
 // (f32s given: the n x n matrices are in global memory) packed in shared memory
 // at f32s.  Returns the FP32 sweeps.
 __device__ int fp32_warm_start(const double2* RHO, double2* Vm, double2* X, int n, double trace,
-                               const JacobiParams& jp, float2* re32, double* ev, double* scal, float* rc32,
-                               float* rs32, int* rp, int* rq, int* iflag, unsigned long long* sweeps_out,
+                               const JacobiParams& jp, float2* re32, double* scal, float* rc32, float* rs32, int* rp,
+                               int* rq, int* iflag, unsigned long long* sweeps_out,
                                unsigned long long* cycles, int* flags, long long& t_prev, float2* f32s) {
   const int ldr = n + 1;
   const bool packed = f32s != nullptr;
@@ -469,7 +429,7 @@ __device__ int fp32_warm_start(const double2* RHO, double2* Vm, double2* X, int 
   }
   __syncthreads();
   mark(1);
-  const double emax = orthonormalise<true>(Vm, n, X, ldr, ev, scal);
+  const double emax = orthonormalise(Vm, n, X, ldr, scal);
   if (threadIdx.x == 0 && !(emax < 1e-4)) atomicOr(flags, 1);  // FP32 basis too far from unitary
   mark(2);
   return sw32;
@@ -496,7 +456,7 @@ __device__ int eig_mixed(double2* RHO, double2* Vm, double2* X, int n, int D, do
       t_prev = t;
     }
   };
-  const int sw32 = fp32_warm_start(RHO, Vm, X, n, trace, jp, re32, ev, scal, rc32, rs32, rp, rq, iflag, sweeps_out,
+  const int sw32 = fp32_warm_start(RHO, Vm, X, n, trace, jp, re32, scal, rc32, rs32, rp, rq, iflag, sweeps_out,
                                    cycles, flags, t_prev, f32s);
   // rho' = V^dagger rho V: W = rho V into X, then the upper triangle of V^dagger W into RHO
   for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
@@ -594,7 +554,7 @@ __device__ int eig_mixed(double2* RHO, double2* Vm, double2* X, int n, int D, do
         W64[idx] = make_double2((double)v.x, (double)v.y);
       }
       __syncthreads();
-      orthonormalise<true>(W64, ns, Gw, ldb, dcur, scal);
+      orthonormalise(W64, ns, Gw, ldb, scal);
       // rows of V and rho': X[r][cand] <- X[r][cand] W, then the columns of rho':
       // rho'[cand][c] <- W^dagger rho'[cand][c]; a row (column) per segment of seg >= ns
       // lanes, 32 / seg of them per warp, so that a small level does not leave most
@@ -671,10 +631,11 @@ __device__ void bond_fail(const BondDesc& bd, V2<T>* Y, double* theta_a, double*
 }
 
 // F[(row, t)][k]: kicked Gamma_b with the lambda of its other legs, in the
-// storage precision T.
+// storage precision T; kcs: cos and sin of half the kick (formed by one warp: every
+// FP64 instruction of the two calls costs a warp 64 cycles of its SMSP).
 template <typename T, bool kCG>
-__device__ void load_F(const SideDesc& sb, const V2<T>* gamma, const double* lam, double th, V2<T>* F, int D) {
-  const T c = (T)cos(0.5 * th), s = (T)sin(0.5 * th);
+__device__ void load_F(const SideDesc& sb, const V2<T>* gamma, const double* lam, const double* kcs, V2<T>* F, int D) {
+  const T c = (T)kcs[0], s = (T)kcs[1];
   for (int idx = threadIdx.x; idx < sb.rows * D; idx += blockDim.x) {
     const int rj = idx / D, k = idx - (idx / D) * D;
     const RowPos p = row_pos(sb, rj);
@@ -1010,9 +971,10 @@ __device__ int os_sweeps(double2* Zt, int rows, double2* Vt, int n, double tol, 
   int* act = iflag + 8;     // [4 warps][32] active pairs of the round
   int* wcnt = iflag + 136;  // active pairs per warp
   const int npw = (m + 31) >> 5;
-  // lanes per pair: the pairs of a round over four warps, one per SMSP, where n allows
+  // lanes per pair: the pairs of a round over four warps, one per SMSP, where n allows, and
+  // at least two entries per lane
   int lpp = 32;
-  while (lpp > 4 && lpp * m > 128) lpp >>= 1;
+  while (lpp > 4 && (lpp * m > 128 || 2 * lpp > rows)) lpp >>= 1;
   const int sub = lane & (lpp - 1), ppw = 32 / lpp, grp = lane / lpp;
   const double tol2 = tol * tol, noise = kNoiseRelSvd * trace, floor2 = floor_abs * floor_abs;
   const double over = 1e-32 * trace;
@@ -1373,7 +1335,7 @@ __device__ void svd_levels(double2* Zt, int rows, double2* Vt, int n, double tr,
       W64[idx] = make_double2((double)v.x, (double)v.y);
     }
     __syncthreads();
-    orthonormalise<false>(W64, ns, Gw, ns + 1, alpha, scal);
+    orthonormalise(W64, ns, Gw, ns + 1, scal);
     // rows of Z (r < rows) and of V (x < n): new column cand[b] = sum_a old column cand[a] W[a][b]
     for (int rr = warp; rr < rows + (Vt ? n : 0); rr += nw) {
       double2* base = rr < rows ? Zt + rr : Vt + (rr - rows);
@@ -1412,7 +1374,7 @@ __device__ void svd_levels(double2* Zt, int rows, double2* Vt, int n, double tr,
 // vectors from FP32, V rotated alongside.
 template <bool kCG>
 __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ partials, const double2* gsum,
-                               const double2* gamma, const double* lam, double th_b, int D, const JacobiParams& jp,
+                               const double2* gamma, const double* lam, const double* kcs, int D, const JacobiParams& jp,
                                unsigned char* big, double* lamo, double* ev, double* rc, double2* re, double* scal,
                                float2* re32, float* rc32, float* rs32, int* order, int* rp, int* iflag,
                                unsigned char* lvl, bool shared_work, bool full, unsigned long long* sweeps_out,
@@ -1455,7 +1417,8 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
     const int sidx = o / D2, kl = o - sidx * D2, k = kl / D, l = kl - (kl / D) * D;
     Cw[(size_t)sidx * D * (D + 1) + k * (D + 1) + l] = acc;
   }
-  load_F<double, kCG>(sb, gamma, lam, th_b, F, D);
+  __syncthreads();  // kcs
+  load_F<double, kCG>(sb, gamma, lam, kcs, F, D);
   __syncthreads();
   pivoted_cholesky2(Cw, Rr, D, mask, iflag + 8, scal + 4);
   // M^T[x][s D + j] = g(s, t_x) sum_k R_s[j][k] lam_k F[x][k], g(s, t) = (1 + i sign) / sqrt 2 for
@@ -1508,8 +1471,8 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
     // Its columns are orthogonal to |E| ~ 1e-6; the series of `orthonormalise` is exact to
     // O(|E|^3), and its FP32 products to ~n |E|^2 1e-7.  A basis further off takes a second
     // pass, which starts from ~|E|^3; one beyond the series' range is flagged.
-    const double emax = orthonormalise<true>(Vx, nv, Xs, nv + 1, ev, scal);
-    const double emax2 = emax > 4e-6 ? orthonormalise<true>(Vx, nv, Xs, nv + 1, ev, scal) : 0.0;
+    const double emax = orthonormalise(Vx, nv, Xs, nv + 1, scal);
+    const double emax2 = emax > 4e-6 ? orthonormalise(Vx, nv, Xs, nv + 1, scal) : 0.0;
     if (threadIdx.x == 0 && (!(emax < 1e-2) || !(emax2 < 1e-8))) atomicOr(flags, 1);
   }
   mark(2);
@@ -1623,7 +1586,14 @@ __device__ void bond_body(const BondDesc bd, const V2<T>* __restrict__ partials,
   int* rq = rp + n / 2;
   int* iflag = rq + n / 2;  // [4]
   const int ldr = n + 1;
-  const double th_b = ldst<kCG>(pending + sb.site);
+  __shared__ double kcs[2];
+  if (threadIdx.x + 32 >= blockDim.x) {  // the last warp, while the others sum the Gram partials
+    const double h = 0.5 * ldst<kCG>(pending + sb.site);
+    if (threadIdx.x + 1 == blockDim.x) {
+      kcs[0] = cos(h);
+      kcs[1] = sin(h);
+    }
+  }
   long long t_prev = clock64();
   auto mark = [&](int phase) {
     if (threadIdx.x == 0) {
@@ -1641,7 +1611,7 @@ __device__ void bond_body(const BondDesc bd, const V2<T>* __restrict__ partials,
     uint32_t dyn;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
     const bool shared_work = svd_shared_work(D) > 0 && dyn >= BondSmem(D, 2 * D).small + svd_shared_bytes(D, true);
-    if (!big || !bond_front_svd<kCG>(bd, partials, gsum, gamma, lam, th_b, D, jp, big, lamo, ev, rc, re, scal, re32,
+    if (!big || !bond_front_svd<kCG>(bd, partials, gsum, gamma, lam, kcs, D, jp, big, lamo, ev, rc, re, scal, re32,
                                      rc32, rs32, order, rp, iflag, smallp + L.small, shared_work, jp.full_basis != 0,
                                      sweeps_out, cycles, flags, t_prev, &Vm)) {
       bond_fail<T, kCG>(bd, Y, theta_a, pending, flags, D);
@@ -1666,7 +1636,8 @@ __device__ void bond_body(const BondDesc bd, const V2<T>* __restrict__ partials,
       const double2 v = cscale(acc, lamo[k] * lamo[l]);
       Cs[o] = mk<T>((T)v.x, (T)v.y);
     }
-    load_F<T, kCG>(sb, gamma, lam, th_b, F, D);
+    __syncthreads();  // kcs
+    load_F<T, kCG>(sb, gamma, lam, kcs, F, D);
     for (int idx = threadIdx.x; idx < n * ldr; idx += blockDim.x) RHO[idx] = make_double2(0.0, 0.0);
     __syncthreads();
     // rho = sum_s phase(s) o (conj(F) C_s F^T), upper triangle, then mirrored;
@@ -1737,26 +1708,40 @@ __device__ void bond_body(const BondDesc bd, const V2<T>* __restrict__ partials,
     for (int j = threadIdx.x; j < n; j += blockDim.x) vs[n * n + j] = make_double2(ev[order[j]], 0.0);
   }
   const int keep = n < D ? n : D;
-  if (threadIdx.x == 0) {
-    const double emax = ev[order[0]];
-    double nrm2 = 0.0;
-    for (int kk = 0; kk < D; ++kk) {
-      double sval = 0.0;
-      if (kk < keep) {
-        const double e = ev[order[kk]];
-        if (e > jp.ev_cut * emax && e > 0.0) sval = sqrt(e);
-      }
-      sv[kk] = sval;
-      nrm2 += sval * sval;
+  const int lo_b = sb.lam_o1 >= 0 ? sb.lam_o1 : sb.lam_o2;
+  const double emax = ev[order[0]];
+  for (int kk = threadIdx.x; kk < D; kk += blockDim.x) {
+    double sval = 0.0;
+    if (kk < keep) {
+      const double e = ev[order[kk]];
+      if (e > jp.ev_cut * emax && e > 0.0) sval = sqrt(e);
     }
-    scal[1] = sqrt(nrm2);
-    double mx = 0.0;
-    const int lo = sb.lam_o1 >= 0 ? sb.lam_o1 : sb.lam_o2;
-    if (lo >= 0)
-      for (int k = 0; k < D; ++k) mx = fmax(mx, ldst<kCG>(lam + lo + k));
-    scal[2] = mx;
+    sv[kk] = sval;
   }
-  load_F<T, kCG>(sb, gamma, lam, th_b, F, D);
+  if (threadIdx.x + 32 >= blockDim.x) {  // the last warp: max of the other leg's lambda
+    double mx = 0.0;
+    if (lo_b >= 0)
+      for (int k = threadIdx.x & 31; k < D; k += 32) mx = fmax(mx, ldst<kCG>(lam + lo_b + k));
+    for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    if (threadIdx.x + 1 == blockDim.x) scal[2] = mx;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double nrm2 = 0.0;
+    for (int kk = 0; kk < D; ++kk) nrm2 += sv[kk] * sv[kk];
+    scal[1] = sqrt(nrm2);
+  }
+  // 1 / lambda_other of every row of end b (pseudo-inverse)
+  for (int rj = threadIdx.x; rj < nb; rj += blockDim.x) {
+    const RowPos p = row_pos(sb, rj);
+    double winv = 1.0;
+    if (lo_b >= 0) {
+      const double lv = ldst<kCG>(lam + lo_b + (sb.lam_o1 >= 0 ? p.r1 : p.r2));
+      winv = lv > kLambdaCut * scal[2] ? 1.0 / lv : 0.0;
+    }
+    rc[rj] = winv;
+  }
+  load_F<T, kCG>(sb, gamma, lam, kcs, F, D);
   __syncthreads();
   const double nrm = scal[1];
   if (!(nrm > 0.0) || !isfinite(nrm)) {
@@ -1786,40 +1771,39 @@ __device__ void bond_body(const BondDesc bd, const V2<T>* __restrict__ partials,
     const int k = kl / D, kk = kl - (kl / D) * D;
     V2<T> acc = mk<T>(0, 0);
     if (sv[kk] > 0.0) {
-      const int col = order[kk];
-      for (int x = 0; x < n; ++x) {
-        const V2<T> fv = F[x * D + k];
-        const V2<T> g = mk<T>(r2, ((sidx == (x & 1)) == (jp.gate_sign > 0)) ? r2 : -r2);
-        V2<T> vv;
-        if constexpr (sizeof(T) == 4) {
-          vv = Vk[x * D + kk];
-        } else {
-          const double2 vd = Vm[x * n + col];
-          vv = mk<T>((T)vd.x, (T)vd.y);
+      if constexpr (sizeof(T) == 4) {
+        for (int x = 0; x < n; ++x) {
+          const V2<T> fv = F[x * D + k];
+          const V2<T> g = mk<T>(r2, ((sidx == (x & 1)) == (jp.gate_sign > 0)) ? r2 : -r2);
+          fma_c<T>(acc, c_mul<T>(fv, g), Vk[x * D + kk]);
         }
-        fma_c<T>(acc, c_mul<T>(fv, g), vv);
+      } else {
+        // the phase depends on x's parity only: two sums, half the FP64 work
+        const int col = order[kk];
+        V2<T> odd = acc;
+#pragma unroll 2
+        for (int x = 0; x < n; x += 2) {
+          fma_c<T>(acc, F[x * D + k], Vm[x * n + col]);
+          fma_c<T>(odd, F[(x + 1) * D + k], Vm[(x + 1) * n + col]);
+        }
+        const T i0 = ((sidx == 0) == (jp.gate_sign > 0)) ? r2 : -r2;  // g(s, 0) = r2 + i i0, g(s, 1) its conjugate
+        acc = mk<T>(fma(r2, acc.x + odd.x, __dmul_rn(-i0, acc.y - odd.y)),
+                    fma(r2, acc.y + odd.y, __dmul_rn(i0, acc.x - odd.x)));
       }
       acc = c_scale<T>(acc, (T)(lamo[k] / sv[kk]));
     }
     Y[o] = acc;
   }
   // Gamma_b'[t][row][kk] = conj(V[(row, t)][order[kk]]) / lambda_other(row)
-  {
-    const double mx = scal[2];
-    for (int idx = threadIdx.x; idx < n * D; idx += blockDim.x) {
-      const int x = idx / D, kk = idx - (idx / D) * D;
-      const int rj = x >> 1, t = x & 1;
-      const RowPos p = row_pos(sb, rj);
-      double winv = 1.0;
-      const int lo = sb.lam_o1 >= 0 ? sb.lam_o1 : sb.lam_o2;
-      if (lo >= 0) {
-        const double lv = ldst<kCG>(lam + lo + (sb.lam_o1 >= 0 ? p.r1 : p.r2));
-        winv = lv > kLambdaCut * mx ? 1.0 / lv : 0.0;
-      }
-      double2 v = make_double2(0.0, 0.0);
-      if (sv[kk] > 0.0) v = cscale(cconj(Vm[x * n + order[kk]]), winv);
-      gamma[elem(sb, t, p, kk)] = mk<T>((T)v.x, (T)v.y);
+  for (int idx = threadIdx.x; idx < n * D; idx += blockDim.x) {
+    const int x = idx / D, kk = idx - (idx / D) * D;
+    const int rj = x >> 1, t = x & 1;
+    V2<T> v = mk<T>(0, 0);
+    if (sv[kk] > 0.0) {
+      const double2 vd = cscale(cconj(Vm[x * n + order[kk]]), rc[rj]);
+      v = mk<T>((T)vd.x, (T)vd.y);
     }
+    gamma[elem(sb, t, row_pos(sb, rj), kk)] = v;
   }
   __syncthreads();
   // new lambda of the bond; kick angles consumed
@@ -1922,7 +1906,8 @@ __device__ void fused_gram(const SideDesc& sa, const V2<T>* gamma, const double*
   V2<T>* A = reinterpret_cast<V2<T>*>(sm);  // [nrows][2D+1]
   const int ld = 2 * D + 1;
   const int D2 = D * D, nout = 2 * D2;
-  const T c = (T)cos(0.5 * th), s = (T)sin(0.5 * th);
+  const V2<T> cs = kick_factors<T>(th);
+  const T c = cs.x, s = cs.y;
   for (int o = threadIdx.x; o < nout; o += blockDim.x) gsum[o] = make_double2(0.0, 0.0);
   const int tr = tile_rows(D, sizeof(V2<T>));
   const int ntiles = (sa.rows + tr - 1) / tr;
@@ -1983,7 +1968,8 @@ __device__ void fused_update(const SideDesc& sa, V2<T>* gamma, const double* lam
       for (int k = 0; k < D; ++k) mx = fmax(mx, __ldcg(lam + lo + k));
     cut[threadIdx.x] = kLambdaCut * mx;
   }
-  const T c = (T)cos(0.5 * th), s = (T)sin(0.5 * th);
+  const V2<T> cs = kick_factors<T>(th);
+  const T c = cs.x, s = cs.y;
   const int ntiles = (sa.rows + tr - 1) / tr;
   for (int tp = 0; tp < ntiles; ++tp) {
     const int row0 = tp * tr;
@@ -2111,7 +2097,8 @@ __device__ bool tc_update_pass(const SideDesc& sa, float2* gamma, const double* 
                                int D, unsigned char* sm, const TcCtx& cx, uint32_t& phase) {
   __shared__ double cut[2];
   float* mask = reinterpret_cast<float*>(sm + tc_update_smem(D) - 128 * 4);
-  const float c = (float)cos(0.5 * th), s = (float)sin(0.5 * th);
+  const float2 cs = kick_factors<float>(th);
+  const float c = cs.x, s = cs.y;
   bool ok = true;
   for (int row0 = 0; row0 < sa.rows && ok; row0 += 128) {
     const int nrows = sa.rows - row0 < 128 ? sa.rows - row0 : 128;
@@ -2141,7 +2128,8 @@ __global__ void __launch_bounds__(128)
   const BondDesc& bd = bonds[blockIdx.x];
   const SideDesc sa = bd.a;
   const double th = pending[sa.site];
-  const float c = (float)cos(0.5 * th), s = (float)sin(0.5 * th);
+  const float2 cs = kick_factors<float>(th);
+  const float c = cs.x, s = cs.y;
   const int D2 = D * D;
   const bool ok = tc_gram_pass<false>(sa, gamma, lam, c, s, D, smem_raw, cx, mphase, sphase, nullptr,
                                       partials + (int64_t)bd.part0 * 2 * D2);
@@ -2181,7 +2169,8 @@ __device__ bool tc_fused_gram(const SideDesc& sa, const float2* gamma, const dou
     for (int o = threadIdx.x; o < nout; o += blockDim.x) gsum[o] = make_double2(0.0, 0.0);
     __syncthreads();
   }
-  const float c = (float)cos(0.5 * th), s = (float)sin(0.5 * th);
+  const float2 cs = kick_factors<float>(th);
+  const float c = cs.x, s = cs.y;
   return tc_gram_pass<true, kNb>(sa, gamma, lam, c, s, D, sm, cx, mphase, sphase, gsum, part);
 }
 
@@ -2344,7 +2333,8 @@ __global__ void __launch_bounds__(kThreads)
     cut[threadIdx.x] = kLambdaCut * mx;
   }
   const double th = theta_a[t.bond];
-  const T c = (T)cos(0.5 * th), s = (T)sin(0.5 * th);
+  const V2<T> cs = kick_factors<T>(th);
+  const T c = cs.x, s = cs.y;
   const int nel = t.nrows * D;
   for (int idx = threadIdx.x; idx < nel; idx += blockDim.x) {
     int r, k;
@@ -2438,7 +2428,8 @@ __global__ void __launch_bounds__(kThreads)
   // conversions and adds (64 cycles of an SMSP's FP64 unit per warp
   // instruction) off the per-element path
   const double th = pending[blockIdx.x];
-  const T c = (T)cos(0.5 * th), s = (T)sin(0.5 * th);
+  const V2<T> cs = kick_factors<T>(th);
+  const T c = cs.x, s = cs.y;
   // base-D digits of the element index (leg deg-1 fastest) and of the stride, stepped with carries
   int dg[3] = {0, 0, 0}, st[3] = {0, 0, 0};
   {
@@ -2983,7 +2974,8 @@ __global__ void __launch_bounds__(kThreads)
     Cs[o] = cscale(g, lamo[k] * lamo[l]);
     Yb[o] = y;
   }
-  load_F<double, false>(sb, gamma, lam, 0.0, F, D);
+  const double no_kick[2] = {1.0, 0.0};
+  load_F<double, false>(sb, gamma, lam, no_kick, F, D);
   // the forward's eigenvectors (sorted by decreasing eigenvalue) and eigenvalues: the
   // output adjoints are expressed in the forward's gauge, so the same V must be used
   {
@@ -3316,7 +3308,8 @@ __global__ void apply_kick_kernel(const SiteDesc* __restrict__ sites, double2* g
   int nel = 1;
   for (int q = 0; q < sd.deg; ++q) nel *= D;
   const double th = theta[blockIdx.x];
-  const double c = cos(0.5 * th), s = sin(0.5 * th);
+  const double2 cs = kick_factors<double>(th);
+  const double c = cs.x, s = cs.y;
   for (int idx = threadIdx.x; idx < nel; idx += blockDim.x) {
     double2 a0, a1;
     kick2<double>(c, s, gamma[sd.off + idx], gamma[sd.off + nel + idx], a0, a1);
@@ -3332,7 +3325,8 @@ __global__ void adj_kick_kernel(const SiteDesc* __restrict__ sites, const double
   int nel = 1;
   for (int q = 0; q < sd.deg; ++q) nel *= D;
   const double th = theta[blockIdx.x];
-  const double c = cos(0.5 * th), s = sin(0.5 * th);
+  const double2 cs = kick_factors<double>(th);
+  const double c = cs.x, s = cs.y;
   double acc = 0.0;
   for (int idx = threadIdx.x; idx < nel; idx += blockDim.x) {
     const double2 g0 = gbar[sd.off + idx], g1 = gbar[sd.off + nel + idx];
