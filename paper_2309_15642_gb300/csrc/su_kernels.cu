@@ -1116,6 +1116,11 @@ __device__ int os_sweeps(double2* Zt, int rows, double2* Vt, int n, double tol, 
 // FP32 one-sided stages: relative threshold jp.tol32 (at the rounding of an FP32 dot product) and
 // this absolute one, in units of the largest squared column norm (its square stays an FP32 normal)
 constexpr float kOsFloor32 = 1e-18f;
+// tol32 of the warm start, whose columns become the basis: below 1e-6 an FP32 dot product does not
+// get, above 1e-5 the FP64 re-orthonormalisation would start too far off
+__device__ __forceinline__ float basis_tol32(const JacobiParams& jp) {
+  return fminf(fmaxf((float)jp.tol32, 1e-6f), 1e-5f);
+}
 // The warm start replaces remaining columns below this fraction of the first pivot by unit vectors of that size
 constexpr float kBasisCut = 1e-6f;
 
@@ -1131,7 +1136,7 @@ constexpr float kBasisCut = 1e-6f;
 // vectors sought, so that no rotation product is accumulated.  When every remaining
 // vector is below kBasisCut of the first pivot the rest of R is replaced by that
 // multiple of the identity: below FP32's resolution any completion serves, and the
-// Jacobi makes it orthogonal to the others.  nv even; len, nv <= ld <= 256.
+// Jacobi makes it orthogonal to the others.  A solve that ends at its sweep cap gives the identity.  nv even; len, nv <= ld <= 256.
 __device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* nrm, const JacobiParams& jp, float* rc,
                          float* rs, float2* re, int* iflag, unsigned long long* work,
                          unsigned long long* rot_count) {
@@ -1225,7 +1230,7 @@ __device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* 
     if (nrm[v] >= 0.f)
       for (int x = lane; x < nv; x += 32) A[(size_t)v * ld + x] = make_float2(x == v ? eta : 0.f, 0.f);
   __syncthreads();
-  const int sw = one_sided_jacobi32(A, ld, nv, nullptr, nv, (float)jp.tol32, kOsFloor32, jp.max_sweeps32, rc, rs, re,
+  const int sw = one_sided_jacobi32(A, ld, nv, nullptr, nv, basis_tol32(jp), kOsFloor32, jp.max_sweeps32, rc, rs, re,
                                     iflag, work, rot_count);
   for (int v = warp; v < nv; v += nw) {
     float s = 0.f;
@@ -1240,7 +1245,8 @@ __device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* 
   for (int idx = threadIdx.x; idx < nv * nv; idx += blockDim.x) {
     const int v = idx / nv, i = idx - (idx / nv) * nv;
     const float2 a = A[(size_t)i * ld + v];
-    X[idx] = make_double2((double)(a.x * nrm[i]), (double)(a.y * nrm[i]));
+    X[idx] = sw > jp.max_sweeps32 ? make_double2(v == i ? 1.0 : 0.0, 0.0)  // not orthogonal yet: the identity
+                                  : make_double2((double)(a.x * nrm[i]), (double)(a.y * nrm[i]));
   }
   __syncthreads();
   return sw;
@@ -1693,6 +1699,8 @@ __device__ void bond_body(const BondDesc bd, const V2<T>* __restrict__ partials,
     for (int i = threadIdx.x; i < n; i += blockDim.x) ev[i] = RHO[i * ldr + i].x;
     __syncthreads();
   }
+  for (int i = threadIdx.x; i < n; i += blockDim.x) order[i] = i;  // an index even if some ev is NaN
+  __syncthreads();
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     int rank = 0;
     const double vi = ev[i];
