@@ -814,7 +814,10 @@ __device__ __forceinline__ void os_rot(float a, float b, float2 g, float& c, flo
   float ig = rsqrtf(g2);
   ig = ig * fmaf(-0.5f * g2, ig * ig, 1.5f);
   const float zeta = (b - a) * (0.5f * ig);
-  const float t = copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
+  float rt, t;  // an approximate t is still a unitary rotation
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(rt) : "f"(fmaf(zeta, zeta, 1.f)));
+  asm("rcp.approx.f32 %0, %1;" : "=f"(t) : "f"(fabsf(zeta) + rt));
+  t = copysignf(t, zeta);
   const float u = fmaf(t, t, 1.f);
   float cc = rsqrtf(u);
   cc = cc * fmaf(-0.5f * u, cc * cc, 1.5f);
@@ -825,112 +828,99 @@ __device__ __forceinline__ void os_rot(float a, float b, float2 g, float& c, flo
 
 // One-sided (Hestenes) Jacobi in FP32 on the n columns of B (Bt [n], stride ld, of
 // `rows` entries), with W^T (Wt [n][n], or null) rotated alongside.  A sweep runs
-// the n - 1 rounds of the round-robin pairing; a round (1) forms |b_p|^2, |b_q|^2
-// and g = b_p^H b_q of its n/2 disjoint pairs from the columns themselves (8 lanes
-// per pair), (2) decides and builds every rotation with one thread per pair: pair
-// (p, q) rotates when |g| > max(tol |b_p| |b_q|, floor_abs), by
-// b_p <- c b_p - s e b_q, b_q <- s b_p + c e b_q, (3) applies the rotations of the
-// active pairs only.  A sweep without rotations ends the solve.  Returns the sweeps
-// (max_sweeps + 1 = cap hit); work[0] += pair checks, work[1] += rotations,
+// the n - 1 rounds of the round-robin pairing; pair (p, q) rotates when
+// |b_p^H b_q| > max(tol |b_p| |b_q|, floor_abs), by b_p <- c b_p - s e b_q,
+// b_q <- s b_p + c e b_q.  A sweep without rotations ends the solve.  Returns the
+// sweeps (max_sweeps + 1 = cap hit); work[0] += pair checks, work[1] += rotations,
 // rot_count[sweep] += rotations of the first kRotSweeps sweeps (either may be
-// null).  rc, rs: n/2 reals; re: n/2 complex; iflag: the integer scratch of
-// jacobi_hermitian.  n <= 256, blockDim.x >= n/2 rounded up to 32.
-__device__ int one_sided_jacobi32(float2* Bt, int ld, int rows, float2* Wt, int n, float tol, float floor_abs,
-                                  int max_sweeps, float* rc, float* rs, float2* re, int* iflag,
-                                  unsigned long long* work, unsigned long long* rot_count) {
+// null).  iflag[3]: scratch.  n even; n, rows <= 256.
+//
+// Bound by issue slots and shared memory, so a pair is read once and written once a
+// round: L = 8, 16 or 32 lanes (by the column length alone, so that every CTA size sums
+// in the same order) hold both columns in registers, form norms and inner product,
+// each builds the rotation for itself, and the columns are written back only if the
+// pair rotates.  One barrier a round, against three with norms, rotations and updates as
+// phases over the CTA.
+__device__ __noinline__ int one_sided_jacobi32(float2* Bt, int ld, int rows, float2* Wt, int n, float tol, float floor_abs,
+                                  int max_sweeps, int* iflag, unsigned long long* work,
+                                  unsigned long long* rot_count) {
+  constexpr int kR = 8;  // entries of a column per lane
   const int m = n / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int sub = lane & 7, grp = lane >> 3;
-  int* act = iflag + 8;     // [4 warps][32] active pairs of the round
-  int* wcnt = iflag + 136;  // active pairs per warp
-  const int npw = (m + 31) >> 5;  // warps that build the rotations (n <= 256: at most 4)
+  const int L = rows <= 8 * kR ? 8 : rows <= 16 * kR ? 16 : 32;
+  const int per = 32 / L, sub = lane & (L - 1), grp = lane / L;
   const float tol2 = tol * tol, floor2 = floor_abs * floor_abs;
-  const int len = rows + (Wt ? n : 0);
   unsigned long long n_chk = 0, n_rot = 0;
   int result = max_sweeps + 1;
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     if (threadIdx.x == 0) iflag[3] = 0;
+    int mine = 0;  // lanes with sub == 0: rotations of this sweep
     for (int r = 0; r < n - 1; ++r) {
-      // (1) norms and inner product of every pair: rc[k] = |b_p|^2, rs[k] = |b_q|^2, re[k] = g
-      for (int k0 = warp * 4; k0 < m; k0 += nw * 4) {
+      for (int k0 = warp * per; k0 < m; k0 += nw * per) {
         const int k = k0 + grp;
-        float a = 0, b = 0;
-        float2 g = make_float2(0.f, 0.f);
-        if (k < m) {
-          int p, q;
-          round_pair(r, k, n, p, q);
-          const float2* bp = Bt + (size_t)p * ld;
-          const float2* bq = Bt + (size_t)q * ld;
-          for (int i = sub; i < rows; i += 8) {
-            const float2 u = bp[i], v = bq[i];
-            a = fmaf(u.x, u.x, fmaf(u.y, u.y, a));
-            b = fmaf(v.x, v.x, fmaf(v.y, v.y, b));
-            fma_conj<float>(g, u, v);
-          }
+        const bool in = k < m;
+        int p = 0, q = 0;
+        if (in) round_pair(r, k, n, p, q);
+        float2* bp = Bt + (size_t)p * ld;
+        float2* bq = Bt + (size_t)q * ld;
+        float2 u[kR], v[kR];
+#pragma unroll
+        for (int t = 0; t < kR; ++t) {  // all loads in flight before the sums
+          const bool on = in && sub + t * L < rows;
+          u[t] = on ? bp[sub + t * L] : make_float2(0.f, 0.f);
+          v[t] = on ? bq[sub + t * L] : make_float2(0.f, 0.f);
         }
-        for (int off = 4; off > 0; off >>= 1) {
+        float a = 0.f, b = 0.f;
+        float2 g = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int t = 0; t < kR; ++t) {
+          a = fmaf(u[t].x, u[t].x, fmaf(u[t].y, u[t].y, a));
+          b = fmaf(v[t].x, v[t].x, fmaf(v[t].y, v[t].y, b));
+          fma_conj<float>(g, u[t], v[t]);
+        }
+        for (int off = L >> 1; off > 0; off >>= 1) {
           a += __shfl_xor_sync(0xffffffffu, a, off);
           b += __shfl_xor_sync(0xffffffffu, b, off);
           g.x += __shfl_xor_sync(0xffffffffu, g.x, off);
           g.y += __shfl_xor_sync(0xffffffffu, g.y, off);
         }
-        if (k < m && sub == 0) {
-          rc[k] = a;
-          rs[k] = b;
-          re[k] = g;
+        const float g2 = fmaf(g.x, g.x, g.y * g.y);
+        if (in && g2 > tol2 * a * b && g2 > floor2) {
+          float c, sn;
+          float2 e;
+          os_rot(a, b, g, c, sn, e);
+          // explicit roundings: the same bits in every kernel that inlines this
+          auto turn = [&](float2& x, float2& y) {
+            const float2 w = make_float2(fmaf(y.x, e.x, -__fmul_rn(y.y, e.y)), fmaf(y.x, e.y, __fmul_rn(y.y, e.x)));
+            y = make_float2(fmaf(sn, x.x, __fmul_rn(c, w.x)), fmaf(sn, x.y, __fmul_rn(c, w.y)));
+            x = make_float2(fmaf(c, x.x, -__fmul_rn(sn, w.x)), fmaf(c, x.y, -__fmul_rn(sn, w.y)));
+          };
+#pragma unroll
+          for (int t = 0; t < kR; ++t) turn(u[t], v[t]);
+#pragma unroll
+          for (int t = 0; t < kR; ++t)
+            if (sub + t * L < rows) {
+              bp[sub + t * L] = u[t];
+              bq[sub + t * L] = v[t];
+            }
+          if (Wt)
+            for (int i = sub; i < n; i += L) {
+              float2* wp = Wt + (size_t)p * n + i;
+              float2* wq = Wt + (size_t)q * n + i;
+              turn(*wp, *wq);
+            }
+          if (sub == 0) ++mine;
         }
-      }
-      __syncthreads();
-      // (2) one thread per pair: test, rotation (c, s, e) into rc, rs, re, compacted active list
-      if (warp < npw) {
-        const int k = threadIdx.x;
-        bool on = false;
-        if (k < m) {
-          const float2 g = re[k];
-          const float a = rc[k], b = rs[k];
-          const float g2 = fmaf(g.x, g.x, g.y * g.y);
-          on = g2 > tol2 * a * b && g2 > floor2;
-          if (on) {
-            float c, sn;
-            float2 e;
-            os_rot(a, b, g, c, sn, e);
-            rc[k] = c;
-            rs[k] = sn;
-            re[k] = e;
-          }
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, on);
-        if (on) act[warp * 32 + __popc(bal & ((1u << lane) - 1u))] = k;
-        if (lane == 0) wcnt[warp] = __popc(bal);
-      }
-      __syncthreads();
-      // prefix counts of the warps' lists (scalars: a runtime-indexed array would live in local memory)
-      const int p1 = wcnt[0], p2 = p1 + (npw > 1 ? wcnt[1] : 0), p3 = p2 + (npw > 2 ? wcnt[2] : 0);
-      const int na = p3 + (npw > 3 ? wcnt[3] : 0);
-      if (threadIdx.x == 0) {
-        iflag[3] += na;
-        n_chk += (unsigned long long)m;
-        n_rot += (unsigned long long)na;
-      }
-      if (na == 0) continue;  // nothing below reads this round's scratch
-      // (3) the active rotations over the rows of B, then of W
-      for (int t = threadIdx.x; t < na * len; t += blockDim.x) {
-        const int ia = t / len, i = t - ia * len;
-        const int k = ia < p1 ? act[ia] : ia < p2 ? act[32 + ia - p1] : ia < p3 ? act[64 + ia - p2] : act[96 + ia - p3];
-        int p, q;
-        round_pair(r, k, n, p, q);
-        float2* xp = i < rows ? Bt + (size_t)p * ld + i : Wt + (size_t)p * n + (i - rows);
-        float2* xq = i < rows ? Bt + (size_t)q * ld + i : Wt + (size_t)q * n + (i - rows);
-        const float c = rc[k], sn = rs[k];
-        // explicit roundings: the same bits in every kernel that inlines this
-        const float2 u = *xp, y = *xq, e = re[k];
-        const float2 v = make_float2(fmaf(y.x, e.x, -__fmul_rn(y.y, e.y)), fmaf(y.x, e.y, __fmul_rn(y.y, e.x)));
-        *xp = make_float2(fmaf(c, u.x, -__fmul_rn(sn, v.x)), fmaf(c, u.y, -__fmul_rn(sn, v.y)));
-        *xq = make_float2(fmaf(sn, u.x, __fmul_rn(c, v.x)), fmaf(sn, u.y, __fmul_rn(c, v.y)));
       }
       __syncthreads();
     }
+    if (mine) atomicAdd(iflag + 3, mine);
+    __syncthreads();
     const int total = iflag[3];
-    if (threadIdx.x == 0 && rot_count && sweep < kRotSweeps) atomicAdd(rot_count + sweep, (unsigned long long)total);
+    if (threadIdx.x == 0) {
+      n_chk += (unsigned long long)m * (n - 1);
+      n_rot += (unsigned long long)total;
+      if (rot_count && sweep < kRotSweeps) atomicAdd(rot_count + sweep, (unsigned long long)total);
+    }
     __syncthreads();
     if (total == 0) {
       result = sweep + 1;
@@ -1137,9 +1127,8 @@ constexpr float kBasisCut = 1e-6f;
 // vector is below kBasisCut of the first pivot the rest of R is replaced by that
 // multiple of the identity: below FP32's resolution any completion serves, and the
 // Jacobi makes it orthogonal to the others.  A solve that ends at its sweep cap gives the identity.  nv even; len, nv <= ld <= 256.
-__device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* nrm, const JacobiParams& jp, float* rc,
-                         float* rs, float2* re, int* iflag, unsigned long long* work,
-                         unsigned long long* rot_count) {
+__device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* nrm, const JacobiParams& jp,
+                         int* iflag, unsigned long long* work, unsigned long long* rot_count) {
   constexpr int kT = kMaxDc128 * 2 / 32;  // elements of a vector per lane
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   auto wsum = [](float v) {
@@ -1230,8 +1219,8 @@ __device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* 
     if (nrm[v] >= 0.f)
       for (int x = lane; x < nv; x += 32) A[(size_t)v * ld + x] = make_float2(x == v ? eta : 0.f, 0.f);
   __syncthreads();
-  const int sw = one_sided_jacobi32(A, ld, nv, nullptr, nv, basis_tol32(jp), kOsFloor32, jp.max_sweeps32, rc, rs, re,
-                                    iflag, work, rot_count);
+  const int sw = one_sided_jacobi32(A, ld, nv, nullptr, nv, basis_tol32(jp), kOsFloor32, jp.max_sweeps32, iflag,
+                                    work, rot_count);
   for (int v = warp; v < nv; v += nw) {
     float s = 0.f;
     for (int x = lane; x < nv; x += 32) {
@@ -1281,8 +1270,8 @@ __host__ __device__ size_t svd_shared_bytes(int D, bool with_work) {
 // the block would be their contamination).  lvl: svd_level_bytes, W64: 2 lv^2 + lv
 // complex doubles.
 __device__ void svd_levels(double2* Zt, int rows, double2* Vt, int n, double tr, const JacobiParams& jp,
-                           double* alpha, double* rscale, int* mark_c, int* cand, double* scal, float2* re32,
-                           float* rc32, float* rs32, int* iflag, unsigned char* lvl, double2* W64,
+                           double* alpha, double* rscale, int* mark_c, int* cand, double* scal,
+                           int* iflag, unsigned char* lvl, double2* W64,
                            unsigned long long* sweeps_out) {
   const int cap = (n / 2 < kMaxLevel) ? n / 2 : kMaxLevel;
   float2* B32 = reinterpret_cast<float2*>(lvl);  // [cap][rows]
@@ -1333,8 +1322,13 @@ __device__ void svd_levels(double2* Zt, int rows, double2* Vt, int n, double tr,
     for (int idx = threadIdx.x; idx < ns * ns; idx += blockDim.x)
       W32[idx] = make_float2((idx / ns) == (idx % ns) ? 1.f : 0.f, 0.f);
     __syncthreads();
-    one_sided_jacobi32(B32, rows, rows, W32, ns, (float)jp.tol32, kOsFloor32, jp.max_sweeps32, rc32, rs32, re32,
-                       iflag, sweeps_out + 6, nullptr);
+    const int swl = one_sided_jacobi32(B32, rows, rows, W32, ns, (float)jp.tol32, kOsFloor32, jp.max_sweeps32, iflag,
+                       sweeps_out + 6, nullptr);
+    if (swl == 1) {  // no rotation: W is the identity
+      for (int a = threadIdx.x; a < ns; a += blockDim.x) rscale[cand[a]] = bscale;
+      __syncthreads();
+      continue;
+    }
     for (int idx = threadIdx.x; idx < ns * ns; idx += blockDim.x) {
       const int a = idx / ns, b = idx - (idx / ns) * ns;
       const float2 v = W32[(size_t)b * ns + a];
@@ -1382,7 +1376,7 @@ template <bool kCG>
 __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ partials, const double2* gsum,
                                const double2* gamma, const double* lam, const double* kcs, int D, const JacobiParams& jp,
                                unsigned char* big, double* lamo, double* ev, double* rc, double2* re, double* scal,
-                               float2* re32, float* rc32, float* rs32, int* order, int* rp, int* iflag,
+                               int* order, int* rp, int* iflag,
                                unsigned char* lvl, bool shared_work, bool full, unsigned long long* sweeps_out,
                                unsigned long long* cycles, int* flags, long long& t_prev, double2** Vm_out) {
   const SideDesc& sb = bd.b;
@@ -1470,7 +1464,7 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
     }
   }
   __syncthreads();
-  const int sw32 = svd_basis(A32, nv, left ? n : rows, rows, Vx, reinterpret_cast<float*>(ev), jp, rc32, rs32, re32,
+  const int sw32 = svd_basis(A32, nv, left ? n : rows, rows, Vx, reinterpret_cast<float*>(ev), jp,
                              iflag, sweeps_out + 6, cycles ? cycles + kPhases : nullptr);
   mark(1);
   {
@@ -1517,7 +1511,7 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
                             sweeps_out + 4, rot);
   mark(4);
   // level marks in rp (n ints, free until a level's Jacobi), candidates in order; M is not needed any more
-  svd_levels(Zt, zr, Vt, n, trace, jp, ev, rc, rp, order, scal, re32, rc32, rs32, iflag, lvl, Mt, sweeps_out);
+  svd_levels(Zt, zr, Vt, n, trace, jp, ev, rc, rp, order, scal, iflag, lvl, Mt, sweeps_out);
   mark(3);
   const int sweeps = sw1 == 1 ? 1
                               : 1 + os_sweeps(Zt, zr, Vt, n, jp.tol, jp.floor_rel * trace, trace, jp.max_sweeps - 1,
@@ -1617,8 +1611,8 @@ __device__ void bond_body(const BondDesc bd, const V2<T>* __restrict__ partials,
     uint32_t dyn;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
     const bool shared_work = svd_shared_work(D) > 0 && dyn >= BondSmem(D, 2 * D).small + svd_shared_bytes(D, true);
-    if (!big || !bond_front_svd<kCG>(bd, partials, gsum, gamma, lam, kcs, D, jp, big, lamo, ev, rc, re, scal, re32,
-                                     rc32, rs32, order, rp, iflag, smallp + L.small, shared_work, jp.full_basis != 0,
+    if (!big || !bond_front_svd<kCG>(bd, partials, gsum, gamma, lam, kcs, D, jp, big, lamo, ev, rc, re, scal,
+                                     order, rp, iflag, smallp + L.small, shared_work, jp.full_basis != 0,
                                      sweeps_out, cycles, flags, t_prev, &Vm)) {
       bond_fail<T, kCG>(bd, Y, theta_a, pending, flags, D);
       return;

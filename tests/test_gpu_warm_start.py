@@ -58,3 +58,8 @@ def test_a_capped_warm_start_leaves_the_work_to_the_fp64_sweeps(dtype, tol, cap)
 @pytest.mark.parametrize("tol32", [1e-9, 1e-2])
 def test_a_warm_start_tolerance_out_of_range_is_brought_into_it(tol32):
     assert _step(16, settings=lambda g: g.set_jacobi(tol32=tol32)) <= 1e-10
+
+
+@pytest.mark.parametrize("D", [3, 4, 9, 23, 24, 31, 32, 33, 64, 65])
+def test_step_of_a_random_state(D):
+    assert _step(D) <= 1e-10
