@@ -35,66 +35,26 @@
 //
 // Included by su_kernels.cu after its row/element helpers.
 #pragma once
-#include <cuda_fp16.h>
-
+#include "oz_mma.cuh"
 #include "tcgen05.cuh"
 
 namespace gpeps {
 
 constexpr int kOzThreads = 512;
-constexpr int kOzSlices = 7;
 constexpr int kOzOperand = kOzSlices * 128 * 64 * 2;  // bytes of 7 slices of 8192 digits
 constexpr int kOzDumpLd = 129;                        // row stride (doubles) of the Gram readout
 constexpr size_t kOzGramSmem = (size_t)128 * kOzDumpLd * 8;
 constexpr size_t kOzUpdateSmem = (size_t)kOzOperand + kOzOperand / 2;
 
-__device__ __forceinline__ int oz_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
-// Biased fixed point: round(x 2^(54 - E)) + 0x80 in each of the 7 digit bytes, E =
-// em - 1022 for the row's largest biased exponent em: byte 6 - i minus 128 is d_i.
-__device__ __forceinline__ unsigned long long oz_fixed(double x, int em, bool negate = false) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)(b >> 52) & 0x7ff, d = em - ex;
-  unsigned long long m = ((b & 0xfffffffffffffull) | 0x10000000000000ull) << 1;
-  m = (m + ((1ull << (d & 63)) >> 1)) >> (d & 63);
-  if (d > 55 || ex == 0) m = 0;
-  const bool neg = ((long long)b < 0) != negate;
-  return (neg ? 0ull - m : m) + 0x0080808080808080ull;
-}
-
 // The digits of 8 consecutive K values of one operand row: one 16-byte store per slice.
 __device__ __forceinline__ void oz_store(unsigned char* p, uint32_t slice_bytes, const unsigned long long* v) {
 #pragma unroll
   for (int i = 0; i < kOzSlices; ++i) {
-    const int byte = 6 - i;
     uint32_t w[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t a = (uint32_t)(v[2 * q] >> (byte >= 4 ? 32 : 0));
-      const uint32_t b = (uint32_t)(v[2 * q + 1] >> (byte >= 4 ? 32 : 0));
-      const uint32_t s = byte & 3;
-      // two bytes -> f16 1024 + byte -> byte - 128
-      const uint32_t t = (__byte_perm(a, b, s | (s << 4) | ((4 + s) << 8) | ((4 + s) << 12)) & 0x00ff00ffu) | 0x64006400u;
-      const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&t), __half2half2(__ushort_as_half(0x6480)));
-      w[q] = *reinterpret_cast<const uint32_t*>(&h);
-    }
+    for (int q = 0; q < 4; ++q) w[q] = oz_pair(v[2 * q], v[2 * q + 1], i);
     *reinterpret_cast<uint4*>(p + (size_t)i * slice_bytes) = make_uint4(w[0], w[1], w[2], w[3]);
   }
-}
-
-// t 2^(ea + eb - 2044 - 52) rounded to FP64 (ea, eb: biased exponents of the two rows);
-// NaN when a row held a value that is not finite.
-__device__ __forceinline__ double oz_value(long long t, int ea, int eb) {
-  if (ea == 0x7ff || eb == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);
-  const unsigned long long u = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
-  if (u == 0) return 0.0;
-  const int n = __clzll((long long)u);
-  const unsigned long long m = u << n;  // top bit at 63: value m 2^(-n) 2^(...)
-  const int e = 1023 + 63 - n + ea + eb - 2044 - 52;
-  if (e <= 0) return 0.0;
-  if (e >= 0x7ff) return __longlong_as_double(t < 0 ? 0xfff0000000000000ll : 0x7ff0000000000000ll);
-  const unsigned long long r = ((unsigned long long)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
-  return __longlong_as_double((long long)(r | (t < 0 ? 0x8000000000000000ull : 0ull)));
 }
 
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, int n, uint32_t accumulate) {

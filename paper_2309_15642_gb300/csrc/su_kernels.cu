@@ -29,6 +29,7 @@
 
 #include "gpeps_internal.cuh"
 #include "jacobi.cuh"
+#include "oz_mma.cuh"
 
 namespace gpeps {
 
@@ -264,18 +265,33 @@ __device__ __forceinline__ void upper_index(int idx, int n, int& i, int& j) {
 // stay FP64.  The FP32 copy of upper entry (i, j) sits in the otherwise unused
 // 16 bytes mirrored below the diagonal, (j, i) for i < j and the padding column
 // (i, n) for i = j (ldg >= n + 1): X1 in its first 8 bytes, X in its last 8.
-// Q pairs the columns j and n-1-j on one lane (n <= 128).
+// Q pairs the columns j and n-1-j on one lane (n <= 128).  With kOz (ex: 2n ints), from
+// kOzMinBond columns on, E and Q are integer digit products on the tensor cores.
+// Cores of fewer columns keep FP64 multiply-adds, and so does the mixed path, whose results keep their bits.
+constexpr int kOzMinBond = 48;
 __device__ __forceinline__ float2* tri32(double2* G, int ldg, int n, int i, int j) {
   return reinterpret_cast<float2*>(i < j ? G + j * ldg + i : G + i * ldg + n);
 }
 
-__device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double* scal) {
+template <bool kOz>
+__device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double* scal, int* ex = nullptr) {
+  const bool oz = kOz && n >= kOzMinBond;
+  if (oz) {
+    oz_product(V, 1, n, true, V, 1, n, ex, G, ldg, 1, n, true);
+    __syncthreads();
+  }
   // E = V^dagger V - I (upper triangle, FP64) and the FP32 copy of X1 = P(E)
   for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
     int i, j;
     upper_index(idx, n, i, j);
-    double2 acc = make_double2(i == j ? -1.0 : 0.0, 0.0);
-    for (int r = 0; r < n; ++r) fma_conj<double>(acc, V[r * n + i], V[r * n + j]);
+    double2 acc = make_double2(0.0, 0.0);
+    if (oz) {
+      acc = G[i * ldg + j];
+      if (i == j) acc.x -= 1.0;
+    } else {
+      if (i == j) acc.x = -1.0;
+      for (int r = 0; r < n; ++r) fma_conj<double>(acc, V[r * n + i], V[r * n + j]);
+    }
     if (i == j) acc.y = 0.0;
     G[i * ldg + j] = acc;
     tri32(G, ldg, n, i, j)[0] =
@@ -311,7 +327,9 @@ __device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double*
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (n <= 128) {
+  if (oz) {
+    oz_correct(V, n, G, ldg, ex);
+  } else if (n <= 128) {
     // Q[r][j] = V[r][j] + sum_{i <= j} V[r][i] M[i][j], one warp per row, in place: lane l
     // forms the column pairs (j, n-1-j) for j = l and l + 32 (below n/2) in one pass of n + 1
     // products each (i = t for column j while t <= j, then i = t - j - 1 for column n-1-j),
@@ -429,7 +447,7 @@ __device__ int fp32_warm_start(const double2* RHO, double2* Vm, double2* X, int 
   }
   __syncthreads();
   mark(1);
-  const double emax = orthonormalise(Vm, n, X, ldr, scal);
+  const double emax = orthonormalise<false>(Vm, n, X, ldr, scal);
   if (threadIdx.x == 0 && !(emax < 1e-4)) atomicOr(flags, 1);  // FP32 basis too far from unitary
   mark(2);
   return sw32;
@@ -554,7 +572,7 @@ __device__ int eig_mixed(double2* RHO, double2* Vm, double2* X, int n, int D, do
         W64[idx] = make_double2((double)v.x, (double)v.y);
       }
       __syncthreads();
-      orthonormalise(W64, ns, Gw, ldb, scal);
+      orthonormalise<false>(W64, ns, Gw, ldb, scal);
       // rows of V and rho': X[r][cand] <- X[r][cand] W, then the columns of rho':
       // rho'[cand][c] <- W^dagger rho'[cand][c]; a row (column) per segment of seg >= ns
       // lanes, 32 / seg of them per warp, so that a small level does not leave most
@@ -1335,7 +1353,7 @@ __device__ void svd_levels(double2* Zt, int rows, double2* Vt, int n, double tr,
       W64[idx] = make_double2((double)v.x, (double)v.y);
     }
     __syncthreads();
-    orthonormalise(W64, ns, Gw, ns + 1, scal);
+    orthonormalise<false>(W64, ns, Gw, ns + 1, scal);
     // rows of Z (r < rows) and of V (x < n): new column cand[b] = sum_a old column cand[a] W[a][b]
     for (int rr = warp; rr < rows + (Vt ? n : 0); rr += nw) {
       double2* base = rr < rows ? Zt + rr : Vt + (rr - rows);
@@ -1471,8 +1489,8 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
     // Its columns are orthogonal to |E| ~ 1e-6; the series of `orthonormalise` is exact to
     // O(|E|^3), and its FP32 products to ~n |E|^2 1e-7.  A basis further off takes a second
     // pass, which starts from ~|E|^3; one beyond the series' range is flagged.
-    const double emax = orthonormalise(Vx, nv, Xs, nv + 1, scal);
-    const double emax2 = emax > 4e-6 ? orthonormalise(Vx, nv, Xs, nv + 1, scal) : 0.0;
+    const double emax = orthonormalise<true>(Vx, nv, Xs, nv + 1, scal, order);
+    const double emax2 = emax > 4e-6 ? orthonormalise<true>(Vx, nv, Xs, nv + 1, scal, order) : 0.0;
     if (threadIdx.x == 0 && (!(emax < 1e-2) || !(emax2 < 1e-8))) atomicOr(flags, 1);
   }
   mark(2);
