@@ -1375,6 +1375,69 @@ __device__ void svd_levels(double2* Zt, int rows, double2* Vt, int n, double tr,
   }
 }
 
+// One simultaneous correction of nearly orthogonal columns: Z <- Z (I + X + X^2 / 2), X
+// skew-Hermitian with the first-order angles X_pq = g_pq / (|z_q|^2 - |z_p|^2), g = Z^H Z, of
+// every pair whose angle is below kRefineAngle (the others, and columns at rounding,
+// are left to the sweeps).  The factor is unitary to |X|^4 / 4, at FP64 rounding; overlaps
+// of 1e-6 become ~1e-11 in one pass and 1e-16 in two, so the sweeps that follow find only
+// nearly degenerate pairs to rotate.  A full sweep costs 12 n^3 / 2 FP64 multiply-adds; here Z^H Z
+// and Z X are digit products on the tensor cores and X^2 / 2 (~1e-10) is FP32.
+// Columns are scaled to norms in [1, 2) by powers of two, so that every product is accurate relative to
+// its column.  n >= kOzMinBond; Z square; G [n][n+1], Y [n][n], X32 [n][n] scratch; ex: 2n ints.
+constexpr double kRefineAngle = 2e-5;
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+__device__ __noinline__ void svd_refine(double2* Zt, int n, double trace, double2* G, double2* Y, float2* X32,
+                                        double* alpha, int* expo, int* ex) {
+  const int ldg = n + 1;
+  column_norms(Zt, n, n, alpha);
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    const bool noise = !(alpha[j] > kNoiseRelSvd * trace);
+    const int e = noise ? 0 : (oz_exp(alpha[j]) - 1023) >> 1;
+    expo[j] = e;
+    alpha[j] = noise ? 0.0 : alpha[j] * pow2(-2 * e);
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) Zt[idx] = cscale(Zt[idx], pow2(-expo[idx / n]));
+  __syncthreads();
+  oz_product(Zt, n, 1, true, Zt, n, 1, ex, G, ldg, 1, n, true);
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
+    int i, j;
+    upper_index(idx, n, i, j);
+    double2 xij = make_double2(0.0, 0.0), xji = xij;
+    if (i < j && alpha[i] > 0.0 && alpha[j] > 0.0) {
+      const double2 g = G[i * ldg + j];
+      const double f = pow2(2 * (expo[j] - expo[i]));
+      const double r = 1.0 / fma(alpha[j], f, -alpha[i]);
+      if ((g.x * g.x + g.y * g.y) * (r * r * f) <= kRefineAngle * kRefineAngle) {
+        xij = cscale(g, r);
+        xji = cscale(cconj(g), -r * f);
+      }
+    }
+    Y[i * n + j] = xij;
+    X32[i * n + j] = make_float2((float)xij.x, (float)xij.y);
+    if (i < j) {
+      Y[j * n + i] = xji;
+      X32[j * n + i] = make_float2((float)xji.x, (float)xji.y);
+    }
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    const int i = idx / n, j = idx - (idx / n) * n;
+    float2 acc = make_float2(0.f, 0.f);
+    for (int k = 0; k < n; ++k) fma_c<float>(acc, X32[i * n + k], X32[k * n + j]);
+    Y[idx] = make_double2(fma(0.5, (double)acc.x, Y[idx].x), fma(0.5, (double)acc.y, Y[idx].y));
+  }
+  __syncthreads();
+  oz_product(Y, 1, n, false, Zt, 1, n, ex, G, ldg, 1, n, false);
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+    const int j = idx / n;
+    Zt[idx] = cscale(cadd(Zt[idx], G[j * ldg + idx - j * n]), pow2(expo[j]));
+  }
+  __syncthreads();
+}
+
 // Front half of the unsquared bond update (complex128): from the Gram blocks of
 // end a (FP64 sums in gsum, or this bond's partials) and end b, the right
 // singular vectors V (Vm [n][n], row x, column j) and squared singular values
@@ -1525,6 +1588,9 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
   // size).  Only then are the small columns a clean block for the FP32 levels,
   // whose rotations leave the last sweeps little to do.
   unsigned long long* rot = cycles ? cycles + kPhases + kRotSweeps : nullptr;
+  if (left && n >= kOzMinBond)
+    for (int pass = 0; pass < 2; ++pass)
+      svd_refine(Zt, n, trace, Xs, Vx, reinterpret_cast<float2*>(Mt), ev, reinterpret_cast<int*>(dsc), order);
   const int sw1 = os_sweeps(Zt, zr, Vt, n, jp.tol, jp.floor_rel * trace, trace, 1, ev, dsc, dinv, re, be, iflag,
                             sweeps_out + 4, rot);
   mark(4);

@@ -63,3 +63,17 @@ def test_a_warm_start_tolerance_out_of_range_is_brought_into_it(tol32):
 @pytest.mark.parametrize("D", [3, 4, 9, 23, 24, 31, 32, 33, 64, 65])
 def test_step_of_a_random_state(D):
     assert _step(D) <= 1e-10
+
+
+def _rank5(lam):
+    lam[:, 5:] = 0.0
+
+
+def _pairs(lam):
+    lam[:, 1::2] = lam[:, 0:-1:2]
+
+
+@pytest.mark.parametrize("D", [24, 32, 64])
+@pytest.mark.parametrize("spectrum", [_rank5, _pairs])
+def test_step_of_a_degenerate_state(D, spectrum):
+    assert _step(D, spectrum=spectrum) <= 1e-10
