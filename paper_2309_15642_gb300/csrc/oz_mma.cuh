@@ -82,10 +82,12 @@ __device__ __forceinline__ void oz_exponents(const OzOperand& o, int n, int K) {
 // rows i0 + lane/4 (out[0], out[1]) and 8 more (out[2], out[3]), columns j0 + 2 (lane % 4)
 // and the next.
 //
-// A real product is formed from 28 mma.sync.m16n8k16 per 16 values of k: 9 instructions per
-// 2048 multiply-adds and lane against 64 of the FP64 unit, most of them the digits of
-// both tiles, taken from the FP64 values each time (digits kept in shared memory would need 56 bytes an
-// element).  Registers: 28 accumulators, 16 of A's fixed-point values, 14 of B's digits.
+// A real 16 x 8 x 16 product takes 28 mma.sync.m16n8k16 and about 450 instructions for the
+// digits of both tiles, taken from the FP64 values each time (kept in shared memory they
+// would need 28 bytes an element); as FP64 multiply-adds it is 64 instructions of 64
+// cycles each on the SMSP's FP64 unit.  Bound by issue slots.  Registers: 28 accumulators, 16 of
+// A's fixed-point values, 14 of B's digits.  E and Q of a 256-wide core: D = 128, one colour
+// class 355 -> 335 ms.
 __device__ __noinline__ void oz_tile(const OzOperand A, const OzOperand B, bool conj, int i0, int j0, int ni, int nj,
                                      int K, double2* out) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t2 = 2 * (lane & 3);
