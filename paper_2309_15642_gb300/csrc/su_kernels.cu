@@ -864,12 +864,14 @@ __device__ __forceinline__ void os_rot(float a, float b, float2 g, float& c, flo
 // phases over the CTA.  One complex128 step of 127 + 433 + 1121 qubits at D = 32 54.9 -> 49.4 ms.
 // All of a lane's loads come before its sums, and t needs no exact divide or root: warm start of a 64-wide core 3.57 ->
 // 2.36 M cycles, of a 128-wide one 15.1 -> 8.7 M.
-__device__ __noinline__ int one_sided_jacobi32(float2* Bt, int ld, int rows, float2* Wt, int n, float tol, float floor_abs,
-                                  int max_sweeps, int* iflag, unsigned long long* work,
-                                  unsigned long long* rot_count) {
-  constexpr int kR = 8;  // entries of a column per lane
+// kR: entries of a column per lane, 8, or 2 for columns of at most 16, where six of the eight would
+// be padding (the same lanes and sums): 127 qubits, D = 4, 5 steps 2.05 -> 1.91 ms.
+template <int kR>
+__device__ __noinline__ int one_sided_rounds32(float2* Bt, int ld, int rows, float2* Wt, int n, float tol,
+                                               float floor_abs, int max_sweeps, int* iflag, unsigned long long* work,
+                                               unsigned long long* rot_count) {
   const int m = n / 2, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int L = rows <= 8 * kR ? 8 : rows <= 16 * kR ? 16 : 32;
+  const int L = rows <= 64 ? 8 : rows <= 128 ? 16 : 32;
   const int per = 32 / L, sub = lane & (L - 1), grp = lane / L;
   const float tol2 = tol * tol, floor2 = floor_abs * floor_abs;
   unsigned long long n_chk = 0, n_rot = 0;
@@ -955,6 +957,13 @@ __device__ __noinline__ int one_sided_jacobi32(float2* Bt, int ld, int rows, flo
     atomicAdd(work + 1, n_rot);
   }
   return result;
+}
+
+__device__ __forceinline__ int one_sided_jacobi32(float2* Bt, int ld, int rows, float2* Wt, int n, float tol,
+                                                  float floor_abs, int max_sweeps, int* iflag,
+                                                  unsigned long long* work, unsigned long long* rot_count) {
+  return rows <= 16 ? one_sided_rounds32<2>(Bt, ld, rows, Wt, n, tol, floor_abs, max_sweeps, iflag, work, rot_count)
+                    : one_sided_rounds32<8>(Bt, ld, rows, Wt, n, tol, floor_abs, max_sweeps, iflag, work, rot_count);
 }
 
 // FP64 sweeps of the one-sided Jacobi on the n columns of Z (Zt [n][rows]), with
