@@ -27,11 +27,10 @@
 // i + j.
 //
 //   oz_gram_kernel    one CTA per row tile (and spin, beyond D = 32): kicks the
-//       rows (writing them, unweighted, to `at` for the update, with the largest
-//       exponent of each row), weights them, and writes the tile's Gram blocks in
-//       FP64 (the partials of gram_kernel).
+//       rows (writing them, unweighted, to `at` for the update), weights them, and
+//       writes the tile's Gram blocks in FP64 (the partials of gram_kernel).
 //   oz_update_kernel  one CTA per 128 rows, spin and 32 new bond indices:
-//       Gamma_a'[s] = mask (Ã_s Y_s) from `at`.
+//       Gamma_a'[s] = mask (Ã_s Y_s) from `at`, the bond index balanced first.
 //
 // Included by su_kernels.cu after its row/element helpers.
 #pragma once
@@ -94,7 +93,7 @@ __global__ void oz_kick_kernel(const BondDesc* __restrict__ bonds, int n, const 
   cs[i] = make_double2(cos(h), sin(h));
 }
 
-// Slot of one row tile in `at`: Ã [s][row][re/im][k] (doubles), and of its largest exponents [s][row].
+// Slot of one row tile in `at`: Ã [s][row][re/im][k] (doubles).
 __device__ __forceinline__ int64_t oz_at(int part, int s, int row, int ri, int tr, int D) {
   return (int64_t)part * 4 * tr * D + ((int64_t)(s * tr + row) * 2 + ri) * D;
 }
@@ -108,21 +107,17 @@ template <int kMode>
 __global__ void __launch_bounds__(kOzThreads, 1)
     oz_gram_kernel(const TileDesc* __restrict__ tiles, const BondDesc* __restrict__ bonds,
                    const double2* __restrict__ gamma, const double* __restrict__ lam, const double2* __restrict__ cs,
-                   double2* __restrict__ partials, double* __restrict__ at, int* __restrict__ rexp, int* flags,
-                   int D) {
+                   double2* __restrict__ partials, double* __restrict__ at, int* flags, int D) {
   constexpr int Kt = kMode == 2 ? 32 : 64, kRows = kMode == 2 ? 256 : 128;
   constexpr uint32_t kSlice = kRows * Kt * 2, kSbo = Kt * 16;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int cmax[kMode == 2 ? 128 : 64], rmax[128];
+  __shared__ int cmax[kMode == 2 ? 128 : 64];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t tslot;
   const TileDesc t = tiles[blockIdx.x];
   const SideDesc sa = bonds[t.bond].a;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x < 128) {
-    if (threadIdx.x < (int)(sizeof(cmax) / 4)) cmax[threadIdx.x] = 0;
-    rmax[threadIdx.x] = 0;
-  }
+  if (threadIdx.x < (int)(sizeof(cmax) / 4)) cmax[threadIdx.x] = 0;
   const uint32_t tmem = tc_setup(&tslot, bars, 512);
   // rows of this warp: 8 rows from rg * 8, bond index k, spin s
   const int rg = kMode == 2 ? (warp & 3) : (warp & 7);
@@ -160,16 +155,12 @@ __global__ void __launch_bounds__(kOzThreads, 1)
           at[oz_at(t.part, s, r, 1, tr, D) + k] = a.y;
         }
       }
-      const int re = __reduce_max_sync(0xffffffffu, max(oz_exp(a.x), oz_exp(a.y)));
-      if (lane == 0 && re) atomicMax(rmax + (kMode == 0 ? s * 64 : 0) + r, re);
       x[i] = make_double2(a.x * w, a.y * w);
-      cm = max(cm, max(oz_exp(x[i].x), oz_exp(x[i].y)));
+      cm = max(cm, max(oz_row_exp(x[i].x), oz_row_exp(x[i].y)));
     }
     if (cm) atomicMax(cmax + (kMode == 0 ? s * 32 : 0) + k, cm);
   }
   __syncthreads();
-  if (threadIdx.x < (kMode == 0 ? 128 : tr))
-    rexp[(int64_t)t.part * 2 * tr + (kMode == 0 ? 0 : s * tr) + threadIdx.x] = rmax[threadIdx.x];
   {
     const int em = cmax[(kMode == 0 ? s * 32 : 0) + k];
 #pragma unroll
@@ -294,16 +285,74 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   tc_teardown(tmem, 512);
 }
 
+// Balance of the bond index in the update, per bond and spin (blockIdx.x, blockIdx.y).
+//
+// Y[k][k'] = lambda_k W[k][k'] / s_k', W formed in FP64 to eps of its row, and near the
+// canonical form Ã[r][k] grows like 1 / lambda_k in rows of small lambda on the other legs.
+// A digit holds 54 bits below its operand row's largest element, so k is balanced before the
+// split: Ã[.][k] 2^b_k, Y[k][.] 2^-b_k, b_k the exponent of max_k' |Y[k][k']| s_k' (exact,
+// integers added to exponents).  The error of an output is then 2^-54 of
+// max_k |Ã[r][k]| 2^b_k / s_k', which the rounding of W alone already makes.  Without it
+// the tensor loses digits like 1 / lambda_min: 9e-11 of a row's scale at 1e-6, 8e-7 at 1e-10.
+// Update of one class of 127 + 433 + 1121 qubits, D = 32: 1.26 -> 1.38 ms.
+//
+// Once per bond and spin: in each of the update's CTAs it would be three dependent passes of
+// loads.  bal: b_k [D], the largest exponents of Y's balanced columns [D].
+__device__ __forceinline__ int64_t oz_bal(int bond, int s, int D) { return ((int64_t)bond * 2 + s) * (2 * D + 1); }
+__global__ void __launch_bounds__(kThreads)
+    oz_balance_kernel(const BondDesc* __restrict__ bonds, const double* __restrict__ lam,
+                      const double2* __restrict__ Yall, int* __restrict__ balance, int D) {
+  __shared__ int snew[kMaxDc128], bal[kMaxDc128], ymax[kMaxDc128];
+  const int s = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kThreads / 32;
+  const double2* Y = Yall + ((int64_t)blockIdx.x * 2 + s) * D * D;
+  int* out = balance + oz_bal(blockIdx.x, s, D);
+  for (int k = threadIdx.x; k < D; k += kThreads) {
+    snew[k] = oz_exp(lam[bonds[blockIdx.x].lam_e + k]) - 2046;  // the bond's new lambda
+    ymax[k] = kOzNone;
+  }
+  __syncthreads();
+  for (int k = warp; k < D; k += nw) {
+    int e = kOzNone;
+    for (int kp = lane; kp < D; kp += 32) {
+      const double2 y = Y[k * D + kp];
+      const int ey = max(oz_exp(y.x), oz_exp(y.y));
+      if (ey) e = max(e, ey + snew[kp]);
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) bal[k] = e;
+  }
+  __syncthreads();
+  for (int kp = lane; kp < D; kp += 32) {
+    int e = kOzNone;
+    for (int k = warp; k < D; k += nw) {
+      const double2 y = Y[k * D + kp];
+      const int ey = max(oz_row_exp(y.x), oz_row_exp(y.y));
+      if (ey) e = max(e, ey >= kOzNan ? 2 * kOzNan : ey - bal[k]);
+    }
+    atomicMax(ymax + kp, e);
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < D; k += kThreads) {
+    out[k] = bal[k];
+    out[D + k] = ymax[k];
+  }
+}
+
 // Rows [row0, row0 + 128) of end a, spin blockIdx.y, new bond indices [32 blockIdx.z, +32):
 // Gamma_a'[s][r][k'] = mask_r sum_k Ã_s[r][k] Y_s[k][k'] as a real product over K = (re/im, k),
 // 32 k at a time: M = 128 rows, N = (re/im, k') = 64.  Launched over the row tiles; the tiles
 // that do not start a 128-row block return at once.
+//
+// kMore: beyond D = 64, where the accumulators (exact to 128 K values) are read and added up
+// after every second chunk; up to there once, after the last.
+template <bool kMore>
 __global__ void __launch_bounds__(kOzThreads, 1)
     oz_update_kernel(const TileDesc* __restrict__ tiles, const BondDesc* __restrict__ bonds, double2* gamma,
                      const double* __restrict__ lam, const double2* __restrict__ Yall, const double* __restrict__ at,
-                     const int* __restrict__ rexp, int* flags, int D) {
+                     const int* __restrict__ balance, int* flags, int D) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int ymax[32];
+  constexpr int kPad = kMore ? kMaxDc128 : 64;
+  __shared__ int ymax[32], rmax[128], bal[kPad];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t tslot;
   __shared__ float mask[128];
@@ -316,79 +365,88 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   const int nrows = sa.rows - t.row0 < 128 ? sa.rows - t.row0 : 128;
   const int tr = tile_rows(D, 16);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x < 32) ymax[threadIdx.x] = 0;
+  const int* plan = balance + oz_bal(t.bond, s, D);
+  if (threadIdx.x < 32) ymax[threadIdx.x] = kp0 + threadIdx.x < D ? plan[D + kp0 + threadIdx.x] : kOzNone;
+  if (threadIdx.x < kPad) bal[threadIdx.x] = threadIdx.x < D ? plan[threadIdx.x] : kOzNone;
   const uint32_t tmem = tc_setup(&tslot, bars, 512);
   tc_row_mask<false>(sa, lam, t.row0, nrows, D, mask, cut);
-  {
-    int e = 0;
-    if (kp0 + lane < D)
-      for (int k = warp; k < D; k += 16) {
-        const double2 y = Y[k * D + kp0 + lane];
-        e = max(e, max(oz_exp(y.x), oz_exp(y.y)));
+  // left operand: 8 rows x 4 groups of 8 k per warp and part (re, im); from the last chunk of
+  // 32 k down for the rows' exponents, so that the first is in registers when its digits follow
+  const int nchunk = (D + 31) / 32;
+  const int ra = warp * 8 + (lane & 7), kg = lane >> 3;
+  const double* arow = at + oz_at(t.part + ra / tr, s, ra % tr, 0, tr, D) + kg * 8;
+  double a[2][8];
+  auto load = [&](int ch) {
+    const int left = ra < nrows ? D - 32 * ch - kg * 8 : 0;
+#pragma unroll
+    for (int ri = 0; ri < 2; ++ri) {
+      const double* src = arow + ri * D + 32 * ch;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) a[ri][e] = 0.0;
+      if ((D & 7) == 0 && left > 0) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const double2 d = *reinterpret_cast<const double2*>(src + 2 * e);
+          a[ri][2 * e] = d.x;
+          a[ri][2 * e + 1] = d.y;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if (e < left) a[ri][e] = src[e];
       }
-    if (e) atomicMax(ymax + lane, e);
+    }
+  };
+  int em = kOzNone;
+  for (int ch = nchunk - 1; ch >= 0; --ch) {
+    load(ch);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int ea = max(oz_row_exp(a[0][e]), oz_row_exp(a[1][e]));
+      if (ea) em = max(em, ea >= kOzNan ? 2 * kOzNan : ea + bal[32 * ch + kg * 8 + e]);
+    }
   }
+  em = max(em, __shfl_xor_sync(0xffffffffu, em, 8));
+  em = max(em, __shfl_xor_sync(0xffffffffu, em, 16));
+  if (kg == 0) rmax[ra] = em;
   __syncthreads();
   unsigned char* sb = smem_raw + kOzOperand;
   constexpr uint32_t kSa = 128 * 64 * 2, kSb = 64 * 64 * 2, kSbo = 64 * 16;
   const uint32_t abase = tc::smem_u32(smem_raw), bbase = tc::smem_u32(sb);
-  const int nchunk = (D + 31) / 32;
   const int m = 32 * (warp & 3) + lane, q0 = 8 * (warp >> 2);
   const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)q0;
   long long ar[8], ai[8];
+  if (kMore)
 #pragma unroll
-  for (int q = 0; q < 8; ++q) ar[q] = ai[q] = 0;
+    for (int q = 0; q < 8; ++q) ar[q] = ai[q] = 0;
   uint32_t phase = 0;
   bool ok = true;
   for (int ch = 0; ch < nchunk && ok; ++ch) {
     const int k0 = 32 * ch;
-    // left operand: 8 rows x 4 groups of 8 k per warp and part (re, im)
+    if (ch) load(ch);
 #pragma unroll
     for (int ri = 0; ri < 2; ++ri) {
-      const int r = warp * 8 + (lane & 7), kg = lane >> 3, kk = k0 + kg * 8;
       unsigned long long v[8];
-      double a[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) a[e] = 0.0;
-      int em = 0;
-      if (r < nrows) {
-        const int part = t.part + r / tr, rr = r % tr;
-        em = rexp[(int64_t)part * 2 * tr + s * tr + rr];
-        const double* src = at + oz_at(part, s, rr, ri, tr, D) + kk;
-        if ((D & 7) == 0 && kk < D) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const double2 d = *reinterpret_cast<const double2*>(src + 2 * e);
-            a[2 * e] = d.x;
-            a[2 * e + 1] = d.y;
-          }
-        } else {
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            if (kk + e < D) a[e] = src[e];
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = oz_fixed(a[e], em);
+      for (int e = 0; e < 8; ++e) v[e] = oz_fixed(a[ri][e], em - bal[k0 + kg * 8 + e]);
       oz_store(smem_raw + warp * kSbo + (ri * 4 + kg) * 128 + (lane & 7) * 16, kSa, v);
     }
     // right operand: row n = (ro, k'), K = (ri, k): ro = ri -> yr; (0, 1) -> -yi; (1, 0) -> yi
     {
-      const int ro = warp >> 3, ri = (warp >> 2) & 1, kp = (warp & 3) * 8 + (lane & 7), kg = lane >> 3;
-      const int em = ymax[kp];
+      const int ro = warp >> 3, ri = (warp >> 2) & 1, kp = (warp & 3) * 8 + (lane & 7), ey = ymax[kp];
       unsigned long long v[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int k = k0 + kg * 8 + e;
         double2 y = make_double2(0.0, 0.0);
         if (k < D && kp0 + kp < D) y = Y[k * D + kp0 + kp];
-        v[e] = oz_fixed(ro == ri ? y.x : y.y, em, ro < ri);
+        v[e] = oz_fixed(ro == ri ? y.x : y.y, ey + bal[k], ro < ri);
       }
       oz_store(sb + (uint32_t)(ro * 4 + (warp & 3)) * kSbo + (ri * 4 + kg) * 128 + (lane & 7) * 16, kSb, v);
     }
     tc::fence_async_smem();
     __syncthreads();
-    const bool fresh = (ch & 1) == 0;
+    const bool fresh = kMore ? (ch & 1) == 0 : ch == 0;
     if (threadIdx.x == 0) {
       tc::fence_after_sync();
       for (int ks = 0; ks < 4; ++ks)
@@ -401,8 +459,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       tc::mma_commit(bars);
     }
     ok = oz_wait(bars, phase);
-    // exact to 128 K values: read the accumulators after every second chunk
-    if (ok && (!fresh || ch + 1 == nchunk)) {
+    if (ok && ((kMore && !fresh) || ch + 1 == nchunk)) {
       long long hr[8], hi[8], lr[8], li[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) hr[q] = hi[q] = lr[q] = li[q] = 0;
@@ -421,16 +478,15 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       }
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        ar[q] += hr[q] * 65536 + (lr[q] >> 8);
-        ai[q] += hi[q] * 65536 + (li[q] >> 8);
+        ar[q] = (kMore ? ar[q] : 0) + hr[q] * 65536 + (lr[q] >> 8);
+        ai[q] = (kMore ? ai[q] : 0) + hi[q] * 65536 + (li[q] >> 8);
       }
       tc::fence_before_sync();
     }
     __syncthreads();
   }
   if (ok && m < nrows) {
-    const int part = t.part + m / tr, rr = m % tr;
-    const int em = rexp[(int64_t)part * 2 * tr + s * tr + rr];
+    const int er = rmax[m];
     const bool cut_row = mask[m] == 0.f;
     const RowPos p = row_pos(sa, t.row0 + m);
 #pragma unroll
@@ -438,7 +494,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       const int kp = kp0 + q0 + q;
       if (kp < D) {
         const int ey = ymax[q0 + q];
-        double2 v = make_double2(oz_value(ar[q], em, ey), oz_value(ai[q], em, ey));
+        double2 v = make_double2(oz_value(ar[q], er, ey), oz_value(ai[q], er, ey));
         if (cut_row) v = cscale(v, 0.0);
         gamma[elem(sa, s, p, kp)] = v;
       }

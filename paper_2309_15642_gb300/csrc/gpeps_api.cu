@@ -74,7 +74,7 @@ struct gpeps_handle {
   size_t s_lam = 0, s_gamma = 0;
   size_t w_pending = 0, w_flags = 0, w_sweeps = 0, w_cycles = 0, w_queue = 0, w_z = 0, w_mean = 0, w_sites = 0, w_inst_site0 = 0,
          w_site_inst = 0, w_site_off = 0, w_partials = 0, w_Y = 0, w_theta_a = 0, w_bond_scratch = 0;
-  size_t w_at = 0, w_rexp = 0, w_cs = 0;  // complex128 tensor-core passes
+  size_t w_at = 0, w_balance = 0, w_cs = 0;  // complex128 tensor-core passes
   size_t bond_slot = 0;  // bytes per bond-kernel CTA of global scratch for its n x n matrices
   int bond_slots = 0;    // slots in the work buffer
   char* d_state = nullptr;
@@ -112,7 +112,7 @@ struct gpeps_handle {
   bool oz() const { return elt == 16 && OzPass::supported(D); }
   bool fused() const { return schedule >= 4 && !oz(); }
   OzPass::Scratch oz_scratch() const {
-    return OzPass::Scratch{at<double>(w_at), at<int>(w_rexp), d_work + w_cs};
+    return OzPass::Scratch{at<double>(w_at), at<int>(w_balance), d_work + w_cs};
   }
   template <typename P>
   P* at(size_t off) const {
@@ -296,7 +296,8 @@ int layer_impl(gpeps_handle* h, int c, PhaseEvents* pe = nullptr, void* vsave = 
                           h->d_work + h->w_bond_scratch, layered_per_sm(h, nbd)));
   if (pe) GP_CUDA(cudaEventRecord(pe->ev[2], h->stream));
   if (h->oz())
-    GP_CUDA(OzPass::update(tiles, nt, bonds, h->gamma(), h->lam(), Y, h->oz_scratch(), h->flags(), h->D, h->stream));
+    GP_CUDA(OzPass::update(tiles, nt, bonds, nbd, h->gamma(), h->lam(), Y, h->oz_scratch(), h->flags(), h->D,
+                           h->stream));
   else if (h->tensor)
     GP_CUDA(Launch<T>::update_tc(bonds, nbd, h->gamma(), h->lam(), Y, theta_a, h->flags(), h->D, h->stream));
   else
@@ -541,7 +542,7 @@ int gpeps_create(const gpeps_graph* graphs, int32_t n_instances, int32_t D, int3
   h->w_theta_a = carve((size_t)h->max_bonds * sizeof(double));
   if (h->oz()) {
     h->w_at = carve((size_t)h->max_parts * OzPass::at_doubles(D) * sizeof(double));
-    h->w_rexp = carve((size_t)h->max_parts * OzPass::rexp_ints(D) * sizeof(int));
+    h->w_balance = carve((size_t)h->max_bonds * OzPass::balance_ints(D) * sizeof(int));
     h->w_cs = carve((size_t)h->max_bonds * sizeof(double2));
   }
   // n x n bond matrices outside shared memory (a CTA indexes its slot by

@@ -168,18 +168,18 @@ struct Launch {
 struct OzPass {
   struct Scratch {
     double* at;   // kicked rows of end a, one slot of at_doubles per row tile
-    int* rexp;    // largest exponent of each of them, one slot of rexp_ints per row tile
+    int* balance; // of the bond index in the update, balance_ints per bond
     void* cs;     // cos and sin of half the kick of end a, two doubles per bond
   };
   static constexpr bool supported(int D) { return D >= kOzMinD && D <= kMaxDc128; }
+  static size_t balance_ints(int D) { return (size_t)2 * (2 * D + 1); }
   static size_t at_doubles(int D) { return (size_t)4 * tile_rows(D, 16) * D; }
-  static size_t rexp_ints(int D) { return (size_t)2 * tile_rows(D, 16); }
   static cudaError_t init();
   static cudaError_t gram(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, int n_bonds, const void* gamma,
                           const double* lam, const double* pending, void* partials, const Scratch& ws, int* flags,
                           int D, cudaStream_t st);
-  static cudaError_t update(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, void* gamma, const double* lam,
-                            const void* Y, const Scratch& ws, int* flags, int D, cudaStream_t st);
+  static cudaError_t update(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, int n_bonds, void* gamma,
+                            const double* lam, const void* Y, const Scratch& ws, int* flags, int D, cudaStream_t st);
 };
 
 constexpr int kMaxGradD = 16;  // bond dimension limit of the reverse mode (shared memory of its bond kernel)

@@ -16,6 +16,14 @@ constexpr int kOzSlices = 7;
 
 __device__ __forceinline__ int oz_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
+// Row exponents: kOzNan marks a row that holds a value that is not finite, kOzNone (or
+// any exponent more than 55 below the others') one that holds nothing.
+constexpr int kOzNan = 1 << 16, kOzNone = -(1 << 16);
+__device__ __forceinline__ int oz_row_exp(double x) {
+  const int e = oz_exp(x);
+  return e == 0x7ff ? kOzNan : e;
+}
+
 // Biased fixed point: round(x 2^(54 - E)) + 0x80 in each of the 7 digit bytes, E =
 // em - 1022 for the row's largest biased exponent em: byte 6 - i minus 128 is d_i.
 __device__ __forceinline__ unsigned long long oz_fixed(double x, int em, bool negate = false) {
@@ -31,7 +39,7 @@ __device__ __forceinline__ unsigned long long oz_fixed(double x, int em, bool ne
 // t 2^(ea + eb - 2044 - 52) rounded to FP64 (ea, eb: biased exponents of the two rows);
 // NaN when a row held a value that is not finite.
 __device__ __forceinline__ double oz_value(long long t, int ea, int eb) {
-  if (ea == 0x7ff || eb == 0x7ff) return __longlong_as_double(0x7ff8000000000000ll);
+  if (ea >= kOzNan || eb >= kOzNan) return __longlong_as_double(0x7ff8000000000000ll);
   const unsigned long long u = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
   if (u == 0) return 0.0;
   const int n = __clzll((long long)u);
@@ -74,7 +82,7 @@ __device__ __forceinline__ void oz_exponents(const OzOperand& o, int n, int K) {
       const int i = o.sk == 1 ? u : w, k = o.sk == 1 ? w : u;
       if (o.tri && k > i) continue;
       const double2 x = *o.elem(i, k);
-      atomicMax(o.e + i, max(oz_exp(x.x), oz_exp(x.y)));
+      atomicMax(o.e + i, max(oz_row_exp(x.x), oz_row_exp(x.y)));
     }
 }
 

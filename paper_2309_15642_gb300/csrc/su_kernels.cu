@@ -2787,7 +2787,9 @@ cudaError_t OzPass::init() {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(oz_gram_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzGramSmem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(oz_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzUpdateSmem);
+  e = cudaFuncSetAttribute(oz_update_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzUpdateSmem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(oz_update_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzUpdateSmem);
 }
 
 cudaError_t OzPass::gram(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, int n_bonds, const void* gamma,
@@ -2800,22 +2802,25 @@ cudaError_t OzPass::gram(const TileDesc* tiles, int n_tiles, const BondDesc* bon
   const double2* g = static_cast<const double2*>(gamma);
   double2* out = static_cast<double2*>(partials);
   if (D <= 32)
-    oz_gram_kernel<0><<<n_tiles, kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, ws.rexp, flags, D);
+    oz_gram_kernel<0><<<n_tiles, kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, flags, D);
   else if (D <= 64)
-    oz_gram_kernel<1><<<dim3(n_tiles, 2), kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, ws.rexp,
-                                                                          flags, D);
+    oz_gram_kernel<1><<<dim3(n_tiles, 2), kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, flags,
+                                                                          D);
   else
-    oz_gram_kernel<2><<<dim3(n_tiles, 2), kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, ws.rexp,
-                                                                          flags, D);
+    oz_gram_kernel<2><<<dim3(n_tiles, 2), kOzThreads, kOzGramSmem, st>>>(tiles, bonds, g, lam, cs, out, ws.at, flags,
+                                                                          D);
   return cudaGetLastError();
 }
 
-cudaError_t OzPass::update(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, void* gamma, const double* lam,
-                           const void* Y, const Scratch& ws, int* flags, int D, cudaStream_t st) {
+cudaError_t OzPass::update(const TileDesc* tiles, int n_tiles, const BondDesc* bonds, int n_bonds, void* gamma,
+                           const double* lam, const void* Y, const Scratch& ws, int* flags, int D, cudaStream_t st) {
   if (n_tiles == 0) return cudaSuccess;
   if (!supported(D)) return cudaErrorInvalidValue;
-  oz_update_kernel<<<dim3(n_tiles, 2, (D + 31) / 32), kOzThreads, kOzUpdateSmem, st>>>(
-      tiles, bonds, static_cast<double2*>(gamma), lam, static_cast<const double2*>(Y), ws.at, ws.rexp, flags, D);
+  const double2* y = static_cast<const double2*>(Y);
+  oz_balance_kernel<<<dim3(n_bonds, 2), kThreads, 0, st>>>(bonds, lam, y, ws.balance, D);
+  auto kernel = D > 64 ? oz_update_kernel<true> : oz_update_kernel<false>;
+  kernel<<<dim3(n_tiles, 2, (D + 31) / 32), kOzThreads, kOzUpdateSmem, st>>>(
+      tiles, bonds, static_cast<double2*>(gamma), lam, y, ws.at, ws.balance, flags, D);
   return cudaGetLastError();
 }
 
