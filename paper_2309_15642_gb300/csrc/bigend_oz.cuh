@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 // Update of one class of 127 + 433 + 1121 qubits, D = 32: 1.26 -> 1.38 ms.
 //
 // Once per bond and spin: in each of the update's CTAs it would be three dependent passes of
-// loads.  bal: b_k [D], the largest exponents of Y's balanced columns [D].
+// loads.  bal: b_k [D], the largest exponents of Y's balanced columns [D], and whether Y = I.
 __device__ __forceinline__ int64_t oz_bal(int bond, int s, int D) { return ((int64_t)bond * 2 + s) * (2 * D + 1); }
 __global__ void __launch_bounds__(kThreads)
     oz_balance_kernel(const BondDesc* __restrict__ bonds, const double* __restrict__ lam,
@@ -311,17 +311,20 @@ __global__ void __launch_bounds__(kThreads)
     ymax[k] = kOzNone;
   }
   __syncthreads();
+  bool one = true;
   for (int k = warp; k < D; k += nw) {
     int e = kOzNone;
     for (int kp = lane; kp < D; kp += 32) {
       const double2 y = Y[k * D + kp];
       const int ey = max(oz_exp(y.x), oz_exp(y.y));
+      one = one && __double2hiint(y.x) == (k == kp ? 0x3ff00000 : 0) &&
+            (__double2loint(y.x) | __double2hiint(y.y) | __double2loint(y.y)) == 0;
       if (ey) e = max(e, ey + snew[kp]);
     }
     e = __reduce_max_sync(0xffffffffu, e);
     if (lane == 0) bal[k] = e;
   }
-  __syncthreads();
+  one = __syncthreads_and(one);
   for (int kp = lane; kp < D; kp += 32) {
     int e = kOzNone;
     for (int k = warp; k < D; k += nw) {
@@ -336,12 +339,15 @@ __global__ void __launch_bounds__(kThreads)
     out[k] = bal[k];
     out[D + k] = ymax[k];
   }
+  if (threadIdx.x == 0) out[2 * D] = one;
 }
 
 // Rows [row0, row0 + 128) of end a, spin blockIdx.y, new bond indices [32 blockIdx.z, +32):
 // Gamma_a'[s][r][k'] = mask_r sum_k Ã_s[r][k] Y_s[k][k'] as a real product over K = (re/im, k),
 // 32 k at a time: M = 128 rows, N = (re/im, k') = 64.  Launched over the row tiles; the tiles
 // that do not start a 128-row block return at once.
+//
+// Y = I (a bond that bond_fail leaves as it was) copies the kicked rows unrounded.
 //
 // kMore: beyond D = 64, where the accumulators (exact to 128 K values) are read and added up
 // after every second chunk; up to there once, after the last.
@@ -370,6 +376,18 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   if (threadIdx.x < kPad) bal[threadIdx.x] = threadIdx.x < D ? plan[threadIdx.x] : kOzNone;
   const uint32_t tmem = tc_setup(&tslot, bars, 512);
   tc_row_mask<false>(sa, lam, t.row0, nrows, D, mask, cut);
+  if (plan[2 * D]) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < nrows * 32; i += kOzThreads) {
+      const int r = i >> 5, kp = kp0 + lane;
+      if (kp >= D) continue;
+      const int64_t src = oz_at(t.part + r / tr, s, r % tr, 0, tr, D) + kp;
+      const double2 v = make_double2(at[src], at[src + D]);
+      gamma[elem(sa, s, row_pos(sa, t.row0 + r), kp)] = mask[r] == 0.f ? cscale(v, 0.0) : v;
+    }
+    tc_teardown(tmem, 512);
+    return;
+  }
   // left operand: 8 rows x 4 groups of 8 k per warp and part (re, im); from the last chunk of
   // 32 k down for the rows' exponents, so that the first is in registers when its digits follow
   const int nchunk = (D + 31) / 32;

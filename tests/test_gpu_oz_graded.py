@@ -75,3 +75,26 @@ def test_graded_tensor_keeps_its_digits(D, lam_min):
     scale = (np.abs(A) * (lam * np.sqrt((np.abs(F) ** 2).sum((0, 2))))).sum(2)  # [s][r]
     err = np.abs(A1[:, :, on] - ref) * s[on] / scale[:, :, None]
     assert err.max() <= 1e-12
+
+
+@pytest.mark.parametrize("D", [17, 33, 65])
+def test_failed_bond_leaves_the_larger_end_unrounded(D):
+    """A bond whose core is not finite keeps its tensors; only the pending kick of the larger end is
+    applied, two multiply-adds an element whatever the rest of its row holds."""
+    rng = np.random.default_rng(D)
+    g0 = _random(rng, 2, D, D, D) * 10.0 ** rng.uniform(-30, 0, (2, D, D, D))
+    g1 = _random(rng, 2, D, D)
+    g1[0, 1, 2] = np.nan
+    lam = np.linspace(1.0, 0.5, D)
+    lam0 = np.where(np.arange(D) < D // 2, lam, 0.0)
+    for th in (0.0, 0.7):
+        g = _handle(D, {0: g0, 1: g1}, {0: lam0, 1: lam, 2: lam, 3: lam})
+        g.kick(torch.tensor([th], dtype=torch.float64, device="cuda"))
+        g.zz_layer(0)
+        assert g.status() == 2
+        got, ref = g.site_tensor(0, 0)[0].cpu().numpy(), _kick(g0, th)
+        assert np.array_equal(g.lambda_tensor(0, 0).cpu().numpy(), lam0)
+        g.close()
+        part = np.abs(g0) + np.abs(g0[::-1])  # an element's two terms
+        assert (np.abs(got - ref) <= 4 * EPS * part).all()
+        assert th or np.array_equal(got, g0)
