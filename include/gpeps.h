@@ -450,6 +450,14 @@ int gpeps_bond_update_noalloc(int32_t D, int32_t dtype, void* gamma_a, int32_t d
  */
 int gpeps_selftest_rotation(int32_t which, int32_t n, const double* in, double* out, void* stream);
 
+/*
+ * Diagnostic: a step of the complex128 bond SVD on its own, by one CTA.  Arrays are device
+ * complex128, n x n row-major, n even, 2 to 256.  which 0: the integer digit product of the
+ * bond core, out[i][j] = sum_k conj(a[i][k]) b[j][k].  Asynchronous on stream.  Errors:
+ * GPEPS_EINVAL for another `which` or n, or a NULL array; GPEPS_ECUDA for a failed launch.
+ */
+int gpeps_selftest_core(int32_t which, int32_t n, const double* a, const double* b, double* out, void* stream);
+
 int gpeps_destroy(gpeps_handle* h);
 const char* gpeps_error_string(int status);
 const char* gpeps_last_cuda_error(void);

@@ -13,12 +13,18 @@
 // exact in f16, their products and the FP32 sums of up to 7 x 128 of them are
 // below 2^24, so every accumulator is an exact integer whatever the order:
 //
-//   sum_k x_k y_k = 2^(Ex+Ey-12) sum_{l=0..6} 2^(-8 l) v_l,  v_l = sum_{i+j=l} sum_k d_i(x_k) d_j(y_k).
+//   sum_k x_k y_k = 2^(Ex+Ey-12) sum_{l=0..7} 2^(-8 l) v_l,  v_l = sum_{i+j=l} sum_k d_i(x_k) d_j(y_k).
 //
-// The levels l > 6 are below 2^-54 of the row maxima's product.  The seven v_l of
-// an output are combined in a 64-bit integer of unit 2^(Ex+Ey-52) and rounded
-// once to FP64.  An FP64 sum of K products rounds K times at 2^-53, so the result
-// is at least as accurate against the row maxima.
+// The eight v_l of an output are combined in a 64-bit integer of unit 2^(Ex+Ey-53), to
+// nearest, and rounded once to FP64.  Error of a sum of K products, in units of
+// 2^(Ex+Ey): K 2^-54 from the 54 bits of x and y, 5 K 2^-62 from the levels l > 7 that
+// are left out, 2^-54 from the combination.  Over Gaussian rows it is 0.41, 0.53 and 0.64
+// x 2^-53 rms for K = 16, 64 and 128; a chain of FP64 multiply-adds makes 0.58, 1.25 and
+// 2.47 (seven levels and a low part cut off rather than rounded made 1.9, 3.6 and 5.1, with a
+// mean of -0.9, in 28 digit products instead of 34; one class of 127 + 433 + 1121 qubits, D = 32:
+// Gram 1.95 -> 2.07, bonds 11.3 -> 11.4, update 1.39 -> 1.58 ms).  Against the terms themselves it is an FP64 sum's only as far as they are within a few bits of the row
+// maxima: the passes scale their operands for that (the Gram's columns are summed over rows
+// against their own norms, the update balances k).
 //
 // The digits of a double cost about 30 integer instructions and no FP64 one.
 // Slices are stored as K-major operands without swizzle, slice after slice, so
@@ -75,6 +81,9 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
                : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// Slice i is the first to add to level l (its seven slices j reach level 7 from i = 1 on).
+__device__ __forceinline__ bool oz_first(int i, int l) { return i == (l == kOzLevels - 1 ? 1 : 0); }
 
 // Commit the issued products and wait (bounded) for them; the outcome is uniform over the CTA.
 __device__ __forceinline__ bool oz_wait(uint64_t* bar, uint32_t& phase) {
@@ -175,26 +184,24 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   tc::fence_async_smem();
   __syncthreads();
   const uint32_t base = tc::smem_u32(smem_raw);
-  // levels [l0, l1) of product `prod` into the accumulators at column (l - l0) * 128
-  auto issue = [&](int prod, int l0, int l1) {
+  // levels [l0, l0 + 4) of product `prod` into the accumulators at column (l - l0) * 128
+  auto issue = [&](int prod, int l0) {
     if (threadIdx.x != 0) return;
     tc::fence_after_sync();
     for (int ks = 0; ks < Kt / 16; ++ks) {
       auto desc = [&](int slice, int row) {
         return tc::smem_desc(base + slice * kSlice + (uint32_t)(row >> 3) * kSbo + ks * 256, 128, kSbo);
       };
-      for (int i = 0; i < l1; ++i) {
-        const int j0 = l0 > i ? l0 - i : 0, j1 = l1 - i;  // j0 <= j < j1
-        if (kMode == 2) {
-          for (int j = j0; j < j1; ++j) {
-            const uint32_t d = tmem + (uint32_t)(i + j - l0) * 128u;
-            mma_f16(d, desc(i, 0), desc(j, prod ? 128 : 0), 128, ks || i ? 1u : 0u);
-            if (!prod) mma_f16(d, desc(i, 128), desc(j, 128), 128, 1u);
-          }
-        } else {
-          for (int j = j0; j < j1; j += 2)
-            mma_f16(tmem + (uint32_t)(i + j - l0) * 128u, desc(i, 0), desc(j, 0), j + 1 < j1 ? 256 : 128,
-                    ks || i ? 1u : 0u);
+      for (int i = 0; i < min(l0 + 4, kOzSlices); ++i) {
+        const int j1 = min(l0 + 4 - i, kOzSlices);
+        for (int j = max(l0 - i, 0); j < j1;) {
+          const uint32_t d = tmem + (uint32_t)(i + j - l0) * 128u;
+          const bool first = !ks && oz_first(i, i + j);  // these accumulators hold nothing yet
+          // two slices j at once where both accumulators are in the same state
+          const int w = kMode != 2 && j + 1 < j1 && first == (!ks && oz_first(i, i + j + 1)) ? 2 : 1;
+          mma_f16(d, desc(i, 0), desc(j, kMode == 2 && prod ? 128 : 0), 128 * w, first ? 0u : 1u);
+          if (kMode == 2 && !prod) mma_f16(d, desc(i, 128), desc(j, 128), 128, 1u);
+          j += w;
         }
       }
     }
@@ -209,7 +216,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   double2* out = partials + (int64_t)t.part * 2 * D2;
   for (int prod = 0; prod < (kMode == 2 ? 2 : 1) && ok; ++prod) {
     long long acc[32];
-    issue(prod, 0, 4);
+    issue(prod, 0);
     ok = oz_wait(bars, phase);
     if (!ok) break;
 #pragma unroll
@@ -222,29 +229,27 @@ __global__ void __launch_bounds__(kOzThreads, 1)
       for (int q = 0; q < 8; ++q) {
         long long h = 0;
 #pragma unroll
-        for (int l = 0; l < 4; ++l)
-          h += (long long)__float2int_rn(__uint_as_float(v[l][q])) * (1ll << (8 * (3 - l)));
-        acc[8 * b + q] = h * 65536;
+        for (int l = 0; l < 4; ++l) h += oz_weigh(__uint_as_float(v[l][q]), l);
+        acc[8 * b + q] = h;
       }
     }
     tc::fence_before_sync();
     __syncthreads();
-    issue(prod, 4, 7);
+    issue(prod, 4);
     ok = oz_wait(bars, phase);
     if (!ok) break;
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-      uint32_t v[3][8];
+      uint32_t v[4][8];
 #pragma unroll
-      for (int l = 0; l < 3; ++l) tmem_ld8(tq + l * 128 + b * 8, v[l]);
+      for (int l = 0; l < 4; ++l) tmem_ld8(tq + l * 128 + b * 8, v[l]);
       tmem_ld_wait();
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        long long h = 0;
+        long long low = 0;
 #pragma unroll
-        for (int l = 0; l < 3; ++l)
-          h += (long long)__float2int_rn(__uint_as_float(v[l][q])) * (1ll << (8 * (2 - l)));
-        acc[8 * b + q] += h >> 8;
+        for (int l = 0; l < 4; ++l) low += oz_weigh(__uint_as_float(v[l][q]), l);
+        acc[8 * b + q] = oz_sum(acc[8 * b + q], low);
       }
     }
     tc::fence_before_sync();
@@ -468,12 +473,18 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     if (threadIdx.x == 0) {
       tc::fence_after_sync();
       for (int ks = 0; ks < 4; ++ks)
-        for (int i = 0; i < kOzSlices; ++i)
-          for (int j = 0; j < kOzSlices - i; j += 4) {
-            const int cnt = kOzSlices - i - j < 4 ? kOzSlices - i - j : 4;
+        for (int i = 0; i < kOzSlices; ++i) {
+          const int j1 = min(kOzLevels - i, kOzSlices);
+          for (int j = 0; j < j1;) {
+            // up to four slices j at once, level 7 by itself where its accumulators hold nothing yet
+            const bool start = fresh && !ks, first = start && oz_first(i, i + j);
+            int w = min(j1 - j, 4);
+            if (start && i == 1 && i + j + w == kOzLevels && w > 1) --w;
             mma_f16(tmem + (uint32_t)(i + j) * 64u, tc::smem_desc(abase + i * kSa + ks * 256, 128, kSbo),
-                    tc::smem_desc(bbase + j * kSb + ks * 256, 128, kSbo), 64 * cnt, fresh && !ks && !i ? 0u : 1u);
+                    tc::smem_desc(bbase + j * kSb + ks * 256, 128, kSbo), 64 * w, first ? 0u : 1u);
+            j += w;
           }
+        }
       tc::mma_commit(bars);
     }
     ok = oz_wait(bars, phase);
@@ -482,22 +493,21 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
       for (int q = 0; q < 8; ++q) hr[q] = hi[q] = lr[q] = li[q] = 0;
 #pragma unroll
-      for (int l = 0; l < kOzSlices; ++l) {
+      for (int l = 0; l < kOzLevels; ++l) {
         uint32_t vr[8], vi[8];
         tmem_ld8(tq + l * 64, vr);
         tmem_ld8(tq + l * 64 + 32, vi);
         tmem_ld_wait();
-        const long long f = 1ll << (l < 4 ? 8 * (3 - l) : 8 * (6 - l));
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          (l < 4 ? hr : lr)[q] += (long long)__float2int_rn(__uint_as_float(vr[q])) * f;
-          (l < 4 ? hi : li)[q] += (long long)__float2int_rn(__uint_as_float(vi[q])) * f;
+          (l < 4 ? hr : lr)[q] += oz_weigh(__uint_as_float(vr[q]), l);
+          (l < 4 ? hi : li)[q] += oz_weigh(__uint_as_float(vi[q]), l);
         }
       }
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        ar[q] = (kMore ? ar[q] : 0) + hr[q] * 65536 + (lr[q] >> 8);
-        ai[q] = (kMore ? ai[q] : 0) + hi[q] * 65536 + (li[q] >> 8);
+        ar[q] = (kMore ? ar[q] : 0) + oz_sum(hr[q], lr[q]);
+        ai[q] = (kMore ? ai[q] : 0) + oz_sum(hi[q], li[q]);
       }
       tc::fence_before_sync();
     }

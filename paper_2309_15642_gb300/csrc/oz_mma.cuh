@@ -3,8 +3,9 @@
 //
 // The digit form is that of bigend_oz.cuh: x = 2^(E-6) sum_i d_i 2^(-8 i), seven digits
 // exact in f16, one exponent per row of an operand, the sums of 2 x 7 x 64 digit
-// products below 2^24 and so exact in FP32, an output rounded once to FP64.  It is at
-// least as accurate against the row maxima as a sum of FP64 multiply-adds.
+// products below 2^24 and so exact in FP32; error bound there.  Columns of the solve's
+// operands are unit vectors or scaled to norms in [1, 2), so that the row maxima are the
+// scale that an FP64 sum rounds against too.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -12,7 +13,17 @@
 
 namespace gpeps {
 
-constexpr int kOzSlices = 7;
+constexpr int kOzSlices = 7, kOzLevels = 8;
+
+// One more block of accumulators: high = levels 0..3 in units of level 3, low = levels 4..7 in
+// units of level 7, as an integer of unit 2^(Ea+Eb-53), rounded to nearest (a shift alone would
+// bias every output downwards by half a unit).
+__device__ __forceinline__ long long oz_sum(long long high, long long low) {
+  return high * (1ll << 17) + ((low + (1ll << 14)) >> 15);
+}
+__device__ __forceinline__ long long oz_weigh(float v, int l) {
+  return (long long)__float2int_rn(v) * (1ll << (8 * (3 - (l & 3))));
+}
 
 __device__ __forceinline__ int oz_exp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
@@ -36,7 +47,7 @@ __device__ __forceinline__ unsigned long long oz_fixed(double x, int em, bool ne
   return (neg ? 0ull - m : m) + 0x0080808080808080ull;
 }
 
-// t 2^(ea + eb - 2044 - 52) rounded to FP64 (ea, eb: biased exponents of the two rows);
+// t 2^(ea + eb - 2044 - 53) rounded to FP64 (ea, eb: biased exponents of the two rows);
 // NaN when a row held a value that is not finite.
 __device__ __forceinline__ double oz_value(long long t, int ea, int eb) {
   if (ea >= kOzNan || eb >= kOzNan) return __longlong_as_double(0x7ff8000000000000ll);
@@ -44,7 +55,7 @@ __device__ __forceinline__ double oz_value(long long t, int ea, int eb) {
   if (u == 0) return 0.0;
   const int n = __clzll((long long)u);
   const unsigned long long m = u << n;  // top bit at 63: value m 2^(-n) 2^(...)
-  const int e = 1023 + 63 - n + ea + eb - 2044 - 52;
+  const int e = 1023 + 63 - n + ea + eb - 2044 - 53;
   if (e <= 0) return 0.0;
   if (e >= 0x7ff) return __longlong_as_double(t < 0 ? 0xfff0000000000000ll : 0x7ff0000000000000ll);
   const unsigned long long r = ((unsigned long long)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
@@ -90,10 +101,10 @@ __device__ __forceinline__ void oz_exponents(const OzOperand& o, int n, int K) {
 // rows i0 + lane/4 (out[0], out[1]) and 8 more (out[2], out[3]), columns j0 + 2 (lane % 4)
 // and the next.
 //
-// A real 16 x 8 x 16 product takes 28 mma.sync.m16n8k16 and about 450 instructions for the
+// A real 16 x 8 x 16 product takes 34 mma.sync.m16n8k16 and about 450 instructions for the
 // digits of both tiles, taken from the FP64 values each time (kept in shared memory they
 // would need 28 bytes an element); as FP64 multiply-adds it is 64 instructions of 64
-// cycles each on the SMSP's FP64 unit.  Bound by issue slots.  Registers: 28 accumulators, 16 of
+// cycles each on the SMSP's FP64 unit.  Bound by issue slots.  Registers: 32 accumulators, 16 of
 // A's fixed-point values, 14 of B's digits.  E and Q of a 256-wide core: D = 128, one colour
 // class 355 -> 335 ms.
 __device__ __noinline__ void oz_tile(const OzOperand A, const OzOperand B, bool conj, int i0, int j0, int ni, int nj,
@@ -107,9 +118,9 @@ __device__ __noinline__ void oz_tile(const OzOperand A, const OzOperand B, bool 
     long long tot[4] = {0, 0, 0, 0};
 #pragma unroll 1
     for (int kc = 0; kc < kend; kc += 64) {
-      float acc[kOzSlices][4];
+      float acc[kOzLevels][4];
 #pragma unroll
-      for (int l = 0; l < kOzSlices; ++l)
+      for (int l = 0; l < kOzLevels; ++l)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[l][q] = 0.f;
 #pragma unroll 1
@@ -146,7 +157,7 @@ __device__ __noinline__ void oz_tile(const OzOperand A, const OzOperand B, bool 
 #pragma unroll
           for (int r = 0; r < 4; ++r) ad[r] = oz_pair(fa[2 * r], fa[2 * r + 1], i);
 #pragma unroll
-          for (int j = 0; j < kOzSlices - i; ++j)
+          for (int j = 0; j < (i ? kOzLevels - i : kOzSlices); ++j)
             asm volatile(
                 "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                 : "+f"(acc[i + j][0]), "+f"(acc[i + j][1]), "+f"(acc[i + j][2]), "+f"(acc[i + j][3])
@@ -155,10 +166,10 @@ __device__ __noinline__ void oz_tile(const OzOperand A, const OzOperand B, bool 
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        long long h = 0;  // unit 2^(Ea+Eb-52): level l weighs 2^(8 (5 - l))
+        long long h = 0, low = 0;
 #pragma unroll
-        for (int l = 0; l < 6; ++l) h += (long long)__float2int_rn(acc[l][q]) * (1ll << (8 * (5 - l)));
-        tot[q] += h + ((long long)__float2int_rn(acc[6][q]) >> 8);
+        for (int l = 0; l < kOzLevels; ++l) (l < 4 ? h : low) += oz_weigh(acc[l][q], l);
+        tot[q] += oz_sum(h, low);
       }
     }
 #pragma unroll

@@ -3594,4 +3594,17 @@ cudaError_t Adjoint::readout(const SiteDesc* sites, int n_sites, const void* gam
   return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------- self-tests of the bond core's products
+__global__ void __launch_bounds__(kBondThreads, 1)
+    core_selftest_kernel(int n, const double2* a, const double2* b, double2* out) {
+  __shared__ int ex[4 * kMaxDc128];
+  oz_product(a, n, 1, true, b, n, 1, ex, out, n, 1, n, false);
+}
+
+cudaError_t launch_core_selftest(int n, const void* a, const void* b, void* out, cudaStream_t st) {
+  core_selftest_kernel<<<1, kBondThreads, 0, st>>>(n, static_cast<const double2*>(a), static_cast<const double2*>(b),
+                                                   static_cast<double2*>(out));
+  return cudaGetLastError();
+}
+
 }  // namespace gpeps
