@@ -453,10 +453,12 @@ int gpeps_selftest_rotation(int32_t which, int32_t n, const double* in, double* 
 /*
  * Diagnostic: a step of the complex128 bond SVD on its own, by one CTA.  Arrays are device
  * complex128, n x n row-major, n even, 2 to 256.  which 0: the integer digit product of the
- * bond core, out[i][j] = sum_k conj(a[i][k]) b[j][k].  Asynchronous on stream.  Errors:
- * GPEPS_EINVAL for another `which` or n, or a NULL array; GPEPS_ECUDA for a failed launch.
+ * bond core, out[i][j] = sum_k conj(a[i][k]) b[j][k].  1: one simultaneous correction of the
+ * nearly orthogonal columns of a (column j in row j) into out; b is scratch of 3 n (n + 1)
+ * complex elements.  Asynchronous on stream.  Errors: GPEPS_EINVAL for another `which` or n,
+ * or a NULL array; GPEPS_ECUDA for a failed launch.
  */
-int gpeps_selftest_core(int32_t which, int32_t n, const double* a, const double* b, double* out, void* stream);
+int gpeps_selftest_core(int32_t which, int32_t n, const double* a, double* b, double* out, void* stream);
 
 int gpeps_destroy(gpeps_handle* h);
 const char* gpeps_error_string(int status);

@@ -182,8 +182,8 @@ struct OzPass {
                             const double* lam, const void* Y, const Scratch& ws, int* flags, int D, cudaStream_t st);
 };
 
-// One CTA: out = conj(a) b^T, n x n, as the digit products of the bond core.
-cudaError_t launch_core_selftest(int n, const void* a, const void* b, void* out, cudaStream_t st);
+// A step of the complex128 bond SVD by one CTA (gpeps_selftest_core).
+cudaError_t launch_core_selftest(int which, int n, const void* a, void* b, void* out, cudaStream_t st);
 
 constexpr int kMaxGradD = 16;  // bond dimension limit of the reverse mode (shared memory of its bond kernel)
 

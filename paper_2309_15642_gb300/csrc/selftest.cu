@@ -1,4 +1,4 @@
-// Diagnostic entry points.  The products of the bond core (kernel in su_kernels.cu), and the FP64 Jacobi rotation helpers of jacobi.cuh next to
+// Diagnostic entry points.  Steps of the bond core (kernel in su_kernels.cu), and the FP64 Jacobi rotation helpers of jacobi.cuh next to
 // the textbook formulas evaluated with CUDA's own FP64 hypot, sqrt and rsqrt, so
 // that a test can hold the helpers' Newton-Raphson refinements to a stated bound.
 #include <cuda_runtime.h>
@@ -55,8 +55,8 @@ extern "C" int gpeps_selftest_rotation(int32_t which, int32_t n, const double* i
   return cudaGetLastError() == cudaSuccess ? GPEPS_OK : GPEPS_ECUDA;
 }
 
-extern "C" int gpeps_selftest_core(int32_t which, int32_t n, const double* a, const double* b, double* out,
+extern "C" int gpeps_selftest_core(int32_t which, int32_t n, const double* a, double* b, double* out,
                                    void* stream) {
-  if (which != 0 || n < 2 || n > 2 * kMaxDc128 || (n & 1) || !a || !b || !out) return GPEPS_EINVAL;
-  return launch_core_selftest(n, a, b, out, static_cast<cudaStream_t>(stream)) == cudaSuccess ? GPEPS_OK : GPEPS_ECUDA;
+  if (which < 0 || which > 1 || n < 2 || n > 2 * kMaxDc128 || (n & 1) || !a || !b || !out) return GPEPS_EINVAL;
+  return launch_core_selftest(which, n, a, b, out, static_cast<cudaStream_t>(stream)) == cudaSuccess ? GPEPS_OK : GPEPS_ECUDA;
 }

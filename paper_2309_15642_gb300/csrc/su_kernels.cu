@@ -1392,19 +1392,37 @@ __device__ void svd_levels(double2* Zt, int rows, double2* Vt, int n, double tr,
 // One simultaneous correction of nearly orthogonal columns: Z <- Z (I + X + X^2 / 2), X
 // skew-Hermitian with the first-order angles X_pq = g_pq / (|z_q|^2 - |z_p|^2), g = Z^H Z, of
 // every pair whose angle is below kRefineAngle (the others, and columns at rounding,
-// are left to the sweeps).  The factor is unitary to |X|^4 / 4, at FP64 rounding; overlaps
-// of 1e-6 become ~1e-11 in one pass and 1e-16 in two, so the sweeps that follow find only
-// nearly degenerate pairs to rotate.  A full sweep costs 12 n^3 / 2 FP64 multiply-adds; here Z^H Z
-// and Z X are digit products on the tensor cores and X^2 / 2 (~1e-10) is FP32.
-// Columns are scaled to norms in [1, 2) by powers of two, so that every product is accurate relative to
+// are left to the sweeps).  Overlaps of 1e-6 become ~1e-11 in one pass and 1e-16 in two, so the
+// sweeps that follow find only nearly degenerate pairs to rotate.
+//
+// The factor is off a unitary one by X^4 / 4 and by the rounding of X^2 / 2, and what it is off
+// stays in the singular values.  Both are held to sqrt(n) 2^-53 an element, what the n
+// rotations of one sweep round: with rho the largest norm of a row of X^2, an element of X^4 / 4 is
+// at most rho^2 / 4, and the FP32 sums (blocks of 16 terms added with their rounding kept) make
+// about 2^-25 rho, so the pass needs rho <= sqrt(n) 2^-28.  Angles below kRefineAngle do not
+// give that by themselves (256 columns with all at the limit are 2e-13 off); where rho is
+// beyond it, the pass is built again from the pairs below 2^-14 / sqrt(n), which cannot exceed
+// it, and the rest is left to the sweeps.  Measured rho: up to 7e-9 at D = 32, 5e-9 at 64,
+// 4e-8 at 128.
+//
+// A full sweep costs 12 n^3 / 2 FP64 multiply-adds; here Z^H Z and Z X are digit products on
+// the tensor cores and X^2 / 2 (~1e-10) is FP32.  Columns are scaled to norms in [1, 2) by
+// powers of two, so that every product is accurate relative to
 // its column.  n >= kOzMinBond; Z square; G [n][n+1], Y [n][n], X32 [n][n] scratch; ex: 2n ints.
 // Measured (127 + 433 + 1121 qubits, D = 32): rotations of the first FP64 sweep 2010 -> 79 of 2016 pairs,
 // second 1516 -> 1; FP64 phase 5.14 -> 3.64 M cycles per bond, the rest of it Z itself and the checks.
 constexpr double kRefineAngle = 2e-5;
+constexpr double kRefineUnit = 1.0 / 16384.0;  // 2^-14
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// s += v, the rounding of the sum added to low (Knuth's two-sum)
+__device__ __forceinline__ void add_kept(float& s, float& low, float v) {
+  const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+  low += __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z));
+  s = t;
+}
 __device__ __noinline__ void svd_refine(double2* Zt, int n, double trace, double2* G, double2* Y, float2* X32,
                                         double* alpha, int* expo, int* ex) {
-  const int ldg = n + 1;
+  const int ldg = n + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   column_norms(Zt, n, n, alpha);
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
     const bool noise = !(alpha[j] > kNoiseRelSvd * trace);
@@ -1417,34 +1435,55 @@ __device__ __noinline__ void svd_refine(double2* Zt, int n, double trace, double
   __syncthreads();
   oz_product(Zt, n, 1, true, Zt, n, 1, ex, G, ldg, 1, n, true);
   __syncthreads();
-  for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
-    int i, j;
-    upper_index(idx, n, i, j);
-    double2 xij = make_double2(0.0, 0.0), xji = xij;
-    if (i < j && alpha[i] > 0.0 && alpha[j] > 0.0) {
-      const double2 g = G[i * ldg + j];
-      const double f = pow2(2 * (expo[j] - expo[i]));
-      const double r = 1.0 / fma(alpha[j], f, -alpha[i]);
-      if ((g.x * g.x + g.y * g.y) * (r * r * f) <= kRefineAngle * kRefineAngle) {
-        xij = cscale(g, r);
-        xji = cscale(cconj(g), -r * f);
+  __shared__ int square;  // largest squared norm of a row of X^2
+  for (double limit = kRefineAngle;; limit = kRefineUnit / sqrt((double)n)) {
+    if (threadIdx.x == 0) square = 0;
+    for (int idx = threadIdx.x; idx < n * (n + 1) / 2; idx += blockDim.x) {
+      int i, j;
+      upper_index(idx, n, i, j);
+      double2 xij = make_double2(0.0, 0.0), xji = xij;
+      if (i < j && alpha[i] > 0.0 && alpha[j] > 0.0) {
+        const double2 g = G[i * ldg + j];
+        const double f = pow2(2 * (expo[j] - expo[i]));
+        const double r = 1.0 / fma(alpha[j], f, -alpha[i]);
+        if ((g.x * g.x + g.y * g.y) * (r * r * f) <= limit * limit) {
+          xij = cscale(g, r);
+          xji = cscale(cconj(g), -r * f);
+        }
+      }
+      Y[i * n + j] = xij;
+      X32[i * n + j] = make_float2((float)xij.x, (float)xij.y);
+      if (i < j) {
+        Y[j * n + i] = xji;
+        X32[j * n + i] = make_float2((float)xji.x, (float)xji.y);
       }
     }
-    Y[i * n + j] = xij;
-    X32[i * n + j] = make_float2((float)xij.x, (float)xij.y);
-    if (i < j) {
-      Y[j * n + i] = xji;
-      X32[j * n + i] = make_float2((float)xji.x, (float)xji.y);
+    __syncthreads();
+    for (int i = warp; i < n; i += nw) {  // a row of X^2 / 2 and its norm, in the columns' own scale
+      float sum = 0.f;
+      for (int j = lane; j < n; j += 32) {
+        float2 acc = make_float2(0.f, 0.f), low = acc;
+        for (int k0 = 0; k0 < n; k0 += 16) {
+          float2 part = make_float2(0.f, 0.f);
+          for (int k = k0; k < min(k0 + 16, n); ++k) fma_c<float>(part, X32[i * n + k], X32[k * n + j]);
+          add_kept(acc.x, low.x, part.x);
+          add_kept(acc.y, low.y, part.y);
+        }
+        double2& y = Y[i * n + j];
+        y.x = fma(0.5, (double)acc.x, fma(0.5, (double)low.x, y.x));
+        y.y = fma(0.5, (double)acc.y, fma(0.5, (double)low.y, y.y));
+        const float f = __int_as_float(min(max(127 + expo[j] - expo[i], 0), 254) << 23);
+        sum = fmaf(acc.x * f, acc.x * f, fmaf(acc.y * f, acc.y * f, sum));
+      }
+      for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+      if (lane == 0) atomicMax(&square, __float_as_int(sum));
     }
+    __syncthreads();
+    constexpr float kSquare = (float)(kRefineUnit * kRefineUnit * kRefineUnit * kRefineUnit);  // 2^-56
+    const bool keep = limit < kRefineAngle || __int_as_float(square) <= kSquare * n;
+    __syncthreads();
+    if (keep) break;
   }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-    const int i = idx / n, j = idx - (idx / n) * n;
-    float2 acc = make_float2(0.f, 0.f);
-    for (int k = 0; k < n; ++k) fma_c<float>(acc, X32[i * n + k], X32[k * n + j]);
-    Y[idx] = make_double2(fma(0.5, (double)acc.x, Y[idx].x), fma(0.5, (double)acc.y, Y[idx].y));
-  }
-  __syncthreads();
   oz_product(Y, 1, n, false, Zt, 1, n, ex, G, ldg, 1, n, false);
   __syncthreads();
   for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
@@ -3594,15 +3633,29 @@ cudaError_t Adjoint::readout(const SiteDesc* sites, int n_sites, const void* gam
   return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- self-tests of the bond core's products
+// ---------------------------------------------------------------- self-tests of the bond core's steps
 __global__ void __launch_bounds__(kBondThreads, 1)
-    core_selftest_kernel(int n, const double2* a, const double2* b, double2* out) {
-  __shared__ int ex[4 * kMaxDc128];
-  oz_product(a, n, 1, true, b, n, 1, ex, out, n, 1, n, false);
+    core_selftest_kernel(int which, int n, const double2* a, double2* b, double2* out) {
+  __shared__ int ex[4 * kMaxDc128], expo[2 * kMaxDc128];
+  __shared__ double alpha[2 * kMaxDc128], trace;
+  if (which == 0) {
+    oz_product(a, n, 1, true, b, n, 1, ex, out, n, 1, n, false);
+    return;
+  }
+  for (int i = threadIdx.x; i < n * n; i += blockDim.x) out[i] = a[i];
+  __syncthreads();
+  column_norms(out, n, n, alpha);
+  if (threadIdx.x == 0) {
+    trace = 0.0;
+    for (int j = 0; j < n; ++j) trace += alpha[j];
+  }
+  __syncthreads();
+  double2* Y = b + n * (n + 1);
+  svd_refine(out, n, trace, b, Y, reinterpret_cast<float2*>(Y + n * n), alpha, expo, ex);
 }
 
-cudaError_t launch_core_selftest(int n, const void* a, const void* b, void* out, cudaStream_t st) {
-  core_selftest_kernel<<<1, kBondThreads, 0, st>>>(n, static_cast<const double2*>(a), static_cast<const double2*>(b),
+cudaError_t launch_core_selftest(int which, int n, const void* a, void* b, void* out, cudaStream_t st) {
+  core_selftest_kernel<<<1, kBondThreads, 0, st>>>(which, n, static_cast<const double2*>(a), static_cast<double2*>(b),
                                                    static_cast<double2*>(out));
   return cudaGetLastError();
 }
