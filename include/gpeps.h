@@ -161,7 +161,7 @@ int gpeps_step_profiled(gpeps_handle* h, const double* theta, int32_t per_qubit,
  * |b_p^H b_q| <= max(tol |b_p| |b_q|, floor_rel ||B||_F^2) (1e-14, 1e-20).  The
  * FP32 stages use tol32 (1e-6; complex128: relative to the two columns, its warm
  * start between 1e-6 and 1e-5) and floor32 (2e-7; mixed only); a complex128
- * warm start that hits its cap leaves the work to the FP64 sweeps; sweep caps
+ * warm start that hits its cap hands the basis it has to the FP64 sweeps; sweep caps
  * max_sweeps (40; hitting it sets GPEPS_FLAG_NOCONV) and max_sweeps32 (20).
  * Host-only; drops a captured step graph.  Errors: GPEPS_EINVAL for
  * non-positive thresholds or caps outside [1, 200] (FP64) / [0, 200] (FP32).

@@ -1146,6 +1146,92 @@ __device__ __forceinline__ float basis_tol32(const JacobiParams& jp) {
 // The warm start replaces remaining columns below this fraction of the first pivot by unit vectors of that size
 constexpr float kBasisCut = 1e-6f;
 
+// Unit columns orthogonal to FP32 rounding from those of a solve that ended at its cap
+// (A [n], stride ld, n entries each): modified Gram-Schmidt, largest column first, so that the
+// small ones lose what they still hold of the large, twice.  False (the same in every thread)
+// where a column lies within 1e-4 of the span of the larger ones, which is no basis to keep.
+__device__ __noinline__ bool orthogonal_units32(float2* A, int n, int ld, float* nrm) {
+  constexpr int kT = kMaxDc128 * 2 / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  auto wsum = [](float v) {
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+  };
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int v = warp; v < n; v += nw) {
+      float s = 0.f;
+      for (int x = lane; x < n; x += 32) {
+        const float2 a = A[(size_t)v * ld + x];
+        s = fmaf(a.x, a.x, fmaf(a.y, a.y, s));
+      }
+      s = wsum(s);
+      if (lane == 0) nrm[v] = s;
+    }
+    __syncthreads();
+    for (int i = 0; i < n; ++i) {
+      // the largest column left: every warp finds it for itself (norms of used ones are -1)
+      float best = -1.f;
+      int p = 0;
+      for (int v = lane; v < n; v += 32)
+        if (nrm[v] > best) {
+          best = nrm[v];
+          p = v;
+        }
+      for (int off = 16; off > 0; off >>= 1) {
+        const float ob = __shfl_xor_sync(0xffffffffu, best, off);
+        const int op = __shfl_xor_sync(0xffffffffu, p, off);
+        if (ob > best || (ob == best && op < p)) {
+          best = ob;
+          p = op;
+        }
+      }
+      float2 q[kT];
+      float s = 0.f;
+#pragma unroll
+      for (int t = 0; t < kT; ++t) {
+        const int x = lane + 32 * t;
+        q[t] = x < n ? A[(size_t)p * ld + x] : make_float2(0.f, 0.f);
+        s = fmaf(q[t].x, q[t].x, fmaf(q[t].y, q[t].y, s));
+      }
+      s = wsum(s);
+      if (!(s > 1e-8f * best)) return false;
+      const float inv = 1.f / sqrtf(s);
+#pragma unroll
+      for (int t = 0; t < kT; ++t) q[t] = make_float2(q[t].x * inv, q[t].y * inv);
+      __syncthreads();  // every warp has the pivot and the norms
+      for (int v = warp; v < n; v += nw) {
+        if (nrm[v] < 0.f) continue;
+        float2* a = A + (size_t)v * ld;
+        float2 d = make_float2(0.f, 0.f);
+        if (v != p)
+#pragma unroll
+          for (int t = 0; t < kT; ++t) {
+            const int x = lane + 32 * t;
+            if (x < n) fma_conj<float>(d, q[t], a[x]);
+          }
+        d.x = wsum(d.x);
+        d.y = wsum(d.y);
+#pragma unroll
+        for (int t = 0; t < kT; ++t) {
+          const int x = lane + 32 * t;
+          if (x < n) {
+            float2 u = q[t];
+            if (v != p) {
+              u = a[x];
+              fma_c<float>(u, make_float2(-d.x, -d.y), q[t]);
+            }
+            a[x] = u;
+          }
+        }
+        __syncwarp();
+        if (v == p && lane == 0) nrm[v] = -1.f;
+      }
+      __syncthreads();
+    }
+  }
+  return true;
+}
+
 // FP32 warm start: a unitary basis of the space of the nv indices of the vectors a_v
 // (A [nv], stride ld, `len` entries each) in which the columns of A = [a_v] are
 // nearly orthogonal: A's right singular vectors to FP32 accuracy, X [nv][nv] (row
@@ -1158,7 +1244,9 @@ constexpr float kBasisCut = 1e-6f;
 // vectors sought, so that no rotation product is accumulated.  When every remaining
 // vector is below kBasisCut of the first pivot the rest of R is replaced by that
 // multiple of the identity: below FP32's resolution any completion serves, and the
-// Jacobi makes it orthogonal to the others.  A solve that ends at its sweep cap gives the identity.  nv even; len, nv <= ld <= 256.
+// Jacobi makes it orthogonal to the others.  A solve that ends at its sweep cap keeps its
+// columns made orthogonal as they are (the identity where they are no basis).  nv even;
+// len, nv <= ld <= 256.
 __device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* nrm, const JacobiParams& jp,
                          int* iflag, unsigned long long* work, unsigned long long* rot_count) {
   constexpr int kT = kMaxDc128 * 2 / 32;  // elements of a vector per lane
@@ -1253,6 +1341,8 @@ __device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* 
   __syncthreads();
   const int sw = one_sided_jacobi32(A, ld, nv, nullptr, nv, basis_tol32(jp), kOsFloor32, jp.max_sweeps32, iflag,
                                     work, rot_count);
+  const bool basis = sw <= jp.max_sweeps32 || orthogonal_units32(A, nv, ld, nrm);
+  __syncthreads();
   for (int v = warp; v < nv; v += nw) {
     float s = 0.f;
     for (int x = lane; x < nv; x += 32) {
@@ -1266,8 +1356,8 @@ __device__ int svd_basis(float2* A, int nv, int len, int ld, double2* X, float* 
   for (int idx = threadIdx.x; idx < nv * nv; idx += blockDim.x) {
     const int v = idx / nv, i = idx - (idx / nv) * nv;
     const float2 a = A[(size_t)i * ld + v];
-    X[idx] = sw > jp.max_sweeps32 ? make_double2(v == i ? 1.0 : 0.0, 0.0)  // not orthogonal yet: the identity
-                                  : make_double2((double)(a.x * nrm[i]), (double)(a.y * nrm[i]));
+    X[idx] = basis ? make_double2((double)(a.x * nrm[i]), (double)(a.y * nrm[i]))
+                   : make_double2(v == i ? 1.0 : 0.0, 0.0);
   }
   __syncthreads();
   return sw;
