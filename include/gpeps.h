@@ -97,8 +97,13 @@ int gpeps_create(const gpeps_graph* graphs, int32_t n_instances, int32_t D, int3
  * largest colour class at D = 32 and 4.2 MB at D = 128; in the mixed path for
  * D > 34 the 2D x 2D bond eigenproblems that do not fit in shared memory, 772 KB
  * at D = 64), Gram partials of the larger ends (2 D^2 complex per tile of 64
- * rows, 32 rows in complex128 beyond D = 64),
- * <Z> outputs and the flag word.  Both need 256-byte alignment (cudaMalloc and
+ * rows), <Z> outputs and the flag word.  In complex128 from D = 17 the partials
+ * are D (D + 1) complex (per tile of 32 rows beyond D = 64) and the kicked rows
+ * of the larger ends come beside them (2 D complex per row, as much as their
+ * tensors); where they and the state would pass 240 GiB, a colour class runs in
+ * groups of bonds that share 48 GiB (or the scratch of 304 bonds, 60 GB at
+ * D = 128).  1121 qubits in complex128: state 0.44, 3.5 and 27 GB, work 0.7, 5.8 and 84 GB at
+ * D = 32, 64 and 128.  Both need 256-byte alignment (cudaMalloc and
  * torch give it).
  */
 int gpeps_query_workspace(const gpeps_handle* h, size_t* state_bytes, size_t* work_bytes);

@@ -22,7 +22,8 @@
 // x 2^-53 rms for K = 16, 64 and 128; a chain of FP64 multiply-adds makes 0.58, 1.25 and
 // 2.47 (seven levels and a low part cut off rather than rounded made 1.9, 3.6 and 5.1, with a
 // mean of -0.9, in 28 digit products instead of 34; one class of 127 + 433 + 1121 qubits, D = 32:
-// Gram 1.95 -> 2.07, bonds 11.3 -> 11.4, update 1.39 -> 1.58 ms).  Against the terms themselves it is an FP64 sum's only as far as they are within a few bits of the row
+// Gram 1.95 -> 2.07, bonds 11.3 -> 11.4, update 1.39 -> 1.58 ms).  Against the terms
+// themselves it is an FP64 sum's only as far as they are within a few bits of the row
 // maxima: the passes scale their operands for that (the Gram's columns are summed over rows
 // against their own norms, the update balances k).
 //
@@ -34,7 +35,8 @@
 //
 //   oz_gram_kernel    one CTA per row tile (and spin, beyond D = 32): kicks the
 //       rows (writing them, unweighted, to `at` for the update), weights them, and
-//       writes the tile's Gram blocks in FP64 (the partials of gram_kernel).
+//       writes the upper triangles of the tile's Gram blocks in FP64 (they are Hermitian to
+//       the bit: both triangles come from the same integers).
 //   oz_update_kernel  one CTA per 128 rows, spin and 32 new bond indices:
 //       Gamma_a'[s] = mask (Ã_s Y_s) from `at`, the bond index balanced first.
 //
@@ -212,8 +214,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   const int m = 32 * (warp & 3) + lane, n0 = 32 * (warp >> 2);
   const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)n0;
   double* dump = reinterpret_cast<double*>(smem_raw);
-  const int D2 = D * D;
-  double2* out = partials + (int64_t)t.part * 2 * D2;
+  const int half = D * (D + 1) / 2;
+  double2* out = partials + (int64_t)t.part * 2 * half + (kMode == 0 ? 0 : s * half);
   for (int prod = 0; prod < (kMode == 2 ? 2 : 1) && ok; ++prod) {
     long long acc[32];
     issue(prod, 0);
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 #pragma unroll
       for (int q = 0; q < 32; ++q) {
         const int l = n0 + q;
-        if (m < D && l < D) out[s * D2 + m * D + l].x = oz_value(acc[q], ea, cmax[l]);
+        if (m <= l && l < D) out[upper_pos(m, l, D)].x = oz_value(acc[q], ea, cmax[l]);
       }
     } else {
       auto ce = [&](int c) { return cmax[kMode == 0 ? (c >> 6) * 32 + (c & 31) : kMode == 1 ? (c & 63) : c]; };
@@ -271,17 +273,21 @@ __global__ void __launch_bounds__(kOzThreads, 1)
   }
   if (ok) {
     if (kMode == 2) {
-      for (int o = threadIdx.x; o < D2; o += kOzThreads) {
-        const int a = o / D, b = o - a * D;
-        out[s * D2 + o].y = dump[a * kOzDumpLd + b] - dump[b * kOzDumpLd + a];
+      for (int o = threadIdx.x; o < half; o += kOzThreads) {
+        int a, b;
+        upper_index(o, D, a, b);
+        out[o].y = dump[a * kOzDumpLd + b] - dump[b * kOzDumpLd + a];
       }
     } else {
       constexpr int kp = kMode == 0 ? 32 : 64;
-      for (int o = threadIdx.x; o < (kMode == 0 ? 2 : 1) * D2; o += kOzThreads) {
-        const int sp = kMode == 0 ? o / D2 : s, ab = kMode == 0 ? o - sp * D2 : o, a = ab / D, b = ab - a * D;
-        const int ra = (kMode == 0 ? sp * 64 : 0) + a, rb = (kMode == 0 ? sp * 64 : 0) + b;
-        out[sp * D2 + ab] = make_double2(dump[ra * kOzDumpLd + rb] + dump[(ra + kp) * kOzDumpLd + rb + kp],
-                                         dump[ra * kOzDumpLd + rb + kp] - dump[(ra + kp) * kOzDumpLd + rb]);
+      for (int o = threadIdx.x; o < (kMode == 0 ? 2 : 1) * half; o += kOzThreads) {
+        const int sp = kMode == 0 && o >= half ? 1 : 0;  // (D <= 32: both spins)
+        int ra, rb;
+        upper_index(o - sp * half, D, ra, rb);
+        ra += sp * 64;
+        rb += sp * 64;
+        out[o] = make_double2(dump[ra * kOzDumpLd + rb] + dump[(ra + kp) * kOzDumpLd + rb + kp],
+                              dump[ra * kOzDumpLd + rb + kp] - dump[(ra + kp) * kOzDumpLd + rb]);
       }
     }
   } else if (threadIdx.x == 0) {

@@ -33,12 +33,26 @@ int cuda_fail(cudaError_t e, const char* where) {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Bonds and row tiles of one set of launches; the scratch slots of a bond (Gram partials, kicked
+// rows, Y) are numbered within it.
+struct LaunchGroup {
+  int bond0 = 0, n_bonds = 0, tile0 = 0, n_tiles = 0, n_parts = 0;
+};
 struct ColourPlan {
   std::vector<BondDesc> bonds;
   std::vector<TileDesc> tiles;
+  std::vector<LaunchGroup> groups;
   size_t w_bonds = 0, w_tiles = 0;  // byte offsets in the work buffer
-  int n_parts = 0;
 };
+// The complex128 tensor-core passes keep the kicked rows of a class beside its Gram partials, as
+// much again as the class's tensors (beyond D = 64 the rows and the partials' upper triangles are
+// less than the full partials were).  Where a batch's state and scratch pass kRoom (of the 298 GB
+// of the card), its classes run in groups of bonds whose partials and rows stay within
+// kGroupScratch, so that every batch that fitted without the rows fits with them.  Multiples of
+// kGroupBonds, two to each of 152 SMs, to keep a group's waves full: ten or more of them, where a
+// group's tail costs a few per cent (two waves of 304 bonds at D = 128 cost 20).
+constexpr size_t kRoom = (size_t)240 << 30, kGroupScratch = (size_t)48 << 30;
+constexpr int kGroupBonds = 304;
 
 struct InstGraph {
   int n = 0;
@@ -111,6 +125,8 @@ struct gpeps_handle {
   // their own (they take a whole SM's shared memory and TMEM), so a step is layered on every schedule
   bool oz() const { return elt == 16 && OzPass::supported(D); }
   bool fused() const { return schedule >= 4 && !oz(); }
+  // bytes of the Gram blocks of one row tile (complex128 tensor-core passes: their upper triangles)
+  size_t gram_part() const { return (oz() ? (size_t)D * (D + 1) : (size_t)2 * D * D) * elt; }
   OzPass::Scratch oz_scratch() const {
     return OzPass::Scratch{at<double>(w_at), at<int>(w_balance), d_work + w_cs};
   }
@@ -232,6 +248,7 @@ SideDesc side_desc(const gpeps_handle* h, int inst, int v, int nbr) {
 
 struct PhaseEvents {
   cudaEvent_t ev[4];
+  float ms[3];  // sums over the class's groups
 };
 
 // CTAs per SM of the layered bond launch (schedule 4 runs its layers, outside
@@ -273,37 +290,46 @@ int fused_step_impl(gpeps_handle* h) {
 template <typename T>
 int layer_impl(gpeps_handle* h, int c, PhaseEvents* pe = nullptr, void* vsave = nullptr) {
   ColourPlan& cp = h->colours[c];
-  const int nt = (int)cp.tiles.size(), nbd = (int)cp.bonds.size();
-  if (nbd == 0) return GPEPS_OK;
-  const TileDesc* tiles = h->at<TileDesc>(cp.w_tiles);
-  const BondDesc* bonds = h->at<BondDesc>(cp.w_bonds);
   void* partials = h->d_work + h->w_partials;
   void* Y = h->d_work + h->w_Y;
   double* theta_a = h->at<double>(h->w_theta_a);
-  if (pe) GP_CUDA(cudaEventRecord(pe->ev[0], h->stream));
-  if (h->oz())
-    GP_CUDA(OzPass::gram(tiles, nt, bonds, nbd, h->gamma(), h->lam(), h->pending(), partials, h->oz_scratch(),
-                         h->flags(), h->D, h->stream));
-  else if (h->tensor)
-    GP_CUDA(Launch<T>::gram_tc(bonds, nbd, h->gamma(), h->lam(), h->pending(), partials, h->flags(), h->D,
-                               h->stream));
-  else
-    GP_CUDA(Launch<T>::gram(tiles, nt, bonds, h->gamma(), h->lam(), h->pending(), partials, h->D, h->stream));
-  if (pe) GP_CUDA(cudaEventRecord(pe->ev[1], h->stream));
-  GP_CUDA(Launch<T>::bond(bonds, nbd, partials, h->gamma(), h->lam(), h->pending(), Y, theta_a, h->flags(),
-                          h->sweeps(), h->cycles(), vsave, h->D, h->jp, h->stream,
-                          h->schedule ? h->at<unsigned int>(h->w_queue) : nullptr, h->n_sms,
-                          h->d_work + h->w_bond_scratch, layered_per_sm(h, nbd)));
-  if (pe) GP_CUDA(cudaEventRecord(pe->ev[2], h->stream));
-  if (h->oz())
-    GP_CUDA(OzPass::update(tiles, nt, bonds, nbd, h->gamma(), h->lam(), Y, h->oz_scratch(), h->flags(), h->D,
-                           h->stream));
-  else if (h->tensor)
-    GP_CUDA(Launch<T>::update_tc(bonds, nbd, h->gamma(), h->lam(), Y, theta_a, h->flags(), h->D, h->stream));
-  else
-    GP_CUDA(Launch<T>::update(tiles, nt, bonds, h->gamma(), h->lam(), Y, theta_a, h->D, h->stream));
-  if (pe) GP_CUDA(cudaEventRecord(pe->ev[3], h->stream));
-  h->bonds_since_reset += nbd;
+  for (const LaunchGroup& lg : cp.groups) {
+    const int nt = lg.n_tiles, nbd = lg.n_bonds;
+    const TileDesc* tiles = h->at<TileDesc>(cp.w_tiles) + lg.tile0;
+    const BondDesc* bonds = h->at<BondDesc>(cp.w_bonds) + lg.bond0;
+    if (pe) GP_CUDA(cudaEventRecord(pe->ev[0], h->stream));
+    if (h->oz())
+      GP_CUDA(OzPass::gram(tiles, nt, bonds, nbd, h->gamma(), h->lam(), h->pending(), partials, h->oz_scratch(),
+                           h->flags(), h->D, h->stream));
+    else if (h->tensor)
+      GP_CUDA(Launch<T>::gram_tc(bonds, nbd, h->gamma(), h->lam(), h->pending(), partials, h->flags(), h->D,
+                                 h->stream));
+    else
+      GP_CUDA(Launch<T>::gram(tiles, nt, bonds, h->gamma(), h->lam(), h->pending(), partials, h->D, h->stream));
+    if (pe) GP_CUDA(cudaEventRecord(pe->ev[1], h->stream));
+    GP_CUDA(Launch<T>::bond(bonds, nbd, partials, h->gamma(), h->lam(), h->pending(), Y, theta_a, h->flags(),
+                            h->sweeps(), h->cycles(), vsave, h->D, h->jp, h->stream,
+                            h->schedule ? h->at<unsigned int>(h->w_queue) : nullptr, h->n_sms,
+                            h->d_work + h->w_bond_scratch, layered_per_sm(h, nbd)));
+    if (pe) GP_CUDA(cudaEventRecord(pe->ev[2], h->stream));
+    if (h->oz())
+      GP_CUDA(OzPass::update(tiles, nt, bonds, nbd, h->gamma(), h->lam(), Y, h->oz_scratch(), h->flags(), h->D,
+                             h->stream));
+    else if (h->tensor)
+      GP_CUDA(Launch<T>::update_tc(bonds, nbd, h->gamma(), h->lam(), Y, theta_a, h->flags(), h->D, h->stream));
+    else
+      GP_CUDA(Launch<T>::update(tiles, nt, bonds, h->gamma(), h->lam(), Y, theta_a, h->D, h->stream));
+    if (pe) {
+      GP_CUDA(cudaEventRecord(pe->ev[3], h->stream));
+      GP_CUDA(cudaEventSynchronize(pe->ev[3]));
+      for (int i = 0; i < 3; ++i) {
+        float ms = 0.f;
+        GP_CUDA(cudaEventElapsedTime(&ms, pe->ev[i], pe->ev[i + 1]));
+        pe->ms[i] += ms;
+      }
+    }
+    h->bonds_since_reset += nbd;
+  }
   return GPEPS_OK;
 }
 
@@ -442,23 +468,44 @@ int gpeps_create(const gpeps_graph* graphs, int32_t n_instances, int32_t D, int3
       if (x.b.rows != y.b.rows) return x.b.rows > y.b.rows;
       return x.a.rows > y.a.rows;
     });
+    const int tr = tile_rows(D, dtype == GPEPS_C128 ? 16 : 8);
+    int most = std::max((int)cp.bonds.size(), 1);  // bonds of a group
+    if (h->oz()) {
+      const size_t part = h->gram_part() + OzPass::at_doubles(D) * sizeof(double);
+      size_t all = 0, largest = part;
+      for (auto& bd : cp.bonds) {
+        const size_t bytes = part * (size_t)((bd.a.rows + tr - 1) / tr);
+        all += bytes;
+        largest = std::max(largest, bytes);
+      }
+      if ((size_t)h->n_gamma * h->elt + all > kRoom)
+        most = (int)std::min<size_t>(most, std::max<size_t>(kGroupScratch / largest / kGroupBonds, 1) * kGroupBonds);
+    }
     for (int bi = 0; bi < (int)cp.bonds.size(); ++bi) {
+      if (bi % most == 0) {
+        LaunchGroup lg;
+        lg.bond0 = bi;
+        lg.tile0 = (int)cp.tiles.size();
+        cp.groups.push_back(lg);
+      }
+      LaunchGroup& lg = cp.groups.back();
       BondDesc& bd = cp.bonds[bi];
-      bd.part0 = cp.n_parts;
-      const int tr = tile_rows(D, dtype == GPEPS_C128 ? 16 : 8);
+      bd.part0 = lg.n_parts;
       bd.n_parts = (bd.a.rows + tr - 1) / tr;
       for (int p = 0; p < bd.n_parts; ++p) {
         TileDesc t{};
-        t.bond = bi;
+        t.bond = lg.n_bonds;
         t.row0 = p * tr;
         t.nrows = std::min(tr, bd.a.rows - t.row0);
-        t.part = cp.n_parts + p;
+        t.part = lg.n_parts + p;
         cp.tiles.push_back(t);
       }
-      cp.n_parts += bd.n_parts;
+      lg.n_parts += bd.n_parts;
+      lg.n_tiles += bd.n_parts;
+      ++lg.n_bonds;
+      h->max_parts = std::max(h->max_parts, lg.n_parts);
+      h->max_bonds = std::max(h->max_bonds, lg.n_bonds);
     }
-    h->max_parts = std::max(h->max_parts, cp.n_parts);
-    h->max_bonds = std::max(h->max_bonds, (int)cp.bonds.size());
   }
   // fused step: every bond of a step, colour by colour; a task waits for the
   // last earlier task on each of its sites.  Class 0 keeps its cost order; a
@@ -509,6 +556,7 @@ int gpeps_create(const gpeps_graph* graphs, int32_t n_instances, int32_t D, int3
   // update pass) takes about a second on its SM: its dependants may wait longer
   h->jp.wait_cycles = kWaitCycles * (D > kMaxD ? 16 : 1);
   h->jp.gate_sign = 1;
+  h->jp.upper_partials = h->oz();
   // layouts
   size_t s = 0;
   h->s_lam = s;
@@ -537,7 +585,7 @@ int gpeps_create(const gpeps_graph* graphs, int32_t n_instances, int32_t D, int3
     cp.w_bonds = carve(cp.bonds.size() * sizeof(BondDesc));
     cp.w_tiles = carve(cp.tiles.size() * sizeof(TileDesc));
   }
-  h->w_partials = carve((size_t)h->max_parts * 2 * D * D * h->elt);
+  h->w_partials = carve((size_t)h->max_parts * h->gram_part());
   h->w_Y = carve((size_t)h->max_bonds * 2 * D * D * h->elt);
   h->w_theta_a = carve((size_t)h->max_bonds * sizeof(double));
   if (h->oz()) {
@@ -641,11 +689,9 @@ int gpeps_zz_layer_profiled(gpeps_handle* h, int32_t colour, float* ms) {
   PhaseEvents pe{};
   for (int i = 0; i < 4; ++i) GP_CUDA(cudaEventCreate(&pe.ev[i]));
   int st = layer(h, colour, &pe);
-  cudaError_t e = cudaEventSynchronize(pe.ev[3]);
-  for (int i = 0; i < 3 && st == GPEPS_OK && e == cudaSuccess; ++i) e = cudaEventElapsedTime(&ms[i], pe.ev[i], pe.ev[i + 1]);
   for (int i = 0; i < 4; ++i) cudaEventDestroy(pe.ev[i]);
   if (st) return st;
-  if (e != cudaSuccess) return cuda_fail(e, "gpeps_zz_layer_profiled");
+  for (int i = 0; i < 3; ++i) ms[i] = pe.ms[i];
   return GPEPS_OK;
 }
 

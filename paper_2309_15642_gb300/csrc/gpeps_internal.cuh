@@ -100,6 +100,7 @@ struct JacobiParams {
   int levels;          // extra FP32 levels at most (0..kMaxExtraLevels)
   long long wait_cycles;  // fused step: a wait for an earlier task gives up after this many SM cycles
   int full_basis;         // complex128: keep a complete unitary V per bond (the reverse mode; see bond_front_svd)
+  int upper_partials;     // complex128: Gram partials as oz_gram_kernel writes them, upper triangles in upper_index order
   int gate_sign;          // +1: the paper's exp(+i pi/4 Z Z); -1: its inverse exp(-i pi/4 Z Z)
 };
 

@@ -235,8 +235,8 @@ BondFootprint bond_footprint(int D, size_t smem_optin, size_t elt) {
 
 
 // Bijection from [0, n(n+1)/2) onto the upper triangle i <= j of an n x n
-// matrix (n even): row r is paired with row n-1-r (lengths n-r and r+1), so a
-// loop over the triangle keeps every lane busy.
+// matrix: row r is paired with row n-1-r (lengths n-r and r+1), so a loop over the
+// triangle keeps every lane busy.  upper_pos is its inverse.
 __device__ __forceinline__ void upper_index(int idx, int n, int& i, int& j) {
   const int w = n + 1;
   const int r = idx / w, c = idx - (idx / w) * w;
@@ -247,6 +247,9 @@ __device__ __forceinline__ void upper_index(int idx, int n, int& i, int& j) {
     i = n - 1 - r;
     j = i + (c - (n - r));
   }
+}
+__device__ __forceinline__ int upper_pos(int i, int j, int n) {
+  return 2 * i < n ? i * (n + 1) + j - i : (n - 1 - i) * (n + 1) + j + 1;
 }
 
 // Re-orthonormalise the columns of V (n x n, row stride n) in FP64.  V is a
@@ -1628,20 +1631,27 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
       t_prev = t;
     }
   };
-  // G_s, FP64
-  for (int o = threadIdx.x; o < 2 * D2; o += blockDim.x) {
+  // G_s, FP64 (with upper_partials from the upper triangles)
+  const int half = D * (D + 1) / 2, part = jp.upper_partials ? half : D2;
+  for (int o = threadIdx.x; o < 2 * part; o += blockDim.x) {
     double2 acc = make_double2(0.0, 0.0);
     if (gsum) {
       acc = gsum[o];
     } else {
       for (int p = 0; p < bd.n_parts; ++p) {
-        const double2 v = partials[(int64_t)p * 2 * D2 + o];
+        const double2 v = partials[(int64_t)p * 2 * part + o];
         acc.x += v.x;
         acc.y += v.y;
       }
     }
-    const int sidx = o / D2, kl = o - sidx * D2, k = kl / D, l = kl - (kl / D) * D;
-    Cw[(size_t)sidx * D * (D + 1) + k * (D + 1) + l] = acc;
+    const int sidx = o / part, kl = o - sidx * part;
+    double2* C = Cw + (size_t)sidx * D * (D + 1);
+    int k = kl / D, l = kl - (kl / D) * D;
+    if (jp.upper_partials) {
+      upper_index(kl, D, k, l);
+      C[l * (D + 1) + k] = cconj(acc);
+    }
+    C[k * (D + 1) + l] = acc;
   }
   __syncthreads();  // kcs
   load_F<double, kCG>(sb, gamma, lam, kcs, F, D);
@@ -2056,7 +2066,8 @@ __device__ __forceinline__ void bond_body_layered(int bi, const BondDesc* __rest
                                                   double2* vsave, int D, JacobiParams jp, unsigned char* big) {
   const BondDesc bd = bonds[bi];
   const int D2 = D * D, nm = 2 * D;
-  bond_body<T, false>(bd, partials + (int64_t)bd.part0 * 2 * D2, nullptr, gamma, lam, pending,
+  const int part = sizeof(T) == 8 && jp.upper_partials ? D * (D + 1) : 2 * D2;
+  bond_body<T, false>(bd, partials + (int64_t)bd.part0 * part, nullptr, gamma, lam, pending,
                       Yout + (int64_t)bi * 2 * D2, theta_a + bi, flags, sweeps_out, cycles,
                       vsave ? vsave + (int64_t)bi * (nm * nm + nm) : nullptr, D, jp, big);
 }
