@@ -450,7 +450,8 @@ int gpeps_bond_update_noalloc(int32_t D, int32_t dtype, void* gamma_a, int32_t d
  * receives the helper's (c, s, Re e, Im e) and then the reference's.  which: 0
  * the two-sided helper of the squared eigensolver (|g|^2 must be above FP32's
  * smallest normal), 1 the one-sided helper of the complex128 bond SVD (any
- * finite scale).  Asynchronous on stream.  Errors: GPEPS_EINVAL for n < 0, an
+ * finite scale with |g|^2 finite and not zero), its s and e formed from its tau = t / |g| and
+ * g; 3 the same helper's own results (tau, c, 1 + t^2, t |g|).  Asynchronous on stream.  Errors: GPEPS_EINVAL for n < 0, an
  * unknown `which` or NULL arrays; GPEPS_ECUDA for a failed launch.
  */
 int gpeps_selftest_rotation(int32_t which, int32_t n, const double* in, double* out, void* stream);

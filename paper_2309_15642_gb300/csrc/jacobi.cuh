@@ -129,9 +129,10 @@ __device__ __forceinline__ float os_down(double v, int E) {
   const int m = ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29);
   return e > 0 && e < 255 ? __int_as_float((hi & 0x80000000) | (e << 23) | m) : 0.f;
 }
-__device__ __forceinline__ double os_up(float f, int E) {  // f 2^(1023 - E), f a normal number
+// f 2^(1023 - E), f a normal number, E >= 1 (zero below the double range, which E > 2044 reaches)
+__device__ __forceinline__ double os_up(float f, int E) {
   const int b = __float_as_int(f), e = ((b >> 23) & 0xff) - 127 + 2046 - E;
-  return __hiloint2double((b & 0x80000000) | (e << 20) | ((b & 0x7fffff) >> 3), b << 29);
+  return e > 0 ? __hiloint2double((b & 0x80000000) | (e << 20) | ((b & 0x7fffff) >> 3), b << 29) : 0.0;
 }
 
 // Rotation of the column pair with squared norms a, b, inner product g = b_p^H b_q
@@ -142,8 +143,9 @@ __device__ __forceinline__ double os_up(float f, int E) {  // f 2^(1023 - E), f 
 // root of g2 tau^2 + (b - a) tau - 1 = 0, so neither |g| nor its inverse is formed:
 // an FP32 value, from operands scaled by the power of two of the largest, and one
 // Newton step with the FP32 derivative (relative error about 1e-7 x 1e-7).  c =
-// 1 / sqrt(1 + t^2) from FP32 and one third-order step, to rounding, so that the
-// rotation is unitary whatever the angle's error.  Returns tau, c, u = 1 + t^2 and
+// 1 / sqrt(1 + t^2) from FP32 and one third-order step (the binomial series of
+// (1 - rho)^(-1/2)), to rounding, so that the rotation is unitary whatever the angle's
+// error.  Returns tau, c, u = 1 + t^2 and
 // w = t |g| (the squared norms become a - w and b + w).
 __device__ __forceinline__ void os_rotation(double a, double b, double2 g, double g2, double& tau, double& c,
                                             double& u, double& w) {

@@ -16,7 +16,8 @@ namespace {
 // One thread per input (a, b, Re g, Im g): the helper's (c, s, e), then the
 // reference: |g| = hypot, zeta = (b - a) / (2 |g|), t = sign(zeta) / (|zeta| +
 // sqrt(1 + zeta^2)) (t = 1 / (2 zeta) beyond 1e150), c = rsqrt(1 + t^2), s = t c,
-// e = conj(g) / |g|.
+// e = conj(g) / |g|.  which 3: what the one-sided sweeps use, tau = t / |g|, c, 1 + t^2 and
+// t |g|, then the same from the reference.
 __global__ void rotation_selftest_kernel(int which, int n, const double* __restrict__ in, double* __restrict__ out) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
@@ -36,6 +37,13 @@ __global__ void rotation_selftest_kernel(int which, int n, const double* __restr
   const double t = fabs(zeta) > 1e150 ? 0.5 / zeta : copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
   const double cr = rsqrt(fma(t, t, 1.0));
   double* o = out + 8 * (size_t)k;
+  if (which == 3) {
+    double tau, cc, u, w;
+    os_rotation(a, b, g, fma(g.x, g.x, g.y * g.y), tau, cc, u, w);
+    const double r[8] = {tau, cc, u, w, t / gr, cr, fma(t, t, 1.0), t * gr};
+    for (int i = 0; i < 8; ++i) o[i] = r[i];
+    return;
+  }
   o[0] = c;
   o[1] = s;
   o[2] = e.x;
@@ -49,7 +57,7 @@ __global__ void rotation_selftest_kernel(int which, int n, const double* __restr
 }  // namespace
 
 extern "C" int gpeps_selftest_rotation(int32_t which, int32_t n, const double* in, double* out, void* stream) {
-  if (n < 0 || (which != 0 && which != 1) || (n > 0 && (!in || !out))) return GPEPS_EINVAL;
+  if (n < 0 || (which != 0 && which != 1 && which != 3) || (n > 0 && (!in || !out))) return GPEPS_EINVAL;
   if (n == 0) return GPEPS_OK;
   rotation_selftest_kernel<<<(n + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(which, n, in, out);
   return cudaGetLastError() == cudaSuccess ? GPEPS_OK : GPEPS_ECUDA;
