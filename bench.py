@@ -168,6 +168,11 @@ NCU_TRAFFIC = {
 TF32_OVER_BF16 = 1.1 / 2.25
 
 # ------------------------------------------------------------------ algorithmic counts
+# complex128: smallest D whose larger ends' passes, and smallest core whose square products, are
+# integer digit products on the tensor cores; from that D every schedule runs layered launches
+C128_DIGITS_D, C128_DIGITS_N = 17, 48
+
+
 def bond_fixed_flops(graphs, D, dtype):
     """(FP64, FP32) flops of one Trotter step's bond eigenproblems that do not depend on how the
     Jacobi sweeps converge, per bond with its own n = 2 D^(deg - 1) (deg of the smaller end;
@@ -176,9 +181,13 @@ def bond_fixed_flops(graphs, D, dtype):
     E-sized products X1^dagger X1 and X^2 (n^3 / 6 MACs each) in FP32; rho' = V^dagger rho V
     3 n^3 / 2 MACs in FP64; the rho formation 2 (n D^2 + n(n+1)/2 D) MACs and the Y matrices
     2 D^2 n MACs in FP32.  Complex128
-    (unsquared form, all FP64): the pivoted Cholesky roots of the two D x D Gram blocks 2 D^3 / 3
-    MACs, the core M = 2D x n, 2D n D MACs, the re-orthonormalisation 4 n^3 / 3, B = M V0 2D n^2
-    and the Y matrices 2 D^2 n MACs.  The Jacobi sweeps and the levels are counted in the kernel."""
+    (unsquared form): in FP64 the pivoted Cholesky roots of the two D x D Gram blocks 2 D^3 / 3
+    MACs, the core M = 2D x n, 2D n D MACs, Z = M^H U0 (or B = M V0) 2D n^2 and the Y matrices
+    2 D^2 n MACs, and below C128_DIGITS_N columns E and Q of the re-orthonormalisation, n^3 / 2
+    each; from there they and the products of the two simultaneous corrections are integer
+    digit products on the tensor cores (as the larger ends' passes from C128_DIGITS_D), which
+    count as neither; in FP32 the E-sized products n^3 / 3 and X^2 of the corrections.  The
+    Jacobi sweeps and the levels are counted in the kernel."""
     import numpy as np
     f64 = f32 = 0.0
     for n_q, edges in graphs:
@@ -186,7 +195,10 @@ def bond_fixed_flops(graphs, D, dtype):
         for a, b in edges:
             n = 2 * D ** (int(min(deg[a], deg[b])) - 1)
             if dtype == "c128":
-                f64 += (2.0 * D ** 3 / 3 + 2 * D * n * D + 4.0 * n ** 3 / 3 + 2 * D * n * n + 2 * D * D * n) * 8
+                digits = n >= C128_DIGITS_N
+                f64 += (2.0 * D ** 3 / 3 + 2 * D * n * D + 2 * D * n * n + 2 * D * D * n) * 8
+                f64 += 0 if digits else n ** 3 * 8
+                f32 += (n ** 3 / 3.0 + (2.0 * n ** 3 if digits and n == 2 * D else 0)) * 8
                 continue
             f64 += (n ** 3 + 1.5 * n ** 3) * 8
             f32 += (2 * (n * D * D + n * (n + 1) / 2 * D) + 2 * D * D * n + n ** 3 / 3.0) * 8
@@ -199,10 +211,15 @@ JACOBI_BLOCK_FLOPS, JACOBI_VEC_FLOPS = 72, 18
 
 
 def one_sided_flops(D, checks, rotations):
-    """Real flops of the complex128 one-sided sweeps: a pair check forms |b_p|^2, |b_q|^2 and
-    b_p^H b_q over the 2D rows (16 flops per row), a rotation updates 2D rows of B and n <= 2D
-    rows of V (18 flops per row pair; counted at n = 2D)."""
-    return checks * 16 * 2 * D + rotations * 18 * 4 * D
+    """Real flops of the complex128 FP64 sweeps: a pair check forms z_p^H z_q over the 2D rows
+    (8 flops per row; the norms are carried), a scaled rotation updates them (16 flops per row
+    pair; V is not accumulated for a square core)."""
+    return checks * 8 * 2 * D + rotations * 16 * 2 * D
+
+
+def one_sided_flops32(D, checks, rotations):
+    """The same of the FP32 stages: norms and inner product (16 flops per row), 18 per row pair."""
+    return checks * 16 * 2 * D + rotations * 18 * 2 * D
 
 
 # ------------------------------------------------------------------ committed oracle values
@@ -601,7 +618,8 @@ def run_gpeps(args, rank, world, local_rank):
     # of the timed region (fused: one launch per step; layered: three per colour class)
     sched = (tuning["chosen"].get("persistent", 0) if tuning else (args.schedule or 0))
     tensor = bool(tuning["chosen"].get("tensor", False)) if tuning else (args.tensor and args.dtype == "mixed")
-    fused = sched >= 4          # schedules 4, 5 and 6: the fused step (two, three or four CTAs per SM)
+    # schedules 4, 5 and 6: the fused step (two, three or four CTAs per SM)
+    fused = sched >= 4 and not (args.dtype == "c128" and w.D >= C128_DIGITS_D)
     prof = {"gram": [], "bond": [], "update": []} if not fused else {"kick": [], "bond_updates": [], "readout": []}
     s0, q0, b0 = g.sweeps()
     c0 = g.bond_counters()
@@ -635,7 +653,7 @@ def run_gpeps(args, rank, world, local_rank):
     fix64, fix32 = bond_fixed_flops(graphs, w.D, args.dtype)
     if args.dtype == "c128":   # one-sided sweeps: the counters are pair checks and rotations
         f64_step = fix64 + one_sided_flops(w.D, work_step[0], work_step[1]) + work_step[4] * 8
-        f32_step = fix32 + one_sided_flops(w.D, work_step[2], work_step[3])
+        f32_step = fix32 + one_sided_flops32(w.D, work_step[2], work_step[3])
     else:
         f64_step = fix64 + work_step[0] * JACOBI_BLOCK_FLOPS + work_step[1] * JACOBI_VEC_FLOPS + work_step[4] * 8
         f32_step = fix32 + work_step[2] * JACOBI_BLOCK_FLOPS + work_step[3] * JACOBI_VEC_FLOPS
@@ -651,7 +669,8 @@ def run_gpeps(args, rank, world, local_rank):
         bonds_per_launch = bonds_step / g.n_colours
         launches_step = g.n_colours
         f32_big = 0.0
-        kernel = "bond_kernel (2D x 2D bond eigenproblem, FP64 Jacobi)"
+        kernel = ("bond_kernel (SVD of the 2D x 2D bond core, FP64 one-sided Jacobi)" if args.dtype == "c128"
+                  else "bond_kernel (2D x 2D bond eigenproblem, FP64 Jacobi)")
     flops_launch = f64_step / launches_step
     achieved = flops_launch / (launch_ms * 1e-3) / 1e9
     roofline = {"kernel": kernel, "bound": "alu",
@@ -722,8 +741,8 @@ def measured_hbm_gbs():
 
 def run_condor_d64(dev, Kc=3, Wc=6):
     """The large configuration: 1121 qubits, D = 64, theta_h = 0.8 (workload condor_d64), in both
-    precisions on the fused step (schedule 4; mixed with FP64 floor 3e-8, its tuned setting at
-    D = 64).  Each: Wc warm-up steps from |0...0> (bonds saturate at step 6), Kc timed steps (CUDA
+    precisions on schedule 4 (the fused step in the mixed path, with FP64 floor 3e-8, its tuned
+    setting at D = 64; layered launches in complex128).  Each: Wc warm-up steps from |0...0> (bonds saturate at step 6), Kc timed steps (CUDA
     events on the library stream), then one profiled step for the step kernel's time and the FP64
     work it executed.  Reports bond updates/s, Trotter steps/s, algorithmic HBM GB/s against the
     measured copy bandwidth, the step kernel's FP64 rate against the derived FP64 peak, the tensor
@@ -772,7 +791,8 @@ def run_condor_d64(dev, Kc=3, Wc=6):
                       "timed_steps": f"{Wc + 1}..{Wc + Kc}",
                       "hbm": {"algorithmic_bytes_per_step": sb, "achieved_gbs": gbs, "peak_gbs": hbm_peak,
                               "frac": gbs / hbm_peak, "peak_source": hbm_src},
-                      "fp64": {"kernel": "step_kernel", "kernel_ms": kernel_ms, "flops_per_launch": f64,
+                      "fp64": {"kernel": "step_kernel" if dtype == "mixed" else "bond_kernel in layered launches",
+                               "kernel_ms": kernel_ms, "flops_per_launch": f64,
                                "achieved_gflops": gf, "peak_gflops": FP64_PEAK_GFLOPS,
                                "frac": gf / FP64_PEAK_GFLOPS},
                       "tensor_pipe": tensor_pipe_record(graphs, wc.D, kernel_ms, tensor),
@@ -844,11 +864,10 @@ def run_bp_record(dev, W=5, K=3, tensor=True):
 def run_large_chi_record(dev, W=7, K=2):
     """The large-chi path (the paper's long-time runs, Figs. 5-7, at chi = 128): workload
     eagle_d128, 127 q, D = 128 (256 x 256 bond cores, degree-3 ends of 16384 rows), theta_h = 1.0,
-    complex128, layered launches (faster than the fused step at this size, where one CTA would
-    hold a whole Gram pass).  W warm-up steps from |0...0> (the first truncation falls in step
+    complex128, layered launches.  W warm-up steps from |0...0> (the first truncation falls in step
     8), K timed steps (CUDA events on the library stream).  Reports bond updates/s, Trotter
-    steps/s and the FP64 rate of the whole step by the counted work (Gram and update products,
-    the bond SVDs' dense phases and the Jacobi work executed)."""
+    steps/s and the FP64 rate of the whole step by the counted work (the bond SVDs' dense phases
+    and the Jacobi work executed; the larger ends' products are integer digit products)."""
     import torch
     from paper_2309_15642_gb300 import GPEPS
     from workloads import kick_angles, workload
@@ -868,7 +887,7 @@ def run_large_chi_record(dev, W=7, K=2):
     ms = e0.elapsed_time(e1)
     work = [b - a for a, b in zip(w0, g.jacobi_work())]
     fix64, _ = bond_fixed_flops(graphs, wl.D, "c128")
-    f64 = K * (fix64 + big_end_flops(graphs, wl.D)) + one_sided_flops(wl.D, work[0], work[1]) + work[4] * 8
+    f64 = K * fix64 + one_sided_flops(wl.D, work[0], work[1]) + work[4] * 8
     gf = f64 / (ms * 1e-3) / 1e9
     out = {"workload": wl.name, "dtype": "c128", "D": wl.D, "value": g.bonds_per_step * K / (ms * 1e-3),
            "unit": "bond updates/s", "trotter_steps_per_s": K / (ms * 1e-3), "ms_per_step": ms / K,
