@@ -725,7 +725,7 @@ int gpeps_step_profiled(gpeps_handle* h, const double* theta, int32_t per_qubit,
 
 int gpeps_set_schedule(gpeps_handle* h, int32_t schedule) {
   if (!h || schedule < 0 || schedule > 6) return GPEPS_EINVAL;
-  if (schedule == 5 && (!h->bound || step_footprint(h->D, h->elt, h->tensor).smem > bond_share_smem(3) ||
+  if (schedule == 5 && (!h->bound || h->D > kMaxD || step_footprint(h->D, h->elt, h->tensor).smem > bond_share_smem(3) ||
                         std::min(3 * h->n_sms, (int)h->tasks.size()) > h->bond_slots))
     return GPEPS_EINVAL;
   if (schedule == 6 && (!h->bound || h->dtype != GPEPS_MIXED_C64 ||

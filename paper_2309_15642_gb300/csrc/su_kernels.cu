@@ -335,7 +335,7 @@ __device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double*
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if (oz) {
     oz_correct(V, n, G, ldg, ex);
-  } else if (n <= 128) {
+  } else {  // n <= 128: wider cores are complex128's
     // Q[r][j] = V[r][j] + sum_{i <= j} V[r][i] M[i][j], one warp per row, in place: lane l
     // forms the column pairs (j, n-1-j) for j = l and l + 32 (below n/2) in one pass of n + 1
     // products each (i = t for column j while t <= j, then i = t - j - 1 for column n-1-j),
@@ -373,24 +373,6 @@ __device__ double orthonormalise(double2* V, int n, double2* G, int ldg, double*
         }
       }
       __syncwarp();
-    }
-  } else {
-    // Q[r][j] = V[r][j] + sum_{i <= j} V[r][i] M[i][j], one warp per row, in place:
-    // 32-column chunks from the right, since a chunk reads only columns at or
-    // left of its own (each lane computes its column before any lane writes)
-    for (int r = warp; r < n; r += nw) {
-      double2* v = V + r * n;
-      for (int c = (n - 1) >> 5; c >= 0; --c) {
-        const int j = lane + 32 * c;
-        double2 acc = make_double2(0.0, 0.0);
-        if (j < n) {
-          acc = v[j];
-          for (int i = 0; i <= j; ++i) fma_c<double>(acc, v[i], G[i * ldg + j]);
-        }
-        __syncwarp();
-        if (j < n) v[j] = acc;
-        __syncwarp();
-      }
     }
   }
   __syncthreads();
@@ -2151,7 +2133,7 @@ __device__ void fused_gram(const SideDesc& sa, const V2<T>* gamma, const double*
   const V2<T> cs = kick_factors<T>(th);
   const T c = cs.x, s = cs.y;
   for (int o = threadIdx.x; o < nout; o += blockDim.x) gsum[o] = make_double2(0.0, 0.0);
-  const int tr = tile_rows(D, sizeof(V2<T>));
+  constexpr int tr = kTileRows;
   const int ntiles = (sa.rows + tr - 1) / tr;
   for (int tp = 0; tp < ntiles; ++tp) {
     const int row0 = tp * tr;
@@ -2197,9 +2179,10 @@ template <typename T>
 __device__ void fused_update(const SideDesc& sa, V2<T>* gamma, const double* lam, const V2<T>* Y, double th, int D,
                              unsigned char* sm) {
   __shared__ double cut[2];
-  const int D2 = D * D, yc = y_cols(D), tr = tile_rows(D, sizeof(V2<T>));
-  V2<T>* Ys = reinterpret_cast<V2<T>*>(sm);  // [D][yc]
-  V2<T>* A = Ys + (size_t)D * yc;
+  constexpr int tr = kTileRows;
+  const int D2 = D * D;
+  V2<T>* Ys = reinterpret_cast<V2<T>*>(sm);  // [D][D]
+  V2<T>* A = Ys + D2;
   const size_t a_elems_r = (size_t)tr * (2 * D + 1), a_elems_c = (size_t)(2 * D) * (tr + 1);
   float* mask = reinterpret_cast<float*>(A + (a_elems_r > a_elems_c ? a_elems_r : a_elems_c));
   const bool kfast = sa.str_k == 1;
@@ -2247,38 +2230,33 @@ __device__ void fused_update(const SideDesc& sa, V2<T>* gamma, const double* lam
       if (sa.lam_o2 >= 0) ok = ok && __ldcg(lam + sa.lam_o2 + p.r2) > cut[1];
       mask[r] = ok ? 1.f : 0.f;
     }
-    const int nout = nrows * yc;
+    const int nout = nrows * D;
     for (int sidx = 0; sidx < 2; ++sidx) {
-      for (int kb = 0; kb < D; kb += yc) {
-        for (int o = threadIdx.x; o < D * yc; o += blockDim.x) {
-          const int k = o / yc, cc = o - (o / yc) * yc;
-          Ys[o] = Y[sidx * D2 + k * D + kb + cc];
+      for (int o = threadIdx.x; o < D2; o += blockDim.x) Ys[o] = Y[sidx * D2 + o];
+      __syncthreads();
+      for (int o = threadIdx.x; o < nout; o += blockDim.x) {
+        int r, kc;
+        if (kfast) {
+          r = o / D;
+          kc = o - r * D;
+        } else {
+          kc = o / nrows;
+          r = o - kc * nrows;
         }
-        __syncthreads();
-        for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-          int r, kc;
-          if (kfast) {
-            r = o / yc;
-            kc = o - r * yc;
-          } else {
-            kc = o / nrows;
-            r = o - kc * nrows;
-          }
-          V2<T> acc = mk<T>(0, 0);
-          const V2<T>* Yc = Ys + kc;
-          if (kfast) {
-            const V2<T>* Ar = A + r * ldr + sidx * D;
-            for (int k = 0; k < D; ++k) fma_c<T>(acc, Ar[k], Yc[k * yc]);
-          } else {
-            const V2<T>* Ar = A + (sidx * D) * ldc + r;
-            for (int k = 0; k < D; ++k) fma_c<T>(acc, Ar[k * ldc], Yc[k * yc]);
-          }
-          const T mk_ = (T)mask[r];
-          const RowPos p = row_pos(sa, row0 + r);
-          gamma[elem(sa, sidx, p, kb + kc)] = mk<T>(acc.x * mk_, acc.y * mk_);
+        V2<T> acc = mk<T>(0, 0);
+        const V2<T>* Yc = Ys + kc;
+        if (kfast) {
+          const V2<T>* Ar = A + r * ldr + sidx * D;
+          for (int k = 0; k < D; ++k) fma_c<T>(acc, Ar[k], Yc[k * D]);
+        } else {
+          const V2<T>* Ar = A + (sidx * D) * ldc + r;
+          for (int k = 0; k < D; ++k) fma_c<T>(acc, Ar[k * ldc], Yc[k * D]);
         }
-        __syncthreads();
+        const T mk_ = (T)mask[r];
+        const RowPos p = row_pos(sa, row0 + r);
+        gamma[elem(sa, sidx, p, kc)] = mk<T>(acc.x * mk_, acc.y * mk_);
       }
+      __syncthreads();
     }
   }
 }
@@ -2442,10 +2420,12 @@ BondFootprint step_footprint(int D, size_t elt, bool tc) {
     if (tc_update_smem(D) > sm) sm = tc_update_smem(D);
     return BondFootprint{(sm + 15) & ~(size_t)15, StepSlot(D, elt).total};
   }
-  const size_t tr = (size_t)tile_rows(D, elt);
+  // complex128 beyond D = 64 has no such passes: its handles take schedule 4 and run layered launches
+  if (D > kMaxD) return BondFootprint{sm, StepSlot(D, elt).total};
+  const size_t tr = kTileRows;
   const size_t gram = tr * (2 * D + 1) * elt;
   const size_t r = tr * (2 * D + 1), c = (size_t)(2 * D) * (tr + 1);
-  const size_t upd = (size_t)D * y_cols(D) * elt + (r > c ? r : c) * elt + tr * 4;
+  const size_t upd = (size_t)D * D * elt + (r > c ? r : c) * elt + tr * 4;
   if (gram > sm) sm = gram;
   if (upd > sm) sm = upd;
   return BondFootprint{(sm + 15) & ~(size_t)15, StepSlot(D, elt).total};
@@ -2558,9 +2538,9 @@ __global__ void __launch_bounds__(kThreads)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TileDesc t = tiles[blockIdx.x];
   const SideDesc sa = bonds[t.bond].a;
-  const int D2 = D * D, yc = y_cols(D);
-  V2<T>* Ys = reinterpret_cast<V2<T>*>(smem_raw);  // [D][yc]: columns kb.. of Y_s of the spin block being written
-  V2<T>* A = Ys + (size_t)D * yc;                  // tile, layout chosen for the write order
+  const int D2 = D * D;
+  V2<T>* Ys = reinterpret_cast<V2<T>*>(smem_raw);  // [D][D]: Y_s of the spin block being written
+  V2<T>* A = Ys + D2;                              // tile, layout chosen for the write order
   const size_t a_elems_r = (size_t)t.nrows * (2 * D + 1), a_elems_c = (size_t)(2 * D) * (t.nrows + 1);
   float* mask = reinterpret_cast<float*>(A + (a_elems_r > a_elems_c ? a_elems_r : a_elems_c));
   __shared__ double cut[2];
@@ -2608,40 +2588,34 @@ __global__ void __launch_bounds__(kThreads)
     mask[r] = ok ? 1.f : 0.f;
   }
   __syncthreads();
-  // one pass per spin block s and block of yc columns kk:
-  // Gamma_a'[s][row][kk] = mask(row) sum_k A_s[row][k] Y_s[k][kk]
-  const int nout = t.nrows * yc;
+  // one pass per spin block s: Gamma_a'[s][row][kk] = mask(row) sum_k A_s[row][k] Y_s[k][kk]
+  const int nout = t.nrows * D;
   for (int sidx = 0; sidx < 2; ++sidx) {
-    for (int kb = 0; kb < D; kb += yc) {
-      for (int o = threadIdx.x; o < D * yc; o += blockDim.x) {
-        const int k = o / yc, cc = o - (o / yc) * yc;
-        Ys[o] = Y[((int64_t)t.bond * 2 + sidx) * D2 + (int64_t)k * D + kb + cc];
+    for (int o = threadIdx.x; o < D2; o += blockDim.x) Ys[o] = Y[((int64_t)t.bond * 2 + sidx) * D2 + o];
+    __syncthreads();
+    for (int o = threadIdx.x; o < nout; o += blockDim.x) {
+      int r, kc;
+      if (kfast) {  // kk fastest
+        r = o / D;
+        kc = o - r * D;
+      } else {  // r fastest
+        kc = o / t.nrows;
+        r = o - kc * t.nrows;
       }
-      __syncthreads();
-      for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-        int r, kc;
-        if (kfast) {  // kk fastest
-          r = o / yc;
-          kc = o - r * yc;
-        } else {  // r fastest
-          kc = o / t.nrows;
-          r = o - kc * t.nrows;
-        }
-        V2<T> acc = mk<T>(0, 0);
-        const V2<T>* Yc = Ys + kc;
-        if (kfast) {
-          const V2<T>* Ar = A + r * ldr + sidx * D;
-          for (int k = 0; k < D; ++k) fma_c<T>(acc, Ar[k], Yc[k * yc]);
-        } else {
-          const V2<T>* Ar = A + (sidx * D) * ldc + r;
-          for (int k = 0; k < D; ++k) fma_c<T>(acc, Ar[k * ldc], Yc[k * yc]);
-        }
-        const T mk_ = (T)mask[r];
-        const RowPos p = row_pos(sa, t.row0 + r);
-        gamma[elem(sa, sidx, p, kb + kc)] = mk<T>(acc.x * mk_, acc.y * mk_);
+      V2<T> acc = mk<T>(0, 0);
+      const V2<T>* Yc = Ys + kc;
+      if (kfast) {
+        const V2<T>* Ar = A + r * ldr + sidx * D;
+        for (int k = 0; k < D; ++k) fma_c<T>(acc, Ar[k], Yc[k * D]);
+      } else {
+        const V2<T>* Ar = A + (sidx * D) * ldc + r;
+        for (int k = 0; k < D; ++k) fma_c<T>(acc, Ar[k * ldc], Yc[k * D]);
       }
-      __syncthreads();
+      const T mk_ = (T)mask[r];
+      const RowPos p = row_pos(sa, t.row0 + r);
+      gamma[elem(sa, sidx, p, kc)] = mk<T>(acc.x * mk_, acc.y * mk_);
     }
+    __syncthreads();
   }
 }
 
@@ -2760,11 +2734,11 @@ __global__ void mean_kernel(const double* __restrict__ z, const int32_t* __restr
 }
 
 // ---------------------------------------------------------------- launchers
-static size_t gram_smem(int D, size_t elt) { return (size_t)tile_rows(D, elt) * (2 * D + 1) * elt; }
+static size_t gram_smem(int D, size_t elt) { return (size_t)kTileRows * (2 * D + 1) * elt; }
 static size_t update_smem(int D, size_t elt) {
-  const size_t tr = (size_t)tile_rows(D, elt);
+  const size_t tr = kTileRows;
   const size_t r = tr * (2 * D + 1), c = (tr + 1) * 2 * D;
-  return (size_t)D * y_cols(D) * elt + (r > c ? r : c) * elt + tr * 4 + 64;
+  return (size_t)D * D * elt + (r > c ? r : c) * elt + tr * 4 + 64;
 }
 
 // Opt in to the dynamic shared memory of the largest supported D (called once
@@ -2791,10 +2765,10 @@ cudaError_t Launch<T>::init() {
   e = cudaFuncSetAttribute(step_kernel<T, 192, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)bond_share_smem(3));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(step_kernel<T, kBondThreads, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kBondSmemMax);
-  if (e != cudaSuccess) return e;
   if constexpr (std::is_same<T, float>::value) {
+    e = cudaFuncSetAttribute(step_kernel<T, kBondThreads, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kBondSmemMax);
+    if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(step_kernel<T, 192, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)bond_share_smem(4));
     if (e != cudaSuccess) return e;
@@ -3021,8 +2995,10 @@ cudaError_t Launch<T>::step(const StepTask* tasks, int n_tasks, unsigned int* qu
     GP_STEP(192, 3, false);
   } else if (per_sm == 2) {
     GP_STEP(256, 2, false);
-  } else {
+  } else if constexpr (std::is_same<T, float>::value) {
     GP_STEP(kBondThreads, 1, false);
+  } else {
+    return cudaErrorInvalidValue;  // complex128 is fused up to D = 16, where two CTAs always fit
   }
 #undef GP_STEP
   return cudaGetLastError();
