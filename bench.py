@@ -419,9 +419,12 @@ def tf32_peak_tflops():
     return 1900.0 * TF32_OVER_BF16, "fallback bf16 1.9 PFLOP/s x nominal TF32/BF16 ratio 1.1/2.25"
 
 
-def tensor_pipe_record(graphs, D, kernel_ms, on):
+def tensor_pipe_record(graphs, D, kernel_ms, on, dtype="mixed"):
     """Tensor-pipe use of the dominant kernel: the TF32 flops its tensor-core passes executed over
     its launch time, against the TF32 peak (a kernel-average figure: the step is FP64-bound)."""
+    if dtype == "c128" and D >= C128_DIGITS_D:
+        return {"tensor_cores": True, "note": "Gram, update and core products as integer digit products "
+                "(kind::f16, mma.sync f16); their rate is not counted here"}
     if not on:
         return {"tensor_cores": False, "utilisation": 0.0,
                 "note": "Gram and update passes on CUDA cores (the autotuner's or the caller's choice)"}
@@ -687,7 +690,8 @@ def run_gpeps(args, rank, world, local_rank):
                 "launch_ms": launch_ms, "units_per_launch": bonds_per_launch, "schedule": sched,
                 "cycles_per_bond_by_phase": phase_cycles, "per_step_ms": layer_ms,
                 "tensor_pipe": tensor_pipe_record(graphs, w.D, launch_ms if fused else
-                                                  layer_ms.get("gram", 0.0) + layer_ms.get("update", 0.0), tensor)}
+                                                  layer_ms.get("gram", 0.0) + layer_ms.get("update", 0.0), tensor,
+                                                  args.dtype)}
     elt = 8 if args.dtype == "mixed" else 16
     sb = step_bytes(graphs, w.D, elt)
     hbm = {"algorithmic_bytes_per_step": sb, "achieved_gbs_whole_step": sb / (ms / K * 1e-3) / 1e9}
@@ -795,7 +799,7 @@ def run_condor_d64(dev, Kc=3, Wc=6):
                                "kernel_ms": kernel_ms, "flops_per_launch": f64,
                                "achieved_gflops": gf, "peak_gflops": FP64_PEAK_GFLOPS,
                                "frac": gf / FP64_PEAK_GFLOPS},
-                      "tensor_pipe": tensor_pipe_record(graphs, wc.D, kernel_ms, tensor),
+                      "tensor_pipe": tensor_pipe_record(graphs, wc.D, kernel_ms, tensor, dtype),
                       "flags": g.status()}
         g.close()
     out["max_abs_dz_per_qubit_mixed_vs_c128"] = float(np.abs(zs["mixed"] - zs["c128"]).max())

@@ -51,10 +51,14 @@ extern "C" {
 /* device flag bits returned by gpeps_status */
 #define GPEPS_FLAG_NOCONV 1
 #define GPEPS_FLAG_NUMERIC 2
-#define GPEPS_FLAG_TIMEOUT 4  /* a wait of the fused step kernel gave up (schedule 4) */
+#define GPEPS_FLAG_TIMEOUT 4  /* a wait gave up: of the fused step (schedules 4 to 6) for an earlier bond, or
+                                 of a tensor-core pass (any schedule) for its products */
 
 /* storage / arithmetic of the evolution */
-#define GPEPS_C128 0       /* complex128 tensors; every product and the eigensolver in FP64 */
+#define GPEPS_C128 0       /* complex128 tensors, results to FP64 rounding: FP64 products, from D = 17
+                              (larger ends) and 2D = 48 (bond core) as integer digit products on the
+                              tensor cores, no less accurate; FP64 sweeps of the bond SVD, started
+                              from FP32 */
 #define GPEPS_MIXED_C64 1  /* complex64 tensors; Gram/contract products in FP32; bond
                               eigensolver, lambda renormalisation and lambda^-1 in FP64 */
 
@@ -135,7 +139,8 @@ int gpeps_kick(gpeps_handle* h, const double* theta, int32_t per_qubit);
  * the other legs, reduce both site tensors, apply the gate, solve the 2D x 2D
  * bond eigenproblem, keep the D largest Schmidt values, renormalise lambda to
  * unit 2-norm and strip lambda^-1 (pseudo-inverse below 1e-13 max(lambda)).
- * Every Schmidt value with a positive squared value is kept (up to D).
+ * Every Schmidt value with a positive squared value is kept (up to D); GPEPS_C128
+ * sets those below 1e-15 of the bond's norm, which are rounding, to zero.
  * Errors: GPEPS_EINVAL for colour outside [0, n_colours).
  */
 int gpeps_zz_layer(gpeps_handle* h, int32_t colour);
@@ -188,10 +193,10 @@ int gpeps_set_levels(gpeps_handle* h, double level_ratio, int32_t levels);
 
 /*
  * Wait limit of the fused step (schedule 4), in SM clock cycles (default
- * 4e9, about 2 s, where a bond update takes at most ~0.2 s (D <= 64); 6.4e10
- * beyond D = 64, where one takes about a second): a bond that waits longer for an earlier bond on one of its
- * sites gives up, raises GPEPS_FLAG_TIMEOUT and runs on what it finds, so a
- * launch always ends.  0 gives up at once whenever a dependency is still
+ * 4e9, about 2 s, where a bond update takes at most ~0.2 s): a bond that waits
+ * longer for an earlier bond on one of its sites gives up, raises
+ * GPEPS_FLAG_TIMEOUT and runs on what it finds, so a launch always ends.  The
+ * tensor-core passes have a limit of their own.  0 gives up at once whenever a dependency is still
  * running (failure-detection tests use it).  Host-only; drops a captured step
  * graph.  Errors: GPEPS_EINVAL for a negative value.
  */
@@ -216,10 +221,16 @@ int gpeps_set_wait_limit(gpeps_handle* h, int64_t cycles);
  * three 192-thread CTAs per SM (where their shared memory fits, D <= 32), 6
  * with four (GPEPS_MIXED_C64 where their shared memory fits, D <= 32; with the
  * tensor cores on, their TMEM, four times 4D columns, must fit the SM's 512).
+ * GPEPS_C128 from D = 17 runs the passes of the larger ends as launches of their
+ * own (each takes an SM's shared memory and tensor memory), so its steps are
+ * layered on every schedule: 4 and 5 are accepted and run the bonds like 2.  A
+ * complex128 colour class (or group of bonds, see gpeps_query_workspace) of no
+ * more bonds than SMs takes one 512-thread CTA per bond on every schedule.
  * Host-only; drops a captured step graph.  Errors: GPEPS_EINVAL for other
  * values, and for 2 to 6 on an unbound handle, when the FP32 level does not
- * fit the CTA's share of shared memory (D above 47 for 2, above 32 for 3, 5
- * and 6), for 6 with complex128, or on a device with more than 256 SMs.
+ * fit the CTA's share of shared memory (mixed: D above 47 for 2, above 32 for 3,
+ * 5 and 6; complex128: D above 73 for 3, above 29 for 5), for 6 with complex128,
+ * or on a device with more than 256 SMs.
  */
 int gpeps_set_schedule(gpeps_handle* h, int32_t schedule);  /* 0..6 */
 
@@ -385,7 +396,9 @@ int gpeps_sweeps(gpeps_handle* h, int64_t* sweeps64, int64_t* sweeps32, int64_t*
  * the matrix from both sides, 72 flops), FP64 eigenvector pair updates (one row
  * of V, 18 flops), the same two counts of the FP32 levels, and the FP64 complex
  * multiply-adds with which the extra FP32 levels' rotations are applied to V
- * and rho' (8 flops each).  Converged pairs are skipped and not counted.  Synchronises the stream.  Errors: GPEPS_EINVAL
+ * and rho' (8 flops each).  Converged pairs are skipped and not counted.
+ * Complex128 counts pair checks and rotations of its one-sided sweeps instead of the
+ * first two, and of the next two.  Synchronises the stream.  Errors: GPEPS_EINVAL
  * for NULL pointers or an unbound handle.
  */
 int gpeps_jacobi_work(gpeps_handle* h, int64_t* work);
@@ -393,15 +406,16 @@ int gpeps_jacobi_work(gpeps_handle* h, int64_t* work);
 /* Counters of the bond-eigenproblem kernel since the last gpeps_reset, summed
  * over bonds, host int64[24].  [0..5] SM cycles (clock64 of one thread per
  * CTA) of its phases: [0] the bond matrix (mixed: the reduced density matrix
- * rho; complex128: the pivoted Cholesky roots of the Gram blocks, the core M
- * and rho = M^H M), [1] first FP32 Jacobi level, [2] FP64 re-orthonormalisation
- * of the FP32 eigenvectors, [3] mixed: V^dagger rho V and the further FP32
- * levels on small-eigenvalue blocks; complex128: B = M V and the further FP32
- * levels on blocks of small columns of B, [4] FP64 Jacobi sweeps (complex128:
- * one-sided, on B), [5] truncation, Y matrices and the smaller end.  [6..13]
+ * rho; complex128: the sum of the Gram partials, the pivoted Cholesky roots of the
+ * Gram blocks and the core M), [1] first FP32 Jacobi level (complex128: the FP32
+ * basis), [2] FP64 re-orthonormalisation of the FP32 eigenvectors, [3] mixed:
+ * V^dagger rho V and the further FP32 levels on small-eigenvalue blocks;
+ * complex128: the further FP32 levels on blocks of small columns of Z, [4] FP64
+ * Jacobi sweeps (complex128: Z = M^H U, the simultaneous corrections and the
+ * one-sided sweeps), [5] truncation, Y matrices and the smaller end.  [6..13]
  * rotations applied in sweep 0..7 of the first FP32 level, [14..21] in FP64
  * sweep 0..7, [22] and [23] SM cycles of the Gram pass and of the update pass
- * of the larger end inside the fused step (schedules 4 and 5; 0 otherwise).
+ * of the larger end inside the fused step (schedules 4 to 6; 0 otherwise).
  * Synchronises. */
 int gpeps_bond_phase_cycles(gpeps_handle* h, int64_t* cycles);
 
@@ -450,9 +464,10 @@ int gpeps_bond_update_noalloc(int32_t D, int32_t dtype, void* gamma_a, int32_t d
  * receives the helper's (c, s, Re e, Im e) and then the reference's.  which: 0
  * the two-sided helper of the squared eigensolver (|g|^2 must be above FP32's
  * smallest normal), 1 the one-sided helper of the complex128 bond SVD (any
- * finite scale with |g|^2 finite and not zero), its s and e formed from its tau = t / |g| and
- * g; 3 the same helper's own results (tau, c, 1 + t^2, t |g|).  Asynchronous on stream.  Errors: GPEPS_EINVAL for n < 0, an
- * unknown `which` or NULL arrays; GPEPS_ECUDA for a failed launch.
+ * finite scale with |g|^2 finite and not zero), its s formed from its tau = t / |g|, c
+ * and |g|, its e from g; 3 the same helper's own results (tau, c, 1 + t^2, t |g|).
+ * Asynchronous on stream.  Errors: GPEPS_EINVAL for n < 0, an unknown `which` or
+ * NULL arrays; GPEPS_ECUDA for a failed launch.
  */
 int gpeps_selftest_rotation(int32_t which, int32_t n, const double* in, double* out, void* stream);
 

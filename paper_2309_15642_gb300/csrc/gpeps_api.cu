@@ -552,9 +552,7 @@ int gpeps_create(const gpeps_graph* graphs, int32_t n_instances, int32_t D, int3
   h->jp.max_sweeps32 = 20;
   h->jp.level_ratio = 1e-5;
   h->jp.levels = 4;
-  // beyond D = 64 one task of the fused step (Gram pass over 16384 rows, bond SVD,
-  // update pass) takes about a second on its SM: its dependants may wait longer
-  h->jp.wait_cycles = kWaitCycles * (D > kMaxD ? 16 : 1);
+  h->jp.wait_cycles = kWaitCycles;
   h->jp.gate_sign = 1;
   h->jp.upper_partials = h->oz();
   // layouts
@@ -725,7 +723,8 @@ int gpeps_step_profiled(gpeps_handle* h, const double* theta, int32_t per_qubit,
 
 int gpeps_set_schedule(gpeps_handle* h, int32_t schedule) {
   if (!h || schedule < 0 || schedule > 6) return GPEPS_EINVAL;
-  if (schedule == 5 && (!h->bound || h->D > kMaxD || step_footprint(h->D, h->elt, h->tensor).smem > bond_share_smem(3) ||
+  if (schedule == 5 && (!h->bound || h->D > kMaxD ||
+                        step_footprint(h->D, h->elt, h->tensor).smem > bond_share_smem(3) ||
                         std::min(3 * h->n_sms, (int)h->tasks.size()) > h->bond_slots))
     return GPEPS_EINVAL;
   if (schedule == 6 && (!h->bound || h->dtype != GPEPS_MIXED_C64 ||

@@ -19,7 +19,12 @@ constexpr int kTileRows = 64;      // rows of a big-side tile (Gram and update l
 // Rows of a big-side tile at (D, element bytes): kTileRows, or 32 for complex128 beyond D = 64,
 // where the digits of 64 rows (229 KB) would not fit the shared memory of a CTA
 __host__ __device__ constexpr int tile_rows(int D, size_t elt) { return (D > kMaxD && elt == 16) ? 32 : kTileRows; }
-constexpr int kOzMinD = 17;        // smallest D of the complex128 tensor-core passes
+// Smallest D of the complex128 tensor-core passes: up to 16 the fused step and the reverse mode
+// run FP64 passes, and the digits, padded to 32 bond indices, gain 0.2 of a layer's 2.9 ms at
+// most.  Gram and update of one class of 8 x 127 qubits, FP64 | digits: D = 12 0.28 | 0.39,
+// 16 0.67 | 0.48, 17 0.90 | 0.59, 24 2.8 | 1.1, 32 8.6 | 1.8, 33 9.9 | 4.2 (the next padding),
+// 64 132 | 17.5 ms.
+constexpr int kOzMinD = 17;
 constexpr int kThreads = 256;      // threads of the streaming and readout CTAs
 constexpr int kBondThreads = 512;  // threads of the bond-eigenproblem CTA (one CTA per SM: more warps hide FP64 latency)
 constexpr double kLambdaCut = 1e-13;  // pseudo-inverse threshold relative to max(lambda)
@@ -97,7 +102,7 @@ struct JacobiParams {
   int levels;          // extra FP32 levels at most (0..kMaxExtraLevels)
   long long wait_cycles;  // fused step: a wait for an earlier task gives up after this many SM cycles
   int full_basis;         // complex128: keep a complete unitary V per bond (the reverse mode; see bond_front_svd)
-  int upper_partials;     // complex128: Gram partials as oz_gram_kernel writes them, upper triangles in upper_index order
+  int upper_partials;     // complex128: Gram partials as oz_gram_kernel writes them (upper triangles)
   int gate_sign;          // +1: the paper's exp(+i pi/4 Z Z); -1: its inverse exp(-i pi/4 Z Z)
 };
 

@@ -1,6 +1,7 @@
-// Diagnostic entry points.  Steps of the bond core (kernel in su_kernels.cu), and the FP64 Jacobi rotation helpers of jacobi.cuh next to
-// the textbook formulas evaluated with CUDA's own FP64 hypot, sqrt and rsqrt, so
-// that a test can hold the helpers' Newton-Raphson refinements to a stated bound.
+// Diagnostic entry points: steps of the bond core (kernel in su_kernels.cu), and the FP64
+// Jacobi rotation helpers of jacobi.cuh next to the textbook formulas evaluated with
+// CUDA's own FP64 hypot, sqrt and rsqrt, so that a test can hold the helpers'
+// refinements to a stated bound.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -66,5 +67,6 @@ extern "C" int gpeps_selftest_rotation(int32_t which, int32_t n, const double* i
 extern "C" int gpeps_selftest_core(int32_t which, int32_t n, const double* a, double* b, double* out,
                                    void* stream) {
   if (which < 0 || which > 1 || n < 2 || n > 2 * kMaxDc128 || (n & 1) || !a || !b || !out) return GPEPS_EINVAL;
-  return launch_core_selftest(which, n, a, b, out, static_cast<cudaStream_t>(stream)) == cudaSuccess ? GPEPS_OK : GPEPS_ECUDA;
+  const cudaError_t e = launch_core_selftest(which, n, a, b, out, static_cast<cudaStream_t>(stream));
+  return e == cudaSuccess ? GPEPS_OK : GPEPS_ECUDA;
 }

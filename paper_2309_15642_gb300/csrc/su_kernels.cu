@@ -269,11 +269,12 @@ __device__ __forceinline__ int upper_pos(int i, int j, int n) {
 // 16 bytes mirrored below the diagonal, (j, i) for i < j and the padding column
 // (i, n) for i = j (ldg >= n + 1): X1 in its first 8 bytes, X in its last 8.
 // Q pairs the columns j and n-1-j on one lane (n <= 128).  With kOz (ex: 2n ints), from
-// kOzMinBond columns on, E and Q are integer digit products on the tensor cores.
-// Cores of fewer columns keep FP64 multiply-adds (a trial with the four n x n products of the
-// mixed path's solve: 8 steps of 16 x 127 qubits at n = 32 took 29.3 ms against 31.3 as digit products, one
-// step of 127 + 433 + 1121 qubits at n = 64 19.7 against 18.0), and so does the mixed path, whose results
-// keep their bits.
+// kOzMinBond columns on, E and Q are integer digit products on the tensor cores, and the
+// corrections (svd_refine) run.  Bonds of one class of 8 x 127 qubits without | with them: n = 48
+// 5.8 | 4.3, 64 9.5 | 8.0, 80 19.7 | 16.7, 128 67 | 58 ms.  They gain on narrower cores too (n = 24
+// 1.44 | 1.23, 32 2.22 | 1.75, 46 5.6 | 4.3): the line is where they were first measured, and
+// D < 24 and the reverse mode keep their FP64 products.  The mixed path, whose results keep
+// their bits, has none.
 constexpr int kOzMinBond = 48;
 __device__ __forceinline__ float2* tri32(double2* G, int ldg, int n, int i, int j) {
   return reinterpret_cast<float2*>(i < j ? G + j * ldg + i : G + i * ldg + n);
@@ -1135,6 +1136,8 @@ constexpr float kBasisCut = 1e-6f;
 // (A [n], stride ld, n entries each): modified Gram-Schmidt, largest column first, so that the
 // small ones lose what they still hold of the large, twice.  False (the same in every thread)
 // where a column lies within 1e-4 of the span of the larger ones, which is no basis to keep.
+// FP64 sweeps a bond after a cap of five, against a start from the identity: D = 16 3.2 | 11.4,
+// 32 4.1 | 15.0, 64 10.4 | 21.6.
 __device__ __noinline__ bool orthogonal_units32(float2* A, int n, int ld, float* nrm) {
   constexpr int kT = kMaxDc128 * 2 / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -1581,8 +1584,8 @@ __device__ __noinline__ void svd_refine(double2* Zt, int n, double trace, double
 // s_j v_j: the right singular vectors without accumulating a rotation product (half
 // the rotation work).  Columns at rounding (|z|^2 <= kNoiseRelSvd ||M||^2) are
 // dropped: their direction is noise.  With `full` (the reverse mode needs a complete
-// unitary V, in the same gauge forward and recomputed) or n < 2D (an end of degree 1): B = M V0 with V0 the right singular
-// vectors from FP32, V rotated alongside.
+// unitary V, in the same gauge forward and recomputed) or n < 2D (an end of degree 1):
+// B = M V0 with V0 the right singular vectors from FP32, V rotated alongside.
 template <bool kCG>
 __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ partials, const double2* gsum,
                                const double2* gamma, const double* lam, const double* kcs, int D, const JacobiParams& jp,
@@ -2895,7 +2898,8 @@ cudaError_t Launch<T>::update(const TileDesc* tiles, int n_tiles, const BondDesc
 }
 
 cudaError_t OzPass::init() {
-  cudaError_t e = cudaFuncSetAttribute(oz_gram_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzGramSmem);
+  cudaError_t e =
+      cudaFuncSetAttribute(oz_gram_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzGramSmem);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(oz_gram_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzGramSmem);
   if (e != cudaSuccess) return e;

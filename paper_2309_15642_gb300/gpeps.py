@@ -21,7 +21,7 @@ DTYPES = {"c128": GPEPS_C128, "mixed": GPEPS_MIXED_C64}
 class GPEPS:
     """A batch of graph PEPS, one per graph in ``graphs`` (list of ``(n_qubits, edges)``).
 
-    ``dtype``: ``"c128"`` (FP64 everywhere) or ``"mixed"`` (complex64 tensors,
+    ``dtype``: ``"c128"`` (complex128, results to FP64 rounding) or ``"mixed"`` (complex64 tensors,
     FP32 Gram/contract products, FP64 bond eigensolver and lambda).
     ``colours``: optional list (one int8 array per graph) of edge colour classes.
     """
