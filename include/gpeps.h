@@ -229,7 +229,7 @@ int gpeps_set_wait_limit(gpeps_handle* h, int64_t cycles);
  * Host-only; drops a captured step graph.  Errors: GPEPS_EINVAL for other
  * values, and for 2 to 6 on an unbound handle, when the FP32 level does not
  * fit the CTA's share of shared memory (mixed: D above 47 for 2, above 32 for 3,
- * 5 and 6; complex128: D above 73 for 3, above 29 for 5), for 6 with complex128,
+ * 5 and 6; complex128: D above 72 for 3, above 29 for 5), for 6 with complex128,
  * or on a device with more than 256 SMs.
  */
 int gpeps_set_schedule(gpeps_handle* h, int32_t schedule);  /* 0..6 */

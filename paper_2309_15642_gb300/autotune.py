@@ -19,7 +19,8 @@ FP32-level thresholds (tol32, floor32 = 2e-7 or 1e-7 of the trace) x FP64 stoppi
 thresholds (tol, floor_rel = 1e-8, 3e-8, 7e-8 or 1e-7 of the trace: up to the ~1e-7
 relative rounding that the bond matrix inherits from its FP32 Gram inputs), the FP64
 floor at most FLOOR_RATIO of the FP32 floor; complex128 keeps its rounding-level
-thresholds and tunes the schedule only.
+thresholds and tunes the schedule only (from D = 17 its steps are layered on every
+schedule, 4 and 5 running the launches of 2).
 """
 from __future__ import annotations
 

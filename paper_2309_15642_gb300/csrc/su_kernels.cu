@@ -1593,6 +1593,8 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
                                int* order, int* rp, int* iflag,
                                unsigned char* lvl, bool shared_work, bool full, unsigned long long* sweeps_out,
                                unsigned long long* cycles, int* flags, long long& t_prev, double2** Vm_out) {
+  constexpr bool kDigits = !kCG;  // the fused step (D < kOzMinD) has no core of kOzMinBond columns
+  static_assert(2 * (kOzMinD - 1) < kOzMinBond, "fused complex128 cores");
   const SideDesc& sb = bd.b;
   const int n = 2 * sb.rows, rows = 2 * D, D2 = D * D;
   const SvdLayout L(D);
@@ -1692,8 +1694,8 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
     // Its columns are orthogonal to |E| ~ 1e-6; the series of `orthonormalise` is exact to
     // O(|E|^3), and its FP32 products to ~n |E|^2 1e-7.  A basis further off takes a second
     // pass, which starts from ~|E|^3; one beyond the series' range is flagged.
-    const double emax = orthonormalise<true>(Vx, nv, Xs, nv + 1, scal, order);
-    const double emax2 = emax > 4e-6 ? orthonormalise<true>(Vx, nv, Xs, nv + 1, scal, order) : 0.0;
+    const double emax = orthonormalise<kDigits>(Vx, nv, Xs, nv + 1, scal, order);
+    const double emax2 = emax > 4e-6 ? orthonormalise<kDigits>(Vx, nv, Xs, nv + 1, scal, order) : 0.0;
     if (threadIdx.x == 0 && (!(emax < 1e-2) || !(emax2 < 1e-8))) atomicOr(flags, 1);
   }
   mark(2);
@@ -1728,9 +1730,11 @@ __device__ bool bond_front_svd(const BondDesc& bd, const double2* __restrict__ p
   // size).  Only then are the small columns a clean block for the FP32 levels,
   // whose rotations leave the last sweeps little to do.
   unsigned long long* rot = cycles ? cycles + kPhases + kRotSweeps : nullptr;
-  if (left && n >= kOzMinBond)
-    for (int pass = 0; pass < 2; ++pass)
-      svd_refine(Zt, n, trace, Xs, Vx, reinterpret_cast<float2*>(Mt), ev, reinterpret_cast<int*>(dsc), order);
+  if constexpr (kDigits) {
+    if (left && n >= kOzMinBond)
+      for (int pass = 0; pass < 2; ++pass)
+        svd_refine(Zt, n, trace, Xs, Vx, reinterpret_cast<float2*>(Mt), ev, reinterpret_cast<int*>(dsc), order);
+  }
   const int sw1 = os_sweeps(Zt, zr, Vt, n, jp.tol, jp.floor_rel * trace, trace, 1, ev, dsc, dinv, re, be, iflag,
                             sweeps_out + 4, rot);
   mark(4);
